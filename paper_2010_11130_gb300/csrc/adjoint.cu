@@ -8,7 +8,7 @@
 // adjoint needs beyond setup and solve: the transpose of A with its values and
 // the outer product restricted to A's pattern.
 #include "air_internal.cuh"
-#include "warp_dense.cuh"
+#include "lane_dense.cuh"
 
 namespace {
 
@@ -42,21 +42,63 @@ __global__ void scatter_t_kernel(int64_t n, const int64_t *rp, const int32_t *ci
 }
 
 // The slots were claimed in any order: sort each row of the transpose by
-// column (an insertion sort; rows hold a few dozen entries).
-__global__ void sort_rows_kernel(int64_t m, const int64_t *rpt, int32_t *cit, double *vt) {
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < m; r += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t b = rpt[r], e = rpt[r + 1];
-        for (int64_t p = b + 1; p < e; ++p) {
-            const int32_t c = cit[p];
-            const double x = vt[p];
-            int64_t q = p - 1;
-            while (q >= b && cit[q] > c) {
-                cit[q + 1] = cit[q];
-                vt[q + 1] = vt[q];
-                --q;
+// column, one warp per row.  Rows of at most 32 SORT_R entries are held in
+// registers (entry lane + 32 r) and every entry's place is the number of
+// smaller columns in the row (the columns of a row are distinct; equal ones,
+// from a malformed matrix, keep their order); longer rows are sorted in place
+// by odd-even transposition.  Bound: the 24 bytes per entry read and written;
+// 20.6 M entries, 36 per row: 0.79 ms (one thread per row and an insertion sort
+// in global memory: 7.6 ms).
+constexpr int SORT_R = 4;
+
+__global__ void __launch_bounds__(256) sort_rows_kernel(int64_t m, const int64_t *rpt, int32_t *cit, double *vt) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < m; row += warps) {
+        const int64_t b = rpt[row];
+        const int64_t len = rpt[row + 1] - b;
+        if (len <= 32 * SORT_R) {
+            int32_t c[SORT_R];
+            double x[SORT_R];
+            int place[SORT_R];
+#pragma unroll
+            for (int r = 0; r < SORT_R; ++r) {
+                const bool on = lane + 32 * r < len;
+                c[r] = on ? cit[b + lane + 32 * r] : INT32_MAX;
+                x[r] = on ? vt[b + lane + 32 * r] : 0.0;
+                place[r] = 0;
             }
-            cit[q + 1] = c;
-            vt[q + 1] = x;
+            __syncwarp();
+#pragma unroll
+            for (int q = 0; q < SORT_R; ++q) {
+                if (32 * q >= len) break;
+                const int top = len - 32 * q < 32 ? (int)(len - 32 * q) : 32;
+                for (int k = 0; k < top; ++k) {
+                    const int32_t o = __shfl_sync(0xffffffffu, c[q], k);
+#pragma unroll
+                    for (int r = 0; r < SORT_R; ++r)
+                        place[r] += o < c[r] || (o == c[r] && k + 32 * q < lane + 32 * r) ? 1 : 0;
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < SORT_R; ++r)
+                if (lane + 32 * r < len) {
+                    cit[b + place[r]] = c[r];
+                    vt[b + place[r]] = x[r];
+                }
+        } else {
+            for (int64_t pass = 0; pass < len; ++pass) {
+                for (int64_t p = b + (pass & 1) + 2 * lane; p + 1 < b + len; p += 64) {
+                    const int32_t c0 = cit[p], c1 = cit[p + 1];
+                    if (c0 <= c1) continue;
+                    const double x0 = vt[p];
+                    cit[p] = c1;
+                    cit[p + 1] = c0;
+                    vt[p] = vt[p + 1];
+                    vt[p + 1] = x0;
+                }
+                __syncwarp();
+            }
         }
     }
 }
@@ -75,105 +117,119 @@ __global__ void outer_kernel(int64_t n, int64_t ncols, const int64_t *rp, const 
     }
 }
 
+// D_f^{-T} of every facet block, one block per lane.
+__global__ void __launch_bounds__(32) invert_transposed_kernel(int64_t nblk, int b, const double *diag, double *inv,
+                                                               int *err) {
+    extern __shared__ double bsm[];
+    const int lane = threadIdx.x, bb = b * b;
+    const int64_t first = (int64_t)blockIdx.x * 32;
+    const int count = nblk - first < 32 ? (int)(nblk - first) : 32;
+    lane_load_blocks(diag, first, count, b, true, bsm);
+    if (lane < count && !lane_invert(bsm + lane, b)) atomicOr(err, AIR_DEVERR_SINGULAR);
+    __syncwarp();
+    for (int k = 0; k < count; ++k)
+        for (int t = lane; t < bb; t += 32) inv[(first + k) * bb + t] = bsm[t * LANE_LD + k];
+}
+
 // One warp per block row f of A^T (rows f b .. f b + b - 1): every
-// off-diagonal block B (columns g b .. g b + b - 1) becomes D_f^{-T} B D_g^T,
-// the diagonal block (stored as its b ones) stays the identity.  Rows of a
-// block row must share one layout of whole blocks; otherwise err gets
-// AIR_DEVERR_CSR and the block row is left unscaled.
+// off-diagonal block T (columns g b .. g b + b - 1) becomes D_f^{-T} T D_g^T,
+// the diagonal block (stored as its b ones) stays the identity.  SCALE_CH
+// blocks at a time, so that the two products fill the lanes (FP64 issue bounds
+// it; 95,200 rows of 6 x 6 blocks: 0.45 ms, with the inverses 0.6 ms, against
+// 3.65 ms for the inverse in the same warp and a product of three factors per
+// entry).  Rows of a block row must share one layout of whole blocks;
+// otherwise err gets AIR_DEVERR_CSR.
+constexpr int SCALE_CH = 6;
+
 __global__ void __launch_bounds__(128) block_scale_t_kernel(int64_t nblk, int b, const double *diag,
-                                                            const int64_t *rpt, const int32_t *cit, double *vt,
-                                                            int *err) {
+                                                            const double *inv, const int64_t *rpt,
+                                                            const int32_t *cit, double *vt, int *err) {
     extern __shared__ double bsm[];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t f = (int64_t)blockIdx.x * 4 + w;
     if (f >= nblk) return;
     const int bb = b * b;
-    double *Dt = bsm + (size_t)w * 6 * bb, *Di = Dt + bb, *W = Di + bb, *T = W + 2 * bb, *G = T + bb;
-    const int64_t r0 = f * b;
-    const int64_t len = rpt[r0 + 1] - rpt[r0];
+    double *Di = bsm + (size_t)w * (1 + 3 * SCALE_CH) * bb, *T = Di + bb, *G = T + SCALE_CH * bb, *Y = G + SCALE_CH * bb;
+    const int64_t r0 = f * b, base = rpt[r0];
+    const int64_t len = rpt[r0 + 1] - base;
     bool ok = len >= 1 && (len - 1) % b == 0;
     for (int i = 1; i < b && ok; ++i) ok = rpt[r0 + i + 1] - rpt[r0 + i] == len;
     if (!ok) {
         if (lane == 0) atomicOr(err, AIR_DEVERR_CSR);
         return;
     }
-    for (int t = lane; t < bb; t += 32) Dt[t] = diag[f * bb + (t % b) * b + t / b];   // D_f^T
-    __syncwarp();
-    if (!warp_inverse(Dt, b, W, Di)) {                                               // Di = D_f^{-T}
-        if (lane == 0) atomicOr(err, AIR_DEVERR_SINGULAR);
-        return;
-    }
+    for (int t = lane; t < bb; t += 32) Di[t] = inv[f * bb + t];
     const int64_t nb = (len - 1) / b;
     int64_t p = 0;                      // position within the row
-    for (int64_t k = 0; k < nb; ++k) {
-        // skip the diagonal entry if it comes first
-        const int32_t c0 = cit[rpt[r0] + p];
-        if (c0 / b == f) ++p;
-        const int64_t off = p;
-        const int32_t cs = cit[rpt[r0] + off];
-        const int64_t g = cs / b;
-        bool good = cs % b == 0 && g != f;
-        for (int i = 0; i < b && good; ++i)
-            for (int j = 0; j < b && good; ++j) good = cit[rpt[r0 + i] + off + j] == (int32_t)(g * b + j);
+    for (int64_t k0 = 0; k0 < nb; k0 += SCALE_CH) {
+        const int ch = nb - k0 < SCALE_CH ? (int)(nb - k0) : SCALE_CH;
+        int64_t off[SCALE_CH];          // where the chunk's blocks start: a diagonal entry before one is skipped
+        bool good = true;
+        for (int k = 0; k < ch; ++k) {
+            // nb blocks and one diagonal entry fill the row: a second entry in column block f would overrun it
+            if (p < len && cit[base + p] / b == f) ++p;
+            if (p + b > len) { good = false; break; }
+            off[k] = p;
+            p += b;
+        }
+        for (int k = 0; k < ch && good; ++k) {
+            const int32_t cs = cit[base + off[k]];
+            const int64_t g = cs / b;
+            good = cs % b == 0 && g != f && cs >= 0 && g < nblk;
+            for (int t = lane; t < bb && good; t += 32) {
+                const int i = t / b, j = t % b;
+                good = cit[base + i * len + off[k] + j] == (int32_t)(g * b + j);
+                T[k * bb + t] = vt[base + i * len + off[k] + j];
+                G[k * bb + t] = diag[g * bb + t];                                     // D_g
+            }
+            good = __all_sync(0xffffffffu, good);
+        }
         if (!good) {
             if (lane == 0) atomicOr(err, AIR_DEVERR_CSR);
             return;
         }
-        for (int t = lane; t < bb; t += 32) {
-            const int i = t / b, j = t % b;
-            T[t] = vt[rpt[r0 + i] + off + j];
-            G[t] = diag[g * bb + t];                                                  // D_g
-        }
         __syncwarp();
-        // T <- Di T G^T
-        double res[4];
-        int cntr = 0;
-        for (int t = lane; t < bb; t += 32) {
-            const int i = t / b, j = t % b;
+        for (int t = lane; t < ch * bb; t += 32) {            // Y = T D_g^T
+            const int k = t / bb, i = t / b % b, j = t % b;
+            const double *Tk = T + k * bb + i * b, *Gk = G + k * bb + j * b;
             double acc = 0.0;
-            for (int a = 0; a < b; ++a) {
-                double inner = 0.0;
-                for (int c = 0; c < b; ++c) inner += T[a * b + c] * G[j * b + c];
-                acc += Di[i * b + a] * inner;
-            }
-            res[cntr++] = acc;
+            for (int c = 0; c < b; ++c) acc += Tk[c] * Gk[c];
+            Y[t] = acc;
         }
         __syncwarp();
-        cntr = 0;
-        for (int t = lane; t < bb; t += 32) {
-            const int i = t / b, j = t % b;
-            vt[rpt[r0 + i] + off + j] = res[cntr++];
+        for (int t = lane; t < ch * bb; t += 32) {            // D_f^{-T} Y
+            const int k = t / bb, i = t / b % b, j = t % b;
+            double acc = 0.0;
+            for (int c = 0; c < b; ++c) acc += Di[i * b + c] * Y[k * bb + c * b + j];
+            vt[base + i * len + off[k] + j] = acc;
         }
         __syncwarp();
-        p = off + b;
     }
 }
 
-// y_k = op(D_k) x_k over the b-blocks: op 0 D, 1 D^T, 2 D^{-1}, 3 D^{-T}.  One warp per block.
-__global__ void __launch_bounds__(128) block_apply_kernel(int64_t nblk, int b, const double *diag, int op,
-                                                          const double *x, double *y, int *err) {
+// y_k = op(D_k) x_k over the b-blocks: op 0 D, 1 D^T, 2 D^{-1}, 3 D^{-T}; 32 blocks per warp, the inverses one block
+// per lane.  x is read before y is written, so that they may be the same vector.
+__global__ void __launch_bounds__(32) block_apply_kernel(int64_t nblk, int b, const double *diag, int op,
+                                                         const double *x, double *y, int *err) {
     extern __shared__ double bsm[];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t k = (int64_t)blockIdx.x * 4 + w;
-    if (k >= nblk) return;
-    const int bb = b * b;
-    double *M = bsm + (size_t)w * 5 * bb, *Mi = M + bb, *W = Mi + bb, *xs = W + 2 * bb;
-    const bool tr = op == 1 || op == 3;
-    for (int t = lane; t < bb; t += 32) M[t] = tr ? diag[k * bb + (t % b) * b + t / b] : diag[k * bb + t];
-    for (int t = lane; t < b; t += 32) xs[t] = x[k * b + t];
+    const int lane = threadIdx.x;
+    const int64_t first = (int64_t)blockIdx.x * 32;
+    const int count = nblk - first < 32 ? (int)(nblk - first) : 32;
+    double *sx = bsm + b * b * LANE_LD;
+    lane_load_blocks(diag, first, count, b, op == 1 || op == 3, bsm);
+    for (int t = lane; t < count * b; t += 32) sx[(t % b) * LANE_LD + t / b] = x[first * b + t];
     __syncwarp();
-    const double *Op = M;
     if (op >= 2) {
-        if (!warp_inverse(M, b, W, Mi)) {
-            if (lane == 0) atomicOr(err, AIR_DEVERR_SINGULAR);
-            return;
-        }
-        Op = Mi;
+        if (lane < count && !lane_solve(bsm + lane, sx + lane, b)) atomicOr(err, AIR_DEVERR_SINGULAR);
+        __syncwarp();
     }
-    for (int i = lane; i < b; i += 32) {
-        double acc = 0.0;
-        for (int j = 0; j < b; ++j) acc += Op[i * b + j] * xs[j];
-        y[k * b + i] = acc;
+    for (int t = lane; t < count * b; t += 32) {
+        const int k = t / b, i = t % b;
+        double v = 0.0;
+        if (op >= 2) v = sx[i * LANE_LD + k];
+        else
+            for (int j = 0; j < b; ++j) v += bsm[(i * b + j) * LANE_LD + k] * sx[j * LANE_LD + k];
+        y[first * b + t] = v;
     }
 }
 
@@ -193,7 +249,7 @@ int air_csr_transpose_impl(int64_t n, int64_t ncols, int64_t nnz, const int64_t 
         AIR_CUDA(cudaMemsetAsync(cnt, 0, (size_t)(ncols > 0 ? ncols : 1) * sizeof(int32_t), s));
         scatter_t_kernel<<<air_counted(blocks_for(n, 256)), 256, 0, s>>>(n, rp, ci, v, ncols, rpt, cnt, cit, vt);
         AIR_LAUNCH();
-        sort_rows_kernel<<<air_counted(blocks_for(ncols, 256)), 256, 0, s>>>(ncols, rpt, cit, vt);
+        sort_rows_kernel<<<air_counted(blocks_for(ncols * 32, 256)), 256, 0, s>>>(ncols, rpt, cit, vt);
         AIR_LAUNCH();
     }
     cudaFreeAsync(cnt, s);
@@ -211,19 +267,26 @@ int air_csr_outer_impl(int64_t n, int64_t ncols, const int64_t *rp, const int32_
 int air_block_scale_transpose_impl(int64_t n, int b, const double *diag, const int64_t *rpt, const int32_t *cit,
                                    double *vt, int *d_err, cudaStream_t s) {
     const int64_t nblk = n / b;
-    const size_t smem = (size_t)4 * 6 * b * b * sizeof(double);
     if (nblk <= 0) return AIR_OK;
-    block_scale_t_kernel<<<air_counted((unsigned)((nblk + 3) / 4)), 128, smem, s>>>(nblk, b, diag, rpt, cit, vt,
+    const size_t smem = (size_t)4 * (1 + 3 * SCALE_CH) * b * b * sizeof(double);
+    AIR_CUDA(air_smem_optin(block_scale_t_kernel));
+    double *inv = nullptr;
+    AIR_CUDA(cudaMallocAsync(&inv, (size_t)(nblk * b * b) * sizeof(double), s));
+    invert_transposed_kernel<<<air_counted((unsigned)((nblk + 31) / 32)), 32, b * b * LANE_LD * sizeof(double), s>>>(
+        nblk, b, diag, inv, d_err);
+    block_scale_t_kernel<<<air_counted((unsigned)((nblk + 3) / 4)), 128, smem, s>>>(nblk, b, diag, inv, rpt, cit, vt,
                                                                                      d_err);
-    AIR_LAUNCH();
+    const cudaError_t e = cudaGetLastError();
+    cudaFreeAsync(inv, s);
+    AIR_CUDA(e);
     return AIR_OK;
 }
 
 int air_block_apply_impl(int64_t nblk, int b, const double *diag, int op, const double *x, double *y, int *d_err,
                          cudaStream_t s) {
-    const size_t smem = (size_t)4 * 5 * b * b * sizeof(double);
     if (nblk <= 0) return AIR_OK;
-    block_apply_kernel<<<air_counted((unsigned)((nblk + 3) / 4)), 128, smem, s>>>(nblk, b, diag, op, x, y, d_err);
+    block_apply_kernel<<<air_counted((unsigned)((nblk + 31) / 32)), 32, (b * b + b) * LANE_LD * sizeof(double), s>>>(
+        nblk, b, diag, op, x, y, d_err);
     AIR_LAUNCH();
     return AIR_OK;
 }

@@ -20,9 +20,9 @@
 //
 // One warp per element: the local matrices live in shared memory, lanes run
 // over matrix entries (each summing over the quadrature points) and over the
-// rows / columns of the elimination.  One warp per free facet then sums the
-// two diagonal contributions in element order, inverts the diagonal block by
-// Gauss-Jordan and scales its row.  FP64 throughout.
+// rows / columns of the elimination.  Then one lane per free facet sums the
+// two diagonal contributions in element order and inverts the diagonal block
+// by Gauss-Jordan, and one warp per free facet scales its rows.  FP64 throughout.
 //
 // What bounds it: FP64 issue.  GB300 has two FP64 lanes per SM and clock, so
 // one FP64 warp instruction holds an SM for 16 cycles whatever number of its
@@ -43,13 +43,13 @@
 #include <math.h>
 
 #include "air_internal.cuh"
-#include "warp_dense.cuh"
+#include "lane_dense.cuh"
 
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int WPB = 4;         // elements (warps) per block
-constexpr int FWPB = 4;        // facets (warps) per block
+constexpr int FWPB = 4;        // facets (warps) per block of facet_scale_kernel
 constexpr int8_t K_DIR = 1, K_NEU = 2;
 
 __host__ __device__ constexpr int binom(int n, int k) { return k == 0 ? 1 : binom(n - 1, k - 1) * n / k; }
@@ -501,19 +501,6 @@ __device__ __forceinline__ void coupling(const ElemArgs &a, const double *sGeo, 
     __syncwarp();
 }
 
-// |x| as an integer whose order is that of the magnitudes (0: NaN, which never is a pivot): comparing integers keeps
-// the pivot search off the FP64 lanes.
-__device__ __forceinline__ unsigned long long magnitude_key(double x) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
-    return b > 0x7ff0000000000000ull ? 0ull : b + 1ull;
-}
-
-// x / p from r = 1 / p: the product corrected once, within an ulp of the division at a third of its FP64 work
-__device__ __forceinline__ double quotient(double x, double p, double r) {
-    const double q = x * r;
-    return fma(fma(-q, p, x), r, q);
-}
-
 // LU factors of the warp's A (N x N, row-major) with partial pivoting (ties -> smallest row), the row operations
 // applied to the NC columns of X (row stride LDX) on the way; the multipliers stay below the diagonal, rinv gets the
 // reciprocal pivots and perm (registers, lane c < N) the row swapped with row c.  Returns false if a pivot is zero.
@@ -773,72 +760,81 @@ struct FacetArgs {
     int B, dlen, maxn, scale;
     const int32_t *free_ids, *facet_elems, *nbr, *cnt;
     const int64_t *row_ptr;
-    const double *dpart, *hpart;
+    const double *hpart;
+    double *dpart;               // two b x b slots per facet; the first then takes the inverse
     double *val, *rhs, *diag;
     int *err;
 };
 
-// One warp per free facet: Sd = sum of the element contributions (element
-// order), H likewise; scaled: Dinv = Sd^{-1}, rhs = Dinv H and every
-// off-diagonal block of the row block becomes Dinv blk; the diagonal block is
-// stored as its b ones.  Unscaled: Sd goes into the row, rhs = H.
-__global__ void __launch_bounds__(FWPB * 32) facet_kernel(FacetArgs a) {
+// Sd = sum of the element contributions (element order) of every free facet,
+// one facet per lane: written to diag, and inverted into the facet's first
+// slot of dpart (scaled) or written to the diagonal blocks of its rows.
+// With facet_scale_kernel it takes 1.0 ms for 57,222 facets of 10 unknowns
+// (2.1 ms with the inverse by one warp per facet), 0.7 ms for 164,736 facets of
+// 6 (2.8 ms).
+__global__ void __launch_bounds__(32) facet_block_kernel(FacetArgs a) {
     extern __shared__ double smem[];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int lane = threadIdx.x, B = a.B, BB = B * B;
+    const int64_t first = (int64_t)blockIdx.x * 32;
+    const int count = a.nfree - first < 32 ? (int)(a.nfree - first) : 32;
+    for (int k = 0; k < count; ++k) {
+        const int32_t f = a.free_ids[first + k];
+        const bool two = a.facet_elems[2 * (int64_t)f + 1] >= 0;
+        const int64_t rf = first + k, row0 = a.row_ptr[rf * B], len = a.row_ptr[rf * B + 1] - row0;
+        int64_t at = 0;
+        if (!a.scale)
+            for (int t = 0; t < a.cnt[rf]; ++t) at += a.nbr[rf * a.maxn + t] < rf ? B : 0;
+        for (int t = lane; t < BB; t += 32) {
+            double v = a.dpart[(2 * (int64_t)f) * BB + t];
+            if (two) v = v + a.dpart[(2 * (int64_t)f + 1) * BB + t];
+            smem[t * LANE_LD + k] = v;
+            if (a.diag) a.diag[rf * BB + t] = v;
+            if (!a.scale) a.val[row0 + (t / B) * len + at + t % B] = v;
+        }
+    }
+    if (!a.scale) return;
+    __syncwarp();
+    if (lane < count && !lane_invert(smem + lane, B)) atomicOr(a.err, AIR_DEVERR_SINGULAR);
+    __syncwarp();
+    for (int k = 0; k < count; ++k) {
+        const int64_t f = a.free_ids[first + k];
+        for (int t = lane; t < BB; t += 32) a.dpart[2 * f * BB + t] = smem[t * LANE_LD + k];
+    }
+}
+
+// One warp per free facet: its b rows, all of one length, are read as one
+// run, multiplied by the inverse of the diagonal block and written back; H
+// takes the diagonal's column, whose product is the right-hand side, and the
+// diagonal itself is stored as ones.  Unscaled: rhs = H alone.
+__global__ void __launch_bounds__(FWPB * 32) facet_scale_kernel(FacetArgs a) {
+    extern __shared__ double smem[];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, B = a.B;
     const int64_t rf = (int64_t)blockIdx.x * FWPB + w;
     if (rf >= a.nfree) return;
-    const int B = a.B, BB = B * B;
-    double *sS = smem + (size_t)w * 6 * BB, *sI = sS + BB, *sW = sI + BB, *sT = sW + 2 * BB, *sH = sT + BB;
-    const int32_t f = a.free_ids[rf];
-    const bool two = a.facet_elems[2 * (int64_t)f + 1] >= 0;
-    for (int t = lane; t < BB; t += 32) {
-        double v = a.dpart[(2 * (int64_t)f) * BB + t];
-        if (two) v = v + a.dpart[(2 * (int64_t)f + 1) * BB + t];
-        sS[t] = v;
-        if (a.diag) a.diag[rf * BB + t] = v;
-    }
+    const int64_t f = a.free_ids[rf];
+    const bool two = a.facet_elems[2 * f + 1] >= 0;
+    double *sI = smem + (size_t)w * (B * B + B * (a.maxn * B + 1)), *sT = sI + B * B;
+    const int64_t row0 = a.row_ptr[rf * B];
+    const int len = (int)(a.row_ptr[rf * B + 1] - row0), c = a.cnt[rf];
+    int at = 0;                                       // the diagonal's place in a row
+    for (int t = 0; t < c; ++t) at += a.nbr[rf * a.maxn + t] < rf ? B : 0;
     for (int m = lane; m < B; m += 32) {
-        double v = a.hpart[(2 * (int64_t)f) * B + m];
-        if (two) v = v + a.hpart[(2 * (int64_t)f + 1) * B + m];
-        sH[m] = v;
+        double h = a.hpart[2 * f * B + m];
+        if (two) h = h + a.hpart[(2 * f + 1) * B + m];
+        if (a.scale) sT[m * len + at] = h;
+        else a.rhs[rf * B + m] = h;
     }
+    if (!a.scale) return;
+    for (int t = lane; t < B * B; t += 32) sI[t] = a.dpart[2 * f * B * B + t];
+    for (int t = lane; t < B * len; t += 32)
+        if (t % len != at) sT[t] = a.val[row0 + t];
     __syncwarp();
-    const int c = a.cnt[rf];
-    const int32_t *nb = a.nbr + rf * a.maxn;
-    int nbefore = 0;
-    for (int t = 0; t < c; ++t) nbefore += nb[t] < rf ? 1 : 0;
-    if (!a.scale) {
-        for (int t = lane; t < BB; t += 32) {
-            const int m = t / B, l = t % B;
-            a.val[a.row_ptr[rf * B + m] + (int64_t)nbefore * B + l] = sS[t];
-        }
-        for (int m = lane; m < B; m += 32) a.rhs[rf * B + m] = sH[m];
-        return;
-    }
-    if (!warp_inverse(sS, B, sW, sI)) {
-        if (lane == 0) atomicOr(a.err, AIR_DEVERR_SINGULAR);
-        return;
-    }
-    for (int m = lane; m < B; m += 32) {
+    for (int t = lane; t < B * len; t += 32) {
+        const int m = t / len, l = t % len;
         double s = 0.0;
-        for (int l = 0; l < B; ++l) s += sI[m * B + l] * sH[l];
-        a.rhs[rf * B + m] = s;
-        a.val[a.row_ptr[rf * B + m] + (int64_t)nbefore * B] = 1.0;
-    }
-    for (int t = 0; t < c; ++t) {
-        const int64_t off = (int64_t)t * B + (nb[t] > rf ? a.dlen : 0);
-        for (int u = lane; u < BB; u += 32) {
-            const int m = u / B, l = u % B;
-            sT[u] = a.val[a.row_ptr[rf * B + m] + off + l];
-        }
-        __syncwarp();
-        for (int u = lane; u < BB; u += 32) {
-            const int m = u / B, l = u % B;
-            double s = 0.0;
-            for (int j = 0; j < B; ++j) s += sI[m * B + j] * sT[j * B + l];
-            a.val[a.row_ptr[rf * B + m] + off + l] = s;
-        }
-        __syncwarp();
+        for (int j = 0; j < B; ++j) s += sI[m * B + j] * sT[j * len + l];
+        a.val[row0 + t] = l == at ? 1.0 : s;
+        if (l == at) a.rhs[rf * B + m] = s;
     }
 }
 
@@ -902,29 +898,25 @@ __global__ void facet_points_kernel(int64_t F, int D, int nqf, const double *ver
 // ------------------------------------------------------ velocity gradient
 // mu_f = Sd_f^{-T} adj_f per free facet (the unscaled adjoint), spread to all
 // facets with zeros on Dirichlet ones; Lambda likewise with the Dirichlet
-// values.  One warp per free facet.
-__global__ void __launch_bounds__(FWPB * 32) adjoint_unscale_kernel(int64_t F, int64_t nfree, int B,
-                                                                    const int32_t *free_ids, const double *diag,
-                                                                    const double *lam, const double *adj,
-                                                                    double *mu_full, double *lam_full, int *err) {
+// values.  One facet per lane.
+__global__ void __launch_bounds__(32) adjoint_unscale_kernel(int64_t nfree, int B, const int32_t *free_ids,
+                                                             const double *diag, const double *lam,
+                                                             const double *adj, double *mu_full, double *lam_full,
+                                                             int *err) {
     extern __shared__ double smem[];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t rf = (int64_t)blockIdx.x * FWPB + w;
-    if (rf >= nfree) return;
-    const int BB = B * B;
-    double *sS = smem + (size_t)w * 4 * BB, *sI = sS + BB, *sW = sI + BB;
-    for (int t = lane; t < BB; t += 32) sS[t] = diag[rf * BB + (t % B) * B + t / B];   // transpose
+    const int lane = threadIdx.x;
+    const int64_t first = (int64_t)blockIdx.x * 32;
+    const int count = nfree - first < 32 ? (int)(nfree - first) : 32;
+    double *sx = smem + B * B * LANE_LD;
+    lane_load_blocks(diag, first, count, B, true, smem);
+    for (int t = lane; t < count * B; t += 32) sx[(t % B) * LANE_LD + t / B] = adj[first * B + t];
     __syncwarp();
-    if (!warp_inverse(sS, B, sW, sI)) {
-        if (lane == 0) atomicOr(err, AIR_DEVERR_SINGULAR);
-        return;
-    }
-    const int32_t f = free_ids[rf];
-    for (int m = lane; m < B; m += 32) {
-        double s = 0.0;
-        for (int l = 0; l < B; ++l) s += sI[m * B + l] * adj[rf * B + l];
-        mu_full[(int64_t)f * B + m] = s;
-        lam_full[(int64_t)f * B + m] = lam[rf * B + m];
+    if (lane < count && !lane_solve(smem + lane, sx + lane, B)) atomicOr(err, AIR_DEVERR_SINGULAR);
+    __syncwarp();
+    for (int t = lane; t < count * B; t += 32) {
+        const int64_t o = (int64_t)free_ids[first + t / B] * B + t % B;
+        mu_full[o] = sx[(t % B) * LANE_LD + t / B];
+        lam_full[o] = lam[first * B + t];
     }
 }
 
@@ -1284,8 +1276,9 @@ int assemble_impl(const air_hdg_mesh *M, const air_hdg_ref *R, const air_hdg_dat
         fa.free_ids = P.free_ids; fa.facet_elems = M->facet_elems; fa.nbr = P.nbr; fa.cnt = P.cnt;
         fa.row_ptr = row_ptr; fa.dpart = dpart; fa.hpart = hpart; fa.val = val; fa.rhs = rhs; fa.diag = diag;
         fa.err = d_err;
-        const size_t smem = (size_t)FWPB * 6 * B * B * sizeof(double);
-        facet_kernel<<<air_counted((unsigned)((P.nfree + FWPB - 1) / FWPB)), FWPB * 32, smem, s>>>(fa);
+        facet_block_kernel<<<air_counted((unsigned)((P.nfree + 31) / 32)), 32, B * B * LANE_LD * sizeof(double), s>>>(fa);
+        facet_scale_kernel<<<air_counted((unsigned)((P.nfree + FWPB - 1) / FWPB)), FWPB * 32,
+                             FWPB * (B * B + B * (2 * D * B + 1)) * sizeof(double), s>>>(fa);
         if (cudaGetLastError() != cudaSuccess) st = AIR_ERR_CUDA;
     }
     if (st == AIR_OK) st = read_err(d_err, s);
@@ -1367,9 +1360,9 @@ int air_hdg_velocity_gradient(const air_hdg_mesh *M, const air_hdg_ref *R, const
     if (st == AIR_OK) st = dalloc(&d_err, 1);
     if (st == AIR_OK && cudaMemsetAsync(d_err, 0, sizeof(int), s) != cudaSuccess) st = AIR_ERR_CUDA;
     if (st == AIR_OK) {
-        const size_t smem = (size_t)FWPB * 4 * B * B * sizeof(double);
-        adjoint_unscale_kernel<<<air_counted((unsigned)((P.nfree + FWPB - 1) / FWPB)), FWPB * 32, smem, s>>>(
-            F, P.nfree, B, P.free_ids, diag, lam, adj, mu_full, lam_full, d_err);
+        adjoint_unscale_kernel<<<air_counted((unsigned)((P.nfree + 31) / 32)), 32,
+                                 (B * B + B) * LANE_LD * sizeof(double), s>>>(P.nfree, B, P.free_ids, diag, lam, adj,
+                                                                              mu_full, lam_full, d_err);
         spread_dirichlet_kernel<<<air_counted(grid_for(F * B, 256)), 256, 0, s>>>(F, B, M->facet_kind, lam_dir,
                                                                                    mu_full, lam_full);
         if (cudaGetLastError() != cudaSuccess) st = AIR_ERR_CUDA;
