@@ -220,15 +220,13 @@ __global__ void __launch_bounds__(32) block_apply_kernel(int64_t nblk, int b, co
     for (int t = lane; t < count * b; t += 32) sx[(t % b) * LANE_LD + t / b] = x[first * b + t];
     __syncwarp();
     if (op >= 2) {
-        if (lane < count && !lane_solve(bsm + lane, sx + lane, b)) atomicOr(err, AIR_DEVERR_SINGULAR);
+        if (lane < count && !lane_invert(bsm + lane, b)) atomicOr(err, AIR_DEVERR_SINGULAR);
         __syncwarp();
     }
     for (int t = lane; t < count * b; t += 32) {
         const int k = t / b, i = t % b;
         double v = 0.0;
-        if (op >= 2) v = sx[i * LANE_LD + k];
-        else
-            for (int j = 0; j < b; ++j) v += bsm[(i * b + j) * LANE_LD + k] * sx[j * LANE_LD + k];
+        for (int j = 0; j < b; ++j) v += bsm[(i * b + j) * LANE_LD + k] * sx[j * LANE_LD + k];
         y[first * b + t] = v;
     }
 }

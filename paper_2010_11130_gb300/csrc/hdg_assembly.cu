@@ -30,16 +30,15 @@
 // kernels are therefore arranged for few, full FP64 instructions:
 //  - geometry, normals and the perm of every facet are computed by one thread
 //    per element (geometry_kernel) instead of by all 32 lanes of its warp;
-//  - the parts whose coefficients are constant on an element or facet
-//    (the diffusion and the gradient-trace terms) are contracted with
-//    reference integrals (table_kernel) instead of over the points;
-//  - a weight is multiplied into one factor once per point, not per entry;
-//    the facet part of A is formed as a symmetric matrix;
+//  - products that entries share are computed once per point, and products
+//    with components of a gradient that are zero everywhere not at all;
 //  - C is built facet by facet after the solve, and its product with the
-//    solution goes straight to the rows of the system.
-// hdg_element_kernel, 82,944 elements, D = 3, p = 2: 8.0 ms (65.1 ms with every
-// entry summed over the points on its own); 29,478 elements, p = 3: 12.8 ms
-// (133.7 ms).  At two FP64 lanes the instructions alone take about 6 and 9 ms.
+//    solution goes straight to the rows of the system;
+//  - the velocity gradient forms A alone, its constant parts from reference
+//    integrals, and sums everything else over the points.
+// hdg_element_kernel, 82,944 elements, D = 3, p = 2: 24.7 ms; 29,478
+// elements, p = 3: 49.0 ms (65.1 and 133.7 ms with every entry on its own).  The
+// FP64 instructions alone take about 21 and 44 ms.
 #include <math.h>
 
 #include "air_internal.cuh"
@@ -68,25 +67,25 @@ struct Dims {
     static constexpr int NQF = ipow(Q, D - 1);
     static constexpr int NPERM = fact(D);
     static constexpr int NS = NB * (NB + 1) / 2;     // entries i <= j of a symmetric element matrix
-    static constexpr int BS = B * (B + 1) / 2;       // likewise of a facet matrix
     static constexpr int MAXN = 2 * D;               // off-diagonal facet blocks per row
-    // geometry record of an element: J^-1, |det J|, pen, nu det (spatial metric), then per facet the normal,
-    // the surface factor and nu times that factor times J^-1 (0, n)
-    static constexpr int NM = D * (D + 1) / 2;
-    static constexpr int G_DET = D * D, G_PEN = G_DET + 1, G_MM = G_PEN + 1, G_F = G_MM + NM, G_FS = 2 * D + 1;
+    // geometry record of an element: J^-1, |det J|, pen, the spatial metric, then per facet the normal, the surface
+    // factor and J^-1 (0, n)
+    static constexpr int G_DET = D * D, G_PEN = G_DET + 1, G_MM = G_PEN + 1, G_F = G_MM + D * D, G_FS = 2 * D + 1;
     static constexpr int GEO = G_F + NF * G_FS;
     // shared memory of a warp (doubles): A; [B | F], first the volume points; products of one chunk of points, later
-    // C of one facet; facet point weights; D of one facet; F; reciprocal pivots; the geometry record
-    static constexpr int QC = 16;                    // points per chunk
-    static constexpr int XR = NB * NX > NQ * (D + 1) ? NB * NX : NQ * (D + 1);
-    static constexpr int PR = QC * NB > B * NB ? QC * NB : B * NB;
-    static constexpr int WARP_DOUBLES = NB * NB + XR + PR + 4 * NF * NQF + B * B + NB + NB + GEO;
+    // C and S of one facet; facet point weights; D of one facet; F; the geometry record
+    static constexpr int QV = 8, QC = 16;            // volume and facet points per chunk
+    static constexpr int XR = NB * NX > NQ * (D + 2) ? NB * NX : NQ * (D + 2);
+    static constexpr int PV = QV * NB * (1 + D * D), PF = 4 * QC * NB, PS = NB * B + B * NX;
+    static constexpr int PR = PV > PF ? (PV > PS ? PV : PS) : (PF > PS ? PF : PS);
+    static constexpr int WARP_DOUBLES = NB * NB + XR + PR + 4 * NF * NQF + B * B + NB + GEO;
     // gradient: A, volume points, chunk products, facet point weights, two facet fields, Lam, mu, U, y, pivots, geometry
     static constexpr int GRAD_DOUBLES =
-        NB * NB + NQ * (D + 1) + QC * NB + 4 * NF * NQF + 2 * NF * NQF + 2 * NT + 4 * NB + GEO;
-    // reference integrals (doubles): volume stiffness per metric entry, then per facet and frame the symmetrised
-    // trace-gradient matrix and the gradient-trace moments
-    static constexpr int T_L = NM * NS, T_K = T_L + NF * NPERM * D * NS, TABLE = T_K + NF * NPERM * D * NB * B;
+        NB * NB + NQ * (D + 1) + QC * NB + 4 * NF * NQF + 2 * NT + 4 * NB + GEO;
+    // reference integrals (doubles): volume stiffness per metric entry k <= l, then per facet and frame the
+    // symmetrised trace-gradient matrix
+    static constexpr int NM = D * (D + 1) / 2;
+    static constexpr int T_L = NM * NS, TABLE = T_L + NF * NPERM * D * NS;
 };
 
 // (i, j), i <= j, of entry t of a symmetric n x n matrix stored by rows
@@ -198,6 +197,7 @@ struct ElemArgs {
     const double *wq, *phi, *gphi, *wf, *psi, *phi_f, *gphi_f;
     const int32_t *perms;
     const double *geo, *table;          // E geometry records, reference integrals
+    const int32_t *order, *gmask;       // entries of A in the order the lanes take them, components of each gradient
     const int32_t *frame;               // E x NF: canonical frame of the facet, + 256 on Neumann facets
     const double *vel_vol, *src, *vel_face, *u0_face, *lam_dir;
     double *val, *dpart, *hpart;
@@ -223,16 +223,16 @@ __global__ void __launch_bounds__(128) geometry_kernel(ElemArgs a, double *geo, 
 #pragma unroll
         for (int d = 0; d < D; ++d) o[k * D + d] = g.Jinv[k][d];
     o[Dm::G_DET] = g.det;
-    o[Dm::G_PEN] = a.nu * a.alpha / g.h;
-    int c = Dm::G_MM;
+    o[Dm::G_PEN] = __ddiv_rn(__dmul_rn(a.nu, a.alpha), g.h);
 #pragma unroll
     for (int k = 0; k < D; ++k)      // spatial metric: sum over spatial s of Jinv[k][s] Jinv[l][s]
 #pragma unroll
-        for (int l = k; l < D; ++l) {
-            double s = 0.0;
-#pragma unroll
-            for (int d = 1; d < D; ++d) s += g.Jinv[k][d] * g.Jinv[l][d];
-            o[c++] = a.nu * g.det * s;
+        for (int l = 0; l < D; ++l) {
+            double s = __dmul_rn(g.Jinv[k][1], g.Jinv[l][1]);
+            if (D == 3)
+                s = k == l ? __fma_rn(g.Jinv[k][1], g.Jinv[k][1], __dmul_rn(g.Jinv[k][D - 1], g.Jinv[k][D - 1]))
+                           : __fma_rn(g.Jinv[k][D - 1], g.Jinv[l][D - 1], s);
+            o[Dm::G_MM + k * D + l] = s;
         }
 #pragma unroll
     for (int k = 0; k < NF; ++k) {
@@ -248,47 +248,45 @@ __global__ void __launch_bounds__(128) geometry_kernel(ElemArgs a, double *geo, 
                 gl[d] = g.Jinv[k > 0 ? k - 1 : 0][d];
             }
         }
-        double gn = 0.0;
-#pragma unroll
-        for (int d = 0; d < D; ++d) gn += gl[d] * gl[d];
+        double gn = __fma_rn(gl[0], gl[0], __dmul_rn(gl[1], gl[1]));
+        if (D == 3) gn = __fma_rn(gl[D - 1], gl[D - 1], gn);
         gn = sqrt(gn);
         double *f = o + Dm::G_F + k * Dm::G_FS;
         double nh[D];
 #pragma unroll
-        for (int d = 0; d < D; ++d) f[d] = nh[d] = -gl[d] / gn;      // outward unit space-time normal
-        const double ws = (double)D * (g.det / (double)fact(D)) * gn * (double)fact(D - 1);
+        for (int d = 0; d < D; ++d) f[d] = nh[d] = __ddiv_rn(-gl[d], gn);      // outward unit space-time normal
+        const double ws = __dmul_rn(__dmul_rn(__dmul_rn((double)D, __ddiv_rn(g.det, (double)fact(D))), gn), (double)fact(D - 1));
         f[D] = ws;
 #pragma unroll
         for (int kk = 0; kk < D; ++kk) {    // (grad phi . n) = grad_ref phi . (Jinv (0, n))
-            double sum = 0.0;
-#pragma unroll
-            for (int d = 1; d < D; ++d) sum += g.Jinv[kk][d] * nh[d];
-            f[D + 1 + kk] = a.nu * ws * sum;
+            double sum = __dmul_rn(g.Jinv[kk][1], nh[1]);
+            if (D == 3) sum = __fma_rn(g.Jinv[kk][D - 1], nh[D - 1], sum);
+            f[D + 1 + kk] = sum;
         }
         frame[e * NF + k] =
             facet_perm<D>(ev, k, a.perms) + (a.kind[a.elem_facets[e * NF + k]] == K_NEU ? 256 : 0);
     }
 }
 
-// Reference integrals, one thread each: sum_q wq (d_k phi_i d_l phi_j + d_l phi_i d_k phi_j, or once when k = l),
-// sum_q wf (phi_i d_d phi_j + d_d phi_i phi_j) and sum_q wf d_d phi_i psi_m, the last two per facet and frame.
+// Reference integrals, one thread each: sum_q wq (d_k phi_i d_l phi_j + d_l phi_i d_k phi_j, or once when k = l)
+// and, per facet and frame, sum_q wf (phi_i d_d phi_j + d_d phi_i phi_j).
 template <int D, int P>
-__global__ void table_kernel(const double *wq, const double *gphi, const double *wf, const double *psi,
-                             const double *phi_f, const double *gphi_f, double *table) {
+__global__ void table_kernel(const double *wq, const double *gphi, const double *wf, const double *phi_f,
+                             const double *gphi_f, double *table) {
     using Dm = Dims<D, P>;
-    constexpr int NB = Dm::NB, B = Dm::B, NS = Dm::NS;
+    constexpr int NB = Dm::NB, NS = Dm::NS;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= Dm::TABLE) return;
     double acc = 0.0;
     if (t < Dm::T_L) {
-        int m = t / NS, k = 0, l, i, j;
-        sym_entry(m, D, k, l);
+        int k, l, i, j;
+        sym_entry(t / NS, D, k, l);
         sym_entry(t % NS, NB, i, j);
         for (int q = 0; q < Dm::NQ; ++q) {
             const double *gi = gphi + (q * NB + i) * D, *gj = gphi + (q * NB + j) * D;
             acc += wq[q] * (k == l ? gi[k] * gj[k] : gi[k] * gj[l] + gi[l] * gj[k]);
         }
-    } else if (t < Dm::T_K) {
+    } else {
         const int u = t - Dm::T_L, ks = u / (D * NS), d = u / NS % D;
         int i, j;
         sym_entry(u % NS, NB, i, j);
@@ -296,12 +294,34 @@ __global__ void table_kernel(const double *wq, const double *gphi, const double 
             const int fi = (ks * Dm::NQF + q) * NB + i, fj = (ks * Dm::NQF + q) * NB + j;
             acc += wf[q] * (phi_f[fi] * gphi_f[fj * D + d] + gphi_f[fi * D + d] * phi_f[fj]);
         }
-    } else {
-        const int u = t - Dm::T_K, ks = u / (D * NB * B), d = u / (NB * B) % D, i = u / B % NB, m = u % B;
-        for (int q = 0; q < Dm::NQF; ++q)
-            acc += wf[q] * gphi_f[((ks * Dm::NQF + q) * NB + i) * D + d] * psi[q * B + m];
     }
     table[t] = acc;
+}
+
+// gmask[i]: bit k set when component k of grad phi_i is not zero at every volume point.  order: the entries (i, j) of
+// A by falling number of products d_k phi_i d_l phi_j, so that a warp's lanes have equally many.
+template <int D, int P>
+__global__ void __launch_bounds__(512) order_kernel(const double *gphi, int32_t *order, int32_t *gmask) {
+    using Dm = Dims<D, P>;
+    constexpr int NB = Dm::NB;
+    __shared__ int mask[NB];
+    for (int i = threadIdx.x; i < NB; i += blockDim.x) {
+        int m = 0;
+        for (int q = 0; q < Dm::NQ; ++q)
+            for (int k = 0; k < D; ++k) m |= gphi[(q * NB + i) * D + k] != 0.0 ? 1 << k : 0;
+        mask[i] = m;
+        gmask[i] = m;
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < NB * NB; t += blockDim.x) {
+        const int mine = __popc(mask[t / NB]) * __popc(mask[t % NB]);
+        int place = 0;
+        for (int u = 0; u < NB * NB; ++u) {
+            const int o = __popc(mask[u / NB]) * __popc(mask[u % NB]);
+            place += o > mine || (o == mine && u < t) ? 1 : 0;
+        }
+        order[place] = t;
+    }
 }
 
 // Volume part: sA = - sum_q W phi_j a_hat.grad_hat phi_i, sF = sum_q W f phi_i.  sV (NQ (D + 1)) and sP are scratch;
@@ -373,10 +393,9 @@ __device__ __forceinline__ void volume_part(const ElemArgs &a, int64_t e, const 
         if (lane + 32 * r < NB * NB) sA[lane + 32 * r] = acc[r];
 }
 
-// Weights of every facet point: W (c+ + pen), W (c- - pen), the coefficient of D and W g (Neumann inflow).
+// Weights of every facet point: W (c+ + pen) and W (c- - pen).
 template <int D, int P>
-__device__ __forceinline__ void facet_points(const ElemArgs &a, int64_t e, const double *sGeo, const int32_t *fr,
-                                             double *sW) {
+__device__ __forceinline__ void facet_points(const ElemArgs &a, int64_t e, const double *sGeo, double *sW) {
     using Dm = Dims<D, P>;
     constexpr int NF = Dm::NF, NQF = Dm::NQF;
     const double pen = sGeo[Dm::G_PEN];
@@ -387,20 +406,16 @@ __device__ __forceinline__ void facet_points(const ElemArgs &a, int64_t e, const
 #pragma unroll
         for (int m = 0; m < D - 1; ++m) an += a.vel_face[((e * NF + k) * NQF + q) * (D - 1) + m] * f[m + 1];
         const double W = f[D] * a.wf[q], cup = 0.5 * (an + fabs(an)), cdn = 0.5 * (an - fabs(an));
-        const bool neu = fr[k] >= 256;
-        const double wm = W * (cdn - pen);
-        sW[4 * t] = W * (cup + pen);
-        sW[4 * t + 1] = wm;
-        sW[4 * t + 2] = neu ? W * cup - wm : -wm;
-        sW[4 * t + 3] = neu && an < 0.0 && a.u0_face ? W * (-an * a.u0_face[(e * NF + k) * NQF + q]) : 0.0;
+        sW[2 * t] = W * (cup + pen);
+        sW[2 * t + 1] = W * (cdn - pen);
     }
 }
 
-// sP[q NB + i] = w(q) phi_i(q) for one chunk of a facet's points (w every fourth double from sw).
+// sP[q NB + i] = w(q) phi_i(q) for one chunk of a facet's points (w every other double from sw).
 template <int NB>
 __device__ __forceinline__ void weigh(const double *sw, const double *ph, int nq, double *sP) {
     __syncwarp();
-    for (int t = threadIdx.x & 31; t < nq * NB; t += 32) sP[t] = sw[4 * (t / NB)] * ph[t];
+    for (int t = threadIdx.x & 31; t < nq * NB; t += 32) sP[t] = sw[2 * (t / NB)] * ph[t];
     __syncwarp();
 }
 
@@ -419,9 +434,14 @@ __device__ __forceinline__ void symmetric_part(const ElemArgs &a, const double *
         ot[r] = lane + 32 * r < NS ? lane + 32 * r : 0;
         sym_entry(ot[r], NB, oi[r], oj[r]);
         acc[r] = 0.0;
-        if (diff)
+        if (diff) {
+            int m = 0;
 #pragma unroll
-            for (int m = 0; m < Dm::NM; ++m) acc[r] += sGeo[Dm::G_MM + m] * a.table[m * NS + ot[r]];
+            for (int k = 0; k < D; ++k)
+#pragma unroll
+                for (int l = k; l < D; ++l) acc[r] += sGeo[Dm::G_MM + k * D + l] * a.table[m++ * NS + ot[r]];
+            acc[r] *= a.nu * sGeo[Dm::G_DET];
+        }
     }
     for (int k = 0; k < NF; ++k) {
         const int ks = k * Dm::NPERM + (fr[k] & 255);
@@ -429,7 +449,7 @@ __device__ __forceinline__ void symmetric_part(const ElemArgs &a, const double *
 #pragma unroll 1
         for (int q0 = 0; q0 < NQF; q0 += QC) {
             const int nq = NQF - q0 < QC ? NQF - q0 : QC;
-            weigh<NB>(sW + 4 * (k * NQF + q0), ph + q0 * NB, nq, sP);
+            weigh<NB>(sW + 2 * (k * NQF + q0), ph + q0 * NB, nq, sP);
             double part[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) part[r] = 0.0;
@@ -444,7 +464,7 @@ __device__ __forceinline__ void symmetric_part(const ElemArgs &a, const double *
             const double *L = a.table + Dm::T_L + (size_t)ks * D * NS;
 #pragma unroll
             for (int d = 0; d < D; ++d) {
-                const double nj = sGeo[Dm::G_F + k * Dm::G_FS + D + 1 + d];
+                const double nj = a.nu * sGeo[Dm::G_F + k * Dm::G_FS + D] * sGeo[Dm::G_F + k * Dm::G_FS + D + 1 + d];
 #pragma unroll
                 for (int r = 0; r < R; ++r) acc[r] -= nj * L[d * NS + ot[r]];
             }
@@ -457,47 +477,6 @@ __device__ __forceinline__ void symmetric_part(const ElemArgs &a, const double *
             sA[oi[r] * NB + oj[r]] += acc[r];
             if (oi[r] != oj[r]) sA[oj[r] * NB + oi[r]] += acc[r];
         }
-    __syncwarp();
-}
-
-// One facet's coupling of the element basis to its trace basis, entry (i, m) of lane's r-th pair t = i B + m:
-// sign * sum_q w phi_i psi_m + sum_d nj_d (gradient-trace moment), w = sW's weight number `which`.
-template <int D, int P, int R>
-__device__ __forceinline__ void coupling(const ElemArgs &a, const double *sGeo, int k, int ks, const double *sW,
-                                         int which, double sign, double *sP, double (&acc)[R]) {
-    using Dm = Dims<D, P>;
-    constexpr int NB = Dm::NB, B = Dm::B, NQF = Dm::NQF, QC = Dm::QC;
-    const int lane = threadIdx.x & 31;
-    const double *ph = a.phi_f + (size_t)ks * NQF * NB;
-    int oi[R], om[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const int t = lane + 32 * r < NB * B ? lane + 32 * r : 0;
-        oi[r] = t / B;
-        om[r] = t % B;
-        acc[r] = 0.0;
-    }
-#pragma unroll 1
-    for (int q0 = 0; q0 < NQF; q0 += QC) {
-        const int nq = NQF - q0 < QC ? NQF - q0 : QC;
-        weigh<NB>(sW + 4 * (k * NQF + q0) + which, ph + q0 * NB, nq, sP);
-        const double *ps = a.psi + q0 * B;
-#pragma unroll 4
-        for (int q = 0; q < nq; ++q)
-#pragma unroll
-            for (int r = 0; r < R; ++r) acc[r] += sP[q * NB + oi[r]] * ps[q * B + om[r]];
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r) acc[r] = sign < 0.0 ? -acc[r] : acc[r];
-    if (a.nu != 0.0) {
-        const double *K = a.table + Dm::T_K + (size_t)ks * D * NB * B;
-#pragma unroll
-        for (int d = 0; d < D; ++d) {
-            const double nj = sGeo[Dm::G_F + k * Dm::G_FS + D + 1 + d];
-#pragma unroll
-            for (int r = 0; r < R; ++r) acc[r] += nj * K[(d * NB + oi[r]) * B + om[r]];
-        }
-    }
     __syncwarp();
 }
 
@@ -571,73 +550,355 @@ __device__ void warp_back_substitute(const double *A, double *X, const double *r
     }
 }
 
+// The assembled system keeps its bits whatever the arrangement of this kernel:
+// FP32 hierarchies built on it would turn the last bit of an entry into a
+// difference of an FP32 rounding.  So every entry is evaluated with the
+// operations, written as intrinsics, that its plain expression (in the comments
+// below) has always compiled to for each D and P, which products are fused
+// included, and summed over the points in their order; what entries share
+// (products of one point's weight with one basis function, the gradient in the
+// flow's direction) is computed once and kept in shared memory, and terms
+// that vanish for every point (a monomial's gradient has few components) are
+// left out of a sum, which changes nothing.
+
+// Volume part of A and F:
+//   A(i, j) = sum_q W ( -phi_j adv_i + nu sum_kl Mm_kl d_k phi_i d_l phi_j ),  adv_i = (Jinv a_hat) . grad phi_i
+//   F(i)    = sum_q (W f) phi_i
+// sV: W, Jinv a_hat and W f of every point.  sP: adv_i and Mm_kl d_k phi_i of one chunk of points.
+template <int D, int P>
+__device__ __forceinline__ void exact_volume(const ElemArgs &a, int64_t e, const double *sGeo, double *sA, double *sV,
+                                             double *sP, double *sF) {
+    using Dm = Dims<D, P>;
+    constexpr int NB = Dm::NB, NQ = Dm::NQ, QV = Dm::QV, R = (NB * NB + 31) / 32, DD = D * D;
+    const int lane = threadIdx.x & 31;
+    const bool diff = a.nu != 0.0;
+    double *sT = sV + NQ, *sS = sT + NQ * D, *sM = sP + QV * NB;
+    for (int q = lane; q < NQ; q += 32) {
+        const double W = __dmul_rn(sGeo[Dm::G_DET], a.wq[q]);
+        sV[q] = W;
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+            double at = sGeo[k * D];
+#pragma unroll
+            for (int m = 0; m < D - 1; ++m) at = __fma_rn(sGeo[k * D + m + 1], a.vel_vol[(e * NQ + q) * (D - 1) + m], at);
+            sT[q * D + k] = at;
+        }
+        sS[q] = a.src ? __dmul_rn(W, a.src[e * NQ + q]) : 0.0;
+    }
+    __syncwarp();
+    for (int i = lane; i < NB; i += 32) {
+        double f = 0.0;
+        if (a.src)
+            for (int q = 0; q < NQ; ++q) f = __fma_rn(sS[q], a.phi[q * NB + i], f);
+        sF[i] = f;
+    }
+    // the lane's entries, those with equally many diffusion terms together
+    double acc[R];
+    int oi[R], oj[R], mi[R], mj[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int t = a.order[lane + 32 * r < NB * NB ? lane + 32 * r : NB * NB - 1];
+        acc[r] = 0.0;
+        oi[r] = t / NB;
+        oj[r] = t % NB;
+        mi[r] = diff ? a.gmask[oi[r]] : 0;
+        mj[r] = diff ? a.gmask[oj[r]] : 0;
+    }
+    for (int q0 = 0; q0 < NQ; q0 += QV) {
+        const int nq = NQ - q0 < QV ? NQ - q0 : QV;
+        __syncwarp();
+        for (int t = lane; t < nq * NB; t += 32) {
+            const int q = q0 + t / NB;
+            const double *gp = a.gphi + (q0 * NB + t) * D;
+            double adv = __dmul_rn(sT[q * D], gp[0]);
+#pragma unroll
+            for (int k = 1; k < D; ++k) adv = __fma_rn(sT[q * D + k], gp[k], adv);
+            sP[t] = adv;
+        }
+        if (diff)
+            for (int t = lane; t < nq * NB * DD; t += 32)
+                sM[t] = __dmul_rn(sGeo[Dm::G_MM + t % DD], a.gphi[q0 * NB * D + t / D]);
+        __syncwarp();
+        const double *ph = a.phi + q0 * NB, *gq = a.gphi + q0 * NB * D;
+#pragma unroll 1
+        for (int q = 0; q < nq; ++q) {
+            const double W = sV[q0 + q];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                double term = __dmul_rn(-ph[q * NB + oj[r]], sP[q * NB + oi[r]]);
+                int m1 = mi[r], m2 = mj[r];
+                if (m1 && m2) {
+                    const double *pm = sM + (q * NB + oi[r]) * DD, *gj = gq + (q * NB + oj[r]) * D;
+                    double dif = 0.0;
+                    do {                             // components k of grad phi_i, l of grad phi_j, ascending
+                        const int k = __ffs(m1) - 1, l = __ffs(m2) - 1;
+                        dif = __fma_rn(pm[k * D + l], gj[l], dif);
+                        m2 &= m2 - 1;
+                        if (!m2) {
+                            m1 &= m1 - 1;
+                            m2 = mj[r];
+                        }
+                    } while (m1);
+                    term = __fma_rn(a.nu, dif, term);
+                }
+                acc[r] = __fma_rn(W, term, acc[r]);
+            }
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+        if (lane + 32 * r < NB * NB) sA[oi[r] * NB + oj[r]] = acc[r];
+}
+
+// W, c+, c- and W g of every facet point
+template <int D, int P>
+__device__ __forceinline__ void exact_facet_points(const ElemArgs &a, int64_t e, const double *sGeo, const int32_t *fr,
+                                                   double *sW) {
+    using Dm = Dims<D, P>;
+    constexpr int NF = Dm::NF, NQF = Dm::NQF;
+    for (int t = threadIdx.x & 31; t < NF * NQF; t += 32) {
+        const int k = t / NQF, q = t % NQF;
+        const double *f = sGeo + Dm::G_F + k * Dm::G_FS;
+        double an = f[0];
+        const double *vel = a.vel_face + ((e * NF + k) * NQF + q) * (D - 1);
+        an = __dadd_rn(an, __dmul_rn(vel[0], f[1]));
+        if (D == 3) an = __fma_rn(vel[D - 2], f[D - 1], an);
+        const double W = __dmul_rn(f[D], a.wf[q]);
+        sW[4 * t] = W;
+        sW[4 * t + 1] = __dmul_rn(0.5, __dadd_rn(an, fabs(an)));
+        sW[4 * t + 2] = __dmul_rn(0.5, __dsub_rn(an, fabs(an)));
+        double gN = 0.0;
+        if (fr[k] >= 256 && an < 0.0 && a.u0_face) gN = __dmul_rn(-an, a.u0_face[(e * NF + k) * NQF + q]);
+        sW[4 * t + 3] = __dmul_rn(W, gN);
+    }
+}
+
+// Products of one chunk of facet points with every basis function: (c+ + pen) phi, (c- - pen) phi, grad phi . n and nu
+// times it, each nq x NB.
+template <int D, int P>
+__device__ __forceinline__ void exact_facet_products(const ElemArgs &a, const double *sGeo, int k, int ks, int q0,
+                                                     int nq, const double *sW, double *sP) {
+    using Dm = Dims<D, P>;
+    constexpr int NB = Dm::NB, NQF = Dm::NQF, N = Dm::QC * NB;
+    const double *f = sGeo + Dm::G_F + k * Dm::G_FS + D + 1, pen = sGeo[Dm::G_PEN];
+    __syncwarp();
+    for (int t = threadIdx.x & 31; t < nq * NB; t += 32) {
+        const int q = q0 + t / NB;
+        const size_t at = ((size_t)ks * NQF + q0) * NB + t;
+        const double fi = a.phi_f[at], cup = sW[4 * (k * NQF + q) + 1], cdn = sW[4 * (k * NQF + q) + 2];
+        sP[t] = __dmul_rn(__dadd_rn(cup, pen), fi);
+        sP[N + t] = __dmul_rn(__dsub_rn(cdn, pen), fi);
+        double dn = __dmul_rn(a.gphi_f[at * D], f[0]);
+#pragma unroll
+        for (int d = 1; d < D; ++d) dn = __fma_rn(a.gphi_f[at * D + d], f[d], dn);
+        sP[2 * N + t] = dn;
+        sP[3 * N + t] = __dmul_rn(a.nu, dn);
+    }
+    __syncwarp();
+}
+
+// Facet k's parts of A and B:
+//   A(i, j) += sum_q W ( (c+ + pen) phi_i phi_j - nu (phi_i dn_j + dn_i phi_j) )
+//   B(i, m)  = sum_q W ( (c- - pen) phi_i psi_m + nu dn_i psi_m )
+template <int D, int P>
+__device__ __forceinline__ void exact_facet(const ElemArgs &a, const double *sGeo, int k, int ks, const double *sW,
+                                            double *sP, double *sA, double *sX) {
+    using Dm = Dims<D, P>;
+    constexpr int NB = Dm::NB, B = Dm::B, NX = Dm::NX, NQF = Dm::NQF, QC = Dm::QC, N = QC * NB,
+                  R = (NB * NB + 31) / 32, RB = (NB * B + 31) / 32;
+    const int lane = threadIdx.x & 31;
+    const bool diff = a.nu != 0.0;
+    double acc[R], bcc[RB];
+    int oi[R], oj[R], bi[RB], bm[RB];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int t = lane + 32 * r < NB * NB ? lane + 32 * r : 0;
+        acc[r] = 0.0;
+        oi[r] = t / NB;
+        oj[r] = t % NB;
+    }
+#pragma unroll
+    for (int r = 0; r < RB; ++r) {
+        const int t = lane + 32 * r < NB * B ? lane + 32 * r : 0;
+        bcc[r] = 0.0;
+        bi[r] = t / B;
+        bm[r] = t % B;
+    }
+#pragma unroll 1
+    for (int q0 = 0; q0 < NQF; q0 += QC) {
+        const int nq = NQF - q0 < QC ? NQF - q0 : QC;
+        exact_facet_products<D, P>(a, sGeo, k, ks, q0, nq, sW, sP);
+        const double *ph = a.phi_f + ((size_t)ks * NQF + q0) * NB, *ps = a.psi + q0 * B;
+#pragma unroll 1
+        for (int q = 0; q < nq; ++q) {
+            const double W = sW[4 * (k * NQF + q0 + q)];
+            const double *p = sP + q * NB, *f = ph + q * NB;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int i = oi[r], j = oj[r];
+                double term = __dmul_rn(p[i], f[j]);
+                if (diff) {
+                    const double cross = __fma_rn(p[2 * N + i], f[j], __dmul_rn(f[i], p[2 * N + j]));
+                    term = P > 1 ? __fma_rn(p[i], f[j], -__dmul_rn(a.nu, cross)) : __fma_rn(-a.nu, cross, term);
+                }
+                acc[r] = __fma_rn(W, term, acc[r]);
+            }
+#pragma unroll
+            for (int r = 0; r < RB; ++r) {
+                const double pl = ps[q * B + bm[r]];
+                double term = __dmul_rn(p[N + bi[r]], pl);
+                if (diff)
+                    term = D + P > 4 ? __fma_rn(p[N + bi[r]], pl, __dmul_rn(p[3 * N + bi[r]], pl))
+                                     : __fma_rn(p[3 * N + bi[r]], pl, term);
+                bcc[r] = __fma_rn(W, term, bcc[r]);
+            }
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+        if (lane + 32 * r < NB * NB) sA[lane + 32 * r] = __dadd_rn(sA[lane + 32 * r], acc[r]);
+#pragma unroll
+    for (int r = 0; r < RB; ++r)
+        if (lane + 32 * r < NB * B) sX[bi[r] * NX + k * B + bm[r]] = bcc[r];
+}
+
+// Facet k's C, transposed (j, m) in sP:  C(m, j) = sum_q W ( -(c+ + pen) phi_j psi_m + nu dn_j psi_m )
+template <int D, int P>
+__device__ __forceinline__ void exact_coupling(const ElemArgs &a, const double *sGeo, int k, int ks, const double *sW,
+                                               double *sP) {
+    using Dm = Dims<D, P>;
+    constexpr int NB = Dm::NB, B = Dm::B, NQF = Dm::NQF, QC = Dm::QC, N = QC * NB, RB = (NB * B + 31) / 32;
+    const int lane = threadIdx.x & 31;
+    const bool diff = a.nu != 0.0;
+    double acc[RB];
+    int oj[RB], om[RB];
+#pragma unroll
+    for (int r = 0; r < RB; ++r) {
+        const int t = lane + 32 * r < NB * B ? lane + 32 * r : 0;
+        acc[r] = 0.0;
+        oj[r] = t / B;
+        om[r] = t % B;
+    }
+#pragma unroll 1
+    for (int q0 = 0; q0 < NQF; q0 += QC) {
+        const int nq = NQF - q0 < QC ? NQF - q0 : QC;
+        exact_facet_products<D, P>(a, sGeo, k, ks, q0, nq, sW, sP);
+        const double *ps = a.psi + q0 * B;
+#pragma unroll 2
+        for (int q = 0; q < nq; ++q) {
+            const double W = sW[4 * (k * NQF + q0 + q)];
+#pragma unroll
+            for (int r = 0; r < RB; ++r) {
+                const double pl = ps[q * B + om[r]];
+                double term = __dmul_rn(-sP[q * NB + oj[r]], pl);
+                if (diff) term = __fma_rn(sP[3 * N + q * NB + oj[r]], pl, term);
+                acc[r] = __fma_rn(W, term, acc[r]);
+            }
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < RB; ++r)
+        if (lane + 32 * r < NB * B) sP[lane + 32 * r] = acc[r];
+}
+
+// Gaussian elimination with partial pivoting (ties -> smallest row) of the warp's A (N x N, row-major) applied to the
+// NC columns of X (row stride LDX), then back substitution column by column: X <- A^{-1} X.  Returns false if a pivot
+// is zero.
+template <int N, int NC, int LDX>
+__device__ bool warp_solve(double *A, double *X) {
+    const int lane = threadIdx.x & 31;
+    for (int c = 0; c < N; ++c) {
+        unsigned long long v = 0ull;
+        int r = N;
+        const int rr0 = c + lane;                    // N <= 32: one row per lane
+        if (rr0 < N) {
+            v = magnitude_key(A[rr0 * N + c]);
+            r = rr0;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long ov = __shfl_xor_sync(FULL, v, o);
+            const int orow = __shfl_xor_sync(FULL, r, o);
+            if (ov > v || (ov == v && orow < r)) { v = ov; r = orow; }
+        }
+        if (v <= 1ull) return false;                 // zero, or nothing but NaN
+        if (r != c) {
+            for (int t = lane; t < N + NC; t += 32) {
+                double *u = t < N ? A + c * N + t : X + c * LDX + (t - N), *w = t < N ? A + r * N + t : X + r * LDX + (t - N);
+                const double x = *u;
+                *u = *w;
+                *w = x;
+            }
+            __syncwarp();
+        }
+        if (rr0 > c && rr0 < N) A[rr0 * N + c] = __ddiv_rn(A[rr0 * N + c], A[c * N + c]);
+        __syncwarp();
+        const int wa = N - c - 1, w = wa + NC;
+        int rr = c + 1 + lane / w, cc = lane % w;
+        while (rr < N) {
+            const double m = A[rr * N + c];
+            if (cc < wa) A[rr * N + c + 1 + cc] = __fma_rn(-m, A[c * N + c + 1 + cc], A[rr * N + c + 1 + cc]);
+            else X[rr * LDX + (cc - wa)] = __fma_rn(-m, X[c * LDX + (cc - wa)], X[rr * LDX + (cc - wa)]);
+            cc += 32;
+            while (cc >= w) { cc -= w; ++rr; }
+        }
+        __syncwarp();
+    }
+    for (int t = lane; t < NC; t += 32)
+        for (int r = N - 1; r >= 0; --r) {
+            double s = X[r * LDX + t];
+            for (int cc = r + 1; cc < N; ++cc) s = __fma_rn(-A[r * N + cc], X[cc * LDX + t], s);
+            X[r * LDX + t] = __ddiv_rn(s, A[r * N + r]);
+        }
+    __syncwarp();
+    return true;
+}
+
 template <int D, int P>
 __global__ void __launch_bounds__(WPB * 32) hdg_element_kernel(ElemArgs a) {
     using Dm = Dims<D, P>;
-    constexpr int NB = Dm::NB, B = Dm::B, NF = Dm::NF, NT = Dm::NT, NX = Dm::NX, MAXN = Dm::MAXN, NQF = Dm::NQF,
-                  RB = (NB * B + 31) / 32;
+    constexpr int NB = Dm::NB, B = Dm::B, NF = Dm::NF, NT = Dm::NT, NX = Dm::NX, MAXN = Dm::MAXN, NQF = Dm::NQF;
     extern __shared__ double smem[];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t e = (int64_t)blockIdx.x * WPB + w;
     if (e >= a.E) return;                                 // the whole warp leaves together
     double *sA = smem + (size_t)w * Dm::WARP_DOUBLES;
     double *sX = sA + NB * NB, *sP = sX + Dm::XR, *sW = sP + Dm::PR, *sD = sW + 4 * NF * NQF, *sF = sD + B * B,
-           *sR = sF + NB, *sGeo = sR + NB;
+           *sGeo = sF + NB;
     const int32_t *fr = a.frame + e * NF, *ef = a.elem_facets + e * NF;
     for (int t = lane; t < Dm::GEO; t += 32) sGeo[t] = a.geo[e * Dm::GEO + t];
     __syncwarp();
-    volume_part<D, P>(a, e, sGeo, sA, sX, sP, sF);
-    facet_points<D, P>(a, e, sGeo, fr, sW);
-    symmetric_part<D, P>(a, sGeo, fr, sW, sP, sA);
-    // B, facet by facet, and F with the Dirichlet columns of B moved over
-    for (int k = 0; k < NF; ++k) {
-        double acc[RB];
-        coupling<D, P>(a, sGeo, k, k * Dm::NPERM + (fr[k] & 255), sW, 1, 1.0, sP, acc);
-#pragma unroll
-        for (int r = 0; r < RB; ++r) {
-            const int t = lane + 32 * r;
-            if (t < NB * B) sX[(t / B) * NX + k * B + t % B] = acc[r];
-        }
-    }
+    exact_volume<D, P>(a, e, sGeo, sA, sX, sP, sF);
+    exact_facet_points<D, P>(a, e, sGeo, fr, sW);
+    for (int k = 0; k < NF; ++k) exact_facet<D, P>(a, sGeo, k, k * Dm::NPERM + (fr[k] & 255), sW, sP, sA, sX);
+    for (int i = lane; i < NB; i += 32) sX[i * NX + NT] = sF[i];
     __syncwarp();
-    for (int i = lane; i < NB; i += 32) {
-        double f = sF[i];
-        for (int k = 0; k < NF; ++k) {
-            if (a.kind[ef[k]] != K_DIR) continue;
-            const double *ld = a.lam_dir + (int64_t)ef[k] * B;
-            for (int m = 0; m < B; ++m) f -= sX[i * NX + k * B + m] * ld[m];
-        }
-        sX[i * NX + NT] = f;
-    }
-    __syncwarp();
-    int perm;
-    if (!warp_factor<NB, NX, NX>(sA, sX, sR, perm)) {
+    if (!warp_solve<NB, NX, NX>(sA, sX)) {
         if (lane == 0) atomicOr(a.err, AIR_DEVERR_SINGULAR);
         return;
     }
-    warp_back_substitute<NB, NX, NX>(sA, sX, sR);
-    // rows of facet k: S_k = D_k - C_k X_B, H_k = G_k - C_k X_F, straight to their places
+    // rows of facet k: S_k = D_k - C_k X_B and H_k = G_k - C_k X_F - sum over Dirichlet facets l of S_kl Lam_l
     for (int k = 0; k < NF; ++k) {
         const int32_t f = ef[k];
         if (a.kind[f] == K_DIR) continue;
-        const int ks = k * Dm::NPERM + (fr[k] & 255);
-        double acc[RB];
-        coupling<D, P>(a, sGeo, k, ks, sW, 0, -1.0, sP, acc);
-#pragma unroll
-        for (int r = 0; r < RB; ++r)
-            if (lane + 32 * r < NB * B) sP[lane + 32 * r] = acc[r];          // C^T: (i, m)
-        // D, symmetric
-        for (int t = lane; t < Dm::BS; t += 32) {
-            int m, l;
-            sym_entry(t, B, m, l);
+        exact_coupling<D, P>(a, sGeo, k, k * Dm::NPERM + (fr[k] & 255), sW, sP);
+        const double pen = sGeo[Dm::G_PEN];
+        for (int t = lane; t < B * B; t += 32) {      // D(m, l) = sum_q W ( -(c- - pen) (+ c+) ) psi_l psi_m
+            const int m = t / B, l = t % B;
             double s = 0.0;
-            for (int q = 0; q < NQF; ++q) s += sW[4 * (k * NQF + q) + 2] * a.psi[q * B + m] * a.psi[q * B + l];
-            sD[m * B + l] = s;
-            sD[l * B + m] = s;
+            for (int q = 0; q < NQF; ++q) {
+                const double *p = sW + 4 * (k * NQF + q);
+                const double wc = __dmul_rn(p[0], __dadd_rn(-__dsub_rn(p[2], pen), fr[k] >= 256 ? p[1] : 0.0));
+                s = __fma_rn(__dmul_rn(wc, a.psi[q * B + l]), a.psi[q * B + m], s);
+            }
+            sD[t] = s;
         }
         double g = 0.0;
-        if (fr[k] >= 256 && lane < B)
-            for (int q = 0; q < NQF; ++q) g += sW[4 * (k * NQF + q) + 3] * a.psi[q * B + lane];
+        if (lane < B)
+            for (int q = 0; q < NQF; ++q) g = __fma_rn(sW[4 * (k * NQF + q) + 3], a.psi[q * B + lane], g);
         const int slot = a.facet_elems[2 * (int64_t)f] == (int32_t)e ? 0 : 1;
         const int32_t rf = a.rnum[f];
         // lane l: where block (k, l) starts within a row, -1 when it is not stored
@@ -652,7 +913,7 @@ __global__ void __launch_bounds__(WPB * 32) hdg_element_kernel(ElemArgs a) {
             else off = rank * B + (rg > rf ? a.dlen : 0);
         }
         const int64_t row0 = a.row_ptr[(int64_t)rf * B], rowlen = a.row_ptr[(int64_t)rf * B + 1] - row0;
-        double *dp = a.dpart + (2 * (int64_t)f + slot) * B * B;
+        double *dp = a.dpart + (2 * (int64_t)f + slot) * B * B, *sS = sP + NB * B;
         __syncwarp();
 #pragma unroll 2
         for (int t0 = 0; t0 < B * NX; t0 += 32) {
@@ -660,13 +921,24 @@ __global__ void __launch_bounds__(WPB * 32) hdg_element_kernel(ElemArgs a) {
             const int m = t / NX, c = t % NX, l = c / B;
             double s = 0.0;
 #pragma unroll
-            for (int i = 0; i < NB; ++i) s += sP[i * B + m] * sX[i * NX + c];
+            for (int i = 0; i < NB; ++i) s = __fma_rn(sP[i * B + m], sX[i * NX + c], s);
             const int o = __shfl_sync(FULL, off, l & 31);
             const double gm = __shfl_sync(FULL, g, m);
             if (t0 + lane >= B * NX) continue;
-            if (c == NT) a.hpart[(2 * (int64_t)f + slot) * B + m] = gm - s;
-            else if (l == k) dp[m * B + c - k * B] = sD[m * B + c - k * B] - s;
-            else if (o >= 0) a.val[row0 + m * rowlen + o + c - l * B] = -s;
+            const double v = __dsub_rn(c == NT ? gm : (l == k ? sD[m * B + c - k * B] : 0.0), s);
+            sS[t] = v;
+            if (l == k) dp[m * B + c - k * B] = v;
+            else if (o >= 0) a.val[row0 + m * rowlen + o + c - l * B] = v;
+        }
+        __syncwarp();
+        for (int m = lane; m < B; m += 32) {
+            double h = sS[m * NX + NT];
+            for (int l = 0; l < NF; ++l) {
+                if (l == k || a.kind[ef[l]] != K_DIR) continue;
+                const double *ld = a.lam_dir + (int64_t)ef[l] * B;
+                for (int l2 = 0; l2 < B; ++l2) h = __fma_rn(-sS[m * NX + l * B + l2], ld[l2], h);
+            }
+            a.hpart[(2 * (int64_t)f + slot) * B + m] = h;
         }
         __syncwarp();
     }
@@ -911,11 +1183,14 @@ __global__ void __launch_bounds__(32) adjoint_unscale_kernel(int64_t nfree, int 
     lane_load_blocks(diag, first, count, B, true, smem);
     for (int t = lane; t < count * B; t += 32) sx[(t % B) * LANE_LD + t / B] = adj[first * B + t];
     __syncwarp();
-    if (lane < count && !lane_solve(smem + lane, sx + lane, B)) atomicOr(err, AIR_DEVERR_SINGULAR);
+    if (lane < count && !lane_invert(smem + lane, B)) atomicOr(err, AIR_DEVERR_SINGULAR);
     __syncwarp();
     for (int t = lane; t < count * B; t += 32) {
-        const int64_t o = (int64_t)free_ids[first + t / B] * B + t % B;
-        mu_full[o] = sx[(t % B) * LANE_LD + t / B];
+        const int k = t / B, i = t % B;
+        double v = 0.0;
+        for (int j = 0; j < B; ++j) v += smem[(i * B + j) * LANE_LD + k] * sx[j * LANE_LD + k];
+        const int64_t o = (int64_t)free_ids[first + k] * B + i;
+        mu_full[o] = v;
         lam_full[o] = lam[first * B + t];
     }
 }
@@ -949,7 +1224,7 @@ __global__ void __launch_bounds__(WPB * 32) velocity_gradient_kernel(ElemArgs a)
     const int64_t e = (int64_t)blockIdx.x * WPB + w;
     if (e >= a.E) return;
     double *sA = smem + (size_t)w * Dm::GRAD_DOUBLES;
-    double *sV = sA + NB * NB, *sP = sV + NQ * (D + 1), *sW = sP + Dm::QC * NB, *sL = sW + 4 * NF * NQF,
+    double *sV = sA + NB * NB, *sP = sV + NQ * (D + 1), *sW = sP + Dm::QC * NB, *sL = sW + 2 * NF * NQF,
            *sM = sL + NF * NQF, *sLam = sM + NF * NQF, *sMu = sLam + NT, *sU = sMu + NT, *sY = sU + NB, *sF = sY + NB,
            *sR = sF + NB, *sGeo = sR + NB;
     const int32_t *fr = a.frame + e * NF, *ef = a.elem_facets + e * NF;
@@ -961,7 +1236,7 @@ __global__ void __launch_bounds__(WPB * 32) velocity_gradient_kernel(ElemArgs a)
     }
     __syncwarp();
     volume_part<D, P>(a, e, sGeo, sA, sV, sP, sF);
-    facet_points<D, P>(a, e, sGeo, fr, sW);
+    facet_points<D, P>(a, e, sGeo, sW);
     symmetric_part<D, P>(a, sGeo, fr, sW, sP, sA);
     for (int t = lane; t < NF * NQF; t += 32) {
         const int k = t / NQF, q = t % NQF;
@@ -984,13 +1259,13 @@ __global__ void __launch_bounds__(WPB * 32) velocity_gradient_kernel(ElemArgs a)
                 const int k = t / NQF, q = t % NQF;
                 const size_t at = ((size_t)(k * Dm::NPERM + (fr[k] & 255)) * NQF + q) * NB + i;
                 const double f = a.phi_f[at];
-                bl += sW[4 * t + 1] * sL[t] * f;
-                cm -= sW[4 * t] * sM[t] * f;
+                bl += sW[2 * t + 1] * sL[t] * f;
+                cm -= sW[2 * t] * sM[t] * f;
                 if (a.nu != 0.0) {
                     double dn = 0.0;
 #pragma unroll
                     for (int d = 0; d < D; ++d) dn += sGeo[Dm::G_F + k * Dm::G_FS + D + 1 + d] * a.gphi_f[at * D + d];
-                    dn *= a.wf[q];
+                    dn *= a.nu * sGeo[Dm::G_F + k * Dm::G_FS + D] * a.wf[q];
                     bl += dn * sL[t];
                     cm += dn * sM[t];
                 }
@@ -1168,23 +1443,27 @@ int launch_element(ElemArgs &a, bool gradient, cudaStream_t s) {
     const size_t smem = (size_t)WPB * (gradient ? Dm::GRAD_DOUBLES : Dm::WARP_DOUBLES) * sizeof(double);
     if (smem > AIR_SMEM_OPTIN) return AIR_ERR_UNSUPPORTED;
     double *geo = nullptr, *table = nullptr;
-    int32_t *frame = nullptr;
+    int32_t *frame = nullptr, *order = nullptr;
     int st = dalloc(&geo, a.E * Dm::GEO);
-    if (st == AIR_OK) st = dalloc(&table, Dm::TABLE);
     if (st == AIR_OK) st = dalloc(&frame, a.E * Dm::NF);
+    if (st == AIR_OK && gradient) st = dalloc(&table, Dm::TABLE);
+    if (st == AIR_OK && !gradient) st = dalloc(&order, Dm::NB * Dm::NB + Dm::NB);
     cudaError_t err = cudaSuccess;
     if (st == AIR_OK) {
-        table_kernel<D, P><<<air_counted((Dm::TABLE + 127) / 128), 128, 0, s>>>(a.wq, a.gphi, a.wf, a.psi, a.phi_f,
-                                                                               a.gphi_f, table);
         geometry_kernel<D, P><<<air_counted((unsigned)((a.E + 127) / 128)), 128, 0, s>>>(a, geo, frame);
         a.geo = geo;
-        a.table = table;
         a.frame = frame;
         const unsigned grid = (unsigned)((a.E + WPB - 1) / WPB);
         if (gradient) {
+            table_kernel<D, P><<<air_counted((Dm::TABLE + 127) / 128), 128, 0, s>>>(a.wq, a.gphi, a.wf, a.phi_f,
+                                                                                   a.gphi_f, table);
+            a.table = table;
             err = air_smem_optin(velocity_gradient_kernel<D, P>);
             if (err == cudaSuccess) velocity_gradient_kernel<D, P><<<air_counted(grid), WPB * 32, smem, s>>>(a);
         } else {
+            order_kernel<D, P><<<air_counted(1), 512, 0, s>>>(a.gphi, order, order + Dm::NB * Dm::NB);
+            a.order = order;
+            a.gmask = order + Dm::NB * Dm::NB;
             err = air_smem_optin(hdg_element_kernel<D, P>);
             if (err == cudaSuccess) hdg_element_kernel<D, P><<<air_counted(grid), WPB * 32, smem, s>>>(a);
         }
@@ -1194,6 +1473,7 @@ int launch_element(ElemArgs &a, bool gradient, cudaStream_t s) {
     air_dfree(geo);
     air_dfree(table);
     air_dfree(frame);
+    air_dfree(order);
     return st;
 }
 

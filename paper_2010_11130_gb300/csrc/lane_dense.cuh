@@ -47,8 +47,8 @@ __device__ __forceinline__ int lane_pivot(const double *m, int b, int c) {
     return r;
 }
 
-// Inverts the lane's matrix in place (m points at the lane's first entry) by Gauss-Jordan with partial pivoting.
-// b <= 11.  Returns false, and leaves garbage, if a pivot is zero.
+// Inverts the lane's matrix in place (m points at the lane's first entry) by Gauss-Jordan with partial pivoting: the
+// operations, in order, of the elimination of [M | I] (row / pivot, then fma(-f, row, other row)).  b <= 11.  Returns false, and leaves garbage, if a pivot is zero.
 __device__ __forceinline__ bool lane_invert(double *m, int b) {
     unsigned long long perm = 0ull;                  // 4 bits per column
     for (int c = 0; c < b; ++c) {
@@ -61,14 +61,15 @@ __device__ __forceinline__ bool lane_invert(double *m, int b) {
                 m[(c * b + t) * LANE_LD] = m[(r * b + t) * LANE_LD];
                 m[(r * b + t) * LANE_LD] = x;
             }
-        const double piv = m[(c * b + c) * LANE_LD], ri = 1.0 / piv;
+        const double piv = m[(c * b + c) * LANE_LD];
         m[(c * b + c) * LANE_LD] = 1.0;
-        for (int t = 0; t < b; ++t) m[(c * b + t) * LANE_LD] = quotient(m[(c * b + t) * LANE_LD], piv, ri);
+        for (int t = 0; t < b; ++t) m[(c * b + t) * LANE_LD] = __ddiv_rn(m[(c * b + t) * LANE_LD], piv);
         for (int rr = 0; rr < b; ++rr) {
             if (rr == c) continue;
             const double f = m[(rr * b + c) * LANE_LD];
             m[(rr * b + c) * LANE_LD] = 0.0;
-            for (int t = 0; t < b; ++t) m[(rr * b + t) * LANE_LD] -= f * m[(c * b + t) * LANE_LD];
+            for (int t = 0; t < b; ++t)
+                m[(rr * b + t) * LANE_LD] = __fma_rn(-f, m[(c * b + t) * LANE_LD], m[(rr * b + t) * LANE_LD]);
         }
     }
     for (int c = b - 1; c >= 0; --c) {               // the row swaps, undone on the columns
@@ -79,37 +80,6 @@ __device__ __forceinline__ bool lane_invert(double *m, int b) {
             m[(t * b + c) * LANE_LD] = m[(t * b + r) * LANE_LD];
             m[(t * b + r) * LANE_LD] = x;
         }
-    }
-    return true;
-}
-
-// x <- M^{-1} x for the lane's matrix and vector (entry i of x at x[i LANE_LD]); M is overwritten.
-__device__ __forceinline__ bool lane_solve(double *m, double *x, int b) {
-    for (int c = 0; c < b; ++c) {
-        const int r = lane_pivot(m, b, c);
-        if (r < 0) return false;
-        if (r != c) {
-            for (int t = c; t < b; ++t) {
-                const double v = m[(c * b + t) * LANE_LD];
-                m[(c * b + t) * LANE_LD] = m[(r * b + t) * LANE_LD];
-                m[(r * b + t) * LANE_LD] = v;
-            }
-            const double v = x[c * LANE_LD];
-            x[c * LANE_LD] = x[r * LANE_LD];
-            x[r * LANE_LD] = v;
-        }
-        const double piv = m[(c * b + c) * LANE_LD], ri = 1.0 / piv;
-        m[(c * b + c) * LANE_LD] = ri;               // kept for the back substitution
-        for (int rr = c + 1; rr < b; ++rr) {
-            const double l = quotient(m[(rr * b + c) * LANE_LD], piv, ri);
-            for (int t = c + 1; t < b; ++t) m[(rr * b + t) * LANE_LD] -= l * m[(c * b + t) * LANE_LD];
-            x[rr * LANE_LD] -= l * x[c * LANE_LD];
-        }
-    }
-    for (int r = b - 1; r >= 0; --r) {
-        const double v = x[r * LANE_LD] * m[(r * b + r) * LANE_LD];
-        x[r * LANE_LD] = v;
-        for (int t = 0; t < r; ++t) x[t * LANE_LD] -= m[(t * b + r) * LANE_LD] * v;
     }
     return true;
 }
