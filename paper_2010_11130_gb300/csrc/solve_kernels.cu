@@ -47,19 +47,18 @@ __device__ __forceinline__ A seg_sum(A s) {
     return s;
 }
 
-// Row kernels (SpMV and masked Jacobi).  VL lanes share a row; each lane
+// CSR SpMV.  VL lanes share a row; each lane
 // owns U entries of it, so all column / value loads of the row and then all
 // x gathers are in flight together (the short HDG rows are otherwise
 // latency-bound).  Entries beyond U*VL fall to a remainder loop.  The loop
 // runs over blocks of rows with a trip count that is uniform across the
 // warp, so every lane reaches the segment shuffles.
-// ROW_JACOBI writes a sweep's new values compactly (y[pos], scattered
-// afterwards); ROW_JACOBI_FULL writes them in place of the rows (y[row]) of a
-// second full vector, and the launch's extra blocks copy the rows the sweep
-// leaves unchanged (crows), so that the sweeps alternate between two vectors.
-enum { ROW_SPMV = 0, ROW_JACOBI = 1, ROW_JACOBI_FULL = 2 };
+// ROW_JACOBI writes the new values to the set's rows of a second full vector,
+// and the launch's extra blocks copy the rows the sweep leaves unchanged
+// (crows), so that the sweeps alternate between two vectors.
+enum { ROW_SPMV = 0, ROW_JACOBI = 1 };
 
-// Block blk of the copy part of a ROW_JACOBI_FULL launch.
+// Block blk of the copy part of a ROW_JACOBI launch.
 template <typename TX>
 __device__ __forceinline__ void copy_rows(int64_t mc, const int32_t *__restrict__ crows, const TX *__restrict__ x,
                                           TX *__restrict__ y, int64_t blk) {
@@ -78,14 +77,10 @@ struct RowArgs {
     const TV *v;
     const TX *x;        // input vector (gathered)
     TX *y;              // output
-    const TX *b;        // SpMV: optional (y = b - A x); Jacobi: right-hand side
-    const TX *dinv;     // Jacobi: 1 / a_ii
-    const int32_t *rows;  // Jacobi: the rows of the relaxed point set (ascending); n = their count
-    const TX *diag;       // if set, the stored values hold no diagonal: a_ii x_i is added from here
-    TX omega;
+    const TX *b;        // optional (y = b - A x)
 };
 
-template <int VL, int U, typename TV, typename TX, int MODE>
+template <int VL, int U, typename TV, typename TX>
 __global__ void __launch_bounds__(256) row_kernel(RowArgs<TV, TX> a) {
     using A = typename Acc<TX>::type;
     const int lane = threadIdx.x & (VL - 1);
@@ -93,10 +88,8 @@ __global__ void __launch_bounds__(256) row_kernel(RowArgs<TV, TX> a) {
     const int64_t ng = ((int64_t)gridDim.x * blockDim.x) / VL;
     const int64_t gw = g0 - (threadIdx.x & 31) / VL;            // first group of this warp
     for (int64_t base = gw; base < a.n; base += ng) {
-        const int64_t pos = base + (g0 - gw);
-        const bool valid = pos < a.n;
-        int64_t row = pos;
-        if (MODE == ROW_JACOBI && valid) row = a.rows[pos];
+        const int64_t row = base + (g0 - gw);
+        const bool valid = row < a.n;
         A acc = 0;
         if (valid) {
             const int64_t rs = a.rp[row], re = a.rp[row + 1];
@@ -113,25 +106,10 @@ __global__ void __launch_bounds__(256) row_kernel(RowArgs<TV, TX> a) {
             for (int u = 0; u < U; ++u) acc += to_acc<A, TV>(vals[u]) * (A)__ldg(a.x + cols[u]);
             for (int64_t e = rs + lane + (int64_t)U * VL; e < re; e += VL)
                 acc += to_acc<A, TV>(a.v[e]) * (A)a.x[a.ci[e]];
-            if (a.diag && lane == 0) acc += (A)a.diag[row] * (A)a.x[row];
         }
         acc = seg_sum<VL, A>(acc);
-        if (lane == 0 && valid) {
-            if (MODE == ROW_SPMV) {
-                a.y[row] = a.b ? (TX)((A)a.b[row] - acc) : (TX)acc;
-            } else {
-                // the new value goes to the compact buffer y[pos]; scatter_kernel writes it back
-                a.y[pos] = (TX)(a.x[row] + a.omega * ((TX)((A)a.b[row] - acc)) * a.dinv[row]);
-            }
-        }
+        if (lane == 0 && valid) a.y[row] = a.b ? (TX)((A)a.b[row] - acc) : (TX)acc;
     }
-}
-
-// x[rows[pos]] = t[pos]: finishes one Jacobi sweep in place.
-template <typename T>
-__global__ void scatter_kernel(int64_t m, const int32_t *__restrict__ rows, const T *__restrict__ t, T *__restrict__ x) {
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < m; p += (int64_t)gridDim.x * blockDim.x)
-        x[rows[p]] = t[p];
 }
 
 template <typename T>
@@ -264,12 +242,12 @@ struct SellArgs {
     const TV *v;
     const int32_t *rows;   // pos -> row id of the vectors
     const TX *x;
-    TX *y;                 // SpMV: y[row]; Jacobi: y[pos] (compact, scattered afterwards)
+    TX *y;
     const TX *b;
     const TX *dinv;
     const TX *diag;        // FP32 diagonal when the stored values hold none
     TX omega;
-    int64_t mc;            // ROW_JACOBI_FULL: rows copied unchanged from x to y, and the blocks before them
+    int64_t mc;            // ROW_JACOBI: rows copied unchanged from x to y, and the blocks before them
     const int32_t *crows;
     int64_t sweep_blocks;
 };
@@ -279,7 +257,7 @@ struct SellArgs {
 template <int UN, typename TV, typename TX, int MODE>
 __global__ void __launch_bounds__(256) sell_kernel(SellArgs<TV, TX> a) {
     using A = typename Acc<TX>::type;
-    if (MODE == ROW_JACOBI_FULL && (int64_t)blockIdx.x >= a.sweep_blocks) {
+    if (MODE == ROW_JACOBI && (int64_t)blockIdx.x >= a.sweep_blocks) {
         copy_rows(a.mc, a.crows, a.x, a.y, (int64_t)blockIdx.x - a.sweep_blocks);
         return;
     }
@@ -311,7 +289,7 @@ __global__ void __launch_bounds__(256) sell_kernel(SellArgs<TV, TX> a) {
     } else {
         if (a.diag) acc += (A)a.diag[row] * (A)a.x[row];
         const TX nv = (TX)(a.x[row] + a.omega * ((TX)((A)a.b[row] - acc)) * a.dinv[row]);
-        a.y[MODE == ROW_JACOBI ? pos : row] = nv;
+        a.y[row] = nv;
     }
 }
 
@@ -374,7 +352,7 @@ struct BSellArgs {
 template <int B, bool PAIRS, typename TV, typename TX, int MODE>
 __global__ void __launch_bounds__(256) bsell_kernel(BSellArgs<TV, TX> a) {
     using A = typename Acc<TX>::type;
-    if (MODE == ROW_JACOBI_FULL && (int64_t)blockIdx.x >= a.sweep_blocks) {
+    if (MODE == ROW_JACOBI && (int64_t)blockIdx.x >= a.sweep_blocks) {
         copy_rows(a.mc, a.crows, a.x, a.y, (int64_t)blockIdx.x - a.sweep_blocks);
         return;
     }
@@ -413,7 +391,7 @@ __global__ void __launch_bounds__(256) bsell_kernel(BSellArgs<TV, TX> a) {
         a.y[row] = a.b ? (TX)((A)a.b[row] - acc) : (TX)acc;
     } else {
         const TX nv = (TX)(a.x[row] + a.omega * ((TX)((A)a.b[row] - acc)) * a.dinv[row]);
-        a.y[MODE == ROW_JACOBI ? pos : row] = nv;
+        a.y[row] = nv;
     }
 }
 
@@ -421,7 +399,7 @@ template <int B, typename TV, typename TX, int MODE>
 void bsell_launch_b(const BSellArgs<TV, TX> &a0, bool pairs, cudaStream_t s) {
     BSellArgs<TV, TX> a = a0;
     a.sweep_blocks = (a.m + 255) / 256;
-    const unsigned g = (unsigned)(a.sweep_blocks + (MODE == ROW_JACOBI_FULL ? (a.mc + 255) / 256 : 0));
+    const unsigned g = (unsigned)(a.sweep_blocks + (MODE == ROW_JACOBI ? (a.mc + 255) / 256 : 0));
     if (pairs) bsell_kernel<B, true, TV, TX, MODE><<<air_counted(g), 256, 0, s>>>(a);
     else bsell_kernel<B, false, TV, TX, MODE><<<air_counted(g), 256, 0, s>>>(a);
 }
@@ -447,7 +425,7 @@ void bsell_launch(int b, const BSellArgs<TV, TX> &a, cudaStream_t s) {
 template <int VL, typename TV, typename TX, int MODE>
 __global__ void __launch_bounds__(256) sell_lanes_kernel(SellArgs<TV, TX> a) {
     using A = typename Acc<TX>::type;
-    if (MODE == ROW_JACOBI_FULL && (int64_t)blockIdx.x >= a.sweep_blocks) {   // whole blocks: no lane is left in a shuffle
+    if (MODE == ROW_JACOBI && (int64_t)blockIdx.x >= a.sweep_blocks) {   // whole blocks: no lane is left in a shuffle
         copy_rows(a.mc, a.crows, a.x, a.y, (int64_t)blockIdx.x - a.sweep_blocks);
         return;
     }
@@ -487,18 +465,18 @@ __global__ void __launch_bounds__(256) sell_lanes_kernel(SellArgs<TV, TX> a) {
     } else {
         if (a.diag) acc += (A)a.diag[row] * (A)a.x[row];
         const TX nv = (TX)(a.x[row] + a.omega * ((TX)((A)a.b[row] - acc)) * a.dinv[row]);
-        a.y[MODE == ROW_JACOBI ? pos : row] = nv;
+        a.y[row] = nv;
     }
 }
 
-// Blocks of the copy part of a ROW_JACOBI_FULL launch.
+// Blocks of the copy part of a ROW_JACOBI launch.
 inline int64_t copy_blocks(int64_t mc) { return (mc + 255) / 256; }
 
 template <int VL, typename TV, typename TX, int MODE>
 void sell_lanes_launch(const SellArgs<TV, TX> &a0, cudaStream_t s) {
     SellArgs<TV, TX> a = a0;
     a.sweep_blocks = (a.m * VL + 255) / 256;
-    const int64_t g = a.sweep_blocks + (MODE == ROW_JACOBI_FULL ? copy_blocks(a.mc) : 0);
+    const int64_t g = a.sweep_blocks + (MODE == ROW_JACOBI ? copy_blocks(a.mc) : 0);
     sell_lanes_kernel<VL, TV, TX, MODE><<<air_counted((unsigned)g), 256, 0, s>>>(a);
 }
 
@@ -515,7 +493,7 @@ void sell_launch(const SellArgs<TV, TX> &a, cudaStream_t s, int lanes = 1) {
     }
     SellArgs<TV, TX> b = a;
     b.sweep_blocks = (a.m + 255) / 256;
-    const int64_t g = b.sweep_blocks + (MODE == ROW_JACOBI_FULL ? copy_blocks(a.mc) : 0);
+    const int64_t g = b.sweep_blocks + (MODE == ROW_JACOBI ? copy_blocks(a.mc) : 0);
     sell_kernel<8, TV, TX, MODE><<<air_counted((unsigned)g), 256, 0, s>>>(b);
 }
 
@@ -697,26 +675,26 @@ __global__ void lincomb_kernel(int64_t n, double *out, const double *a, double c
     }
 }
 
-template <int U, typename TV, typename TX, int MODE>
+template <int U, typename TV, typename TX>
 void launch_row(const RowArgs<TV, TX> &a, cudaStream_t s) {
     unsigned g = grid_cap(a.n * 4, 256, 152 * 16);
-    row_kernel<4, U, TV, TX, MODE><<<air_counted(g), 256, 0, s>>>(a);
+    row_kernel<4, U, TV, TX><<<air_counted(g), 256, 0, s>>>(a);
 }
 
 // Entries per lane: enough for the longest row when rows are at most 64
 // long, else for the average row with the remainder loop taking the rest.
-template <typename TV, typename TX, int MODE>
+template <typename TV, typename TX>
 void row_dispatch(const RowArgs<TV, TX> &a, int64_t nnz, int32_t maxrow, cudaStream_t s) {
     double avg = a.n > 0 ? (double)nnz / (double)a.n : 0.0;
     int want = maxrow > 0 && maxrow <= 64 ? (maxrow + 3) / 4 : (int)((avg * 1.25 + 3.0) / 4.0);
-    if (want <= 1) launch_row<1, TV, TX, MODE>(a, s);
-    else if (want <= 2) launch_row<2, TV, TX, MODE>(a, s);
-    else if (want <= 4) launch_row<4, TV, TX, MODE>(a, s);
-    else if (want <= 6) launch_row<6, TV, TX, MODE>(a, s);
-    else if (want <= 8) launch_row<8, TV, TX, MODE>(a, s);
-    else if (want <= 10) launch_row<10, TV, TX, MODE>(a, s);
-    else if (want <= 12) launch_row<12, TV, TX, MODE>(a, s);
-    else launch_row<16, TV, TX, MODE>(a, s);
+    if (want <= 1) launch_row<1, TV, TX>(a, s);
+    else if (want <= 2) launch_row<2, TV, TX>(a, s);
+    else if (want <= 4) launch_row<4, TV, TX>(a, s);
+    else if (want <= 6) launch_row<6, TV, TX>(a, s);
+    else if (want <= 8) launch_row<8, TV, TX>(a, s);
+    else if (want <= 10) launch_row<10, TV, TX>(a, s);
+    else if (want <= 12) launch_row<12, TV, TX>(a, s);
+    else launch_row<16, TV, TX>(a, s);
 }
 
 template <typename TV, typename TX>
@@ -724,36 +702,14 @@ void spmv_dispatch(int64_t n, int64_t nnz, int32_t maxrow, const int64_t *rp, co
                    const TX *x, TX *y, const TX *b, cudaStream_t s) {
     RowArgs<TV, TX> a{};
     a.n = n; a.rp = rp; a.ci = ci; a.v = v; a.x = x; a.y = y; a.b = b;
-    row_dispatch<TV, TX, ROW_SPMV>(a, nnz, maxrow, s);
+    row_dispatch<TV, TX>(a, nnz, maxrow, s);
 }
 
-// One Jacobi sweep over the point set `which` (0 = F, 1 = C), in place on x:
-// new values of the set's rows go to tmp, then are scattered back.
-template <typename TV, typename T>
-void jacobi_dispatch(const AirLevel &L, const T *diag, const T *dinv, int which, T omega, const T *b, T *x, T *tmp,
-                     cudaStream_t s, bool scatter = true) {
-    const Sell &S = L.sset[which];
-    if (S.m == 0) return;
-    if (S.b > 0) {
-        BSellArgs<TV, T> ba{};
-        ba.m = S.m; ba.ptr = S.ptr; ba.bc = S.bc; ba.v = (const TV *)S.v; ba.dv = (const T *)S.dv; ba.rows = S.rows;
-        ba.x = x; ba.y = tmp; ba.b = b; ba.dinv = dinv; ba.omega = omega;
-        bsell_launch<TV, T, ROW_JACOBI>(S.b, ba, s);
-        if (scatter) scatter_kernel<T><<<air_counted(grid_cap(S.m, 256)), 256, 0, s>>>(S.m, S.rows, tmp, x);
-        return;
-    }
-    SellArgs<TV, T> a{};
-    a.m = S.m; a.ptr = S.ptr; a.ci = S.ci; a.v = (const TV *)S.v; a.rows = S.rows;
-    a.x = x; a.y = tmp; a.b = b; a.dinv = dinv; a.diag = diag; a.omega = omega;
-    sell_launch<TV, T, ROW_JACOBI>(a, s, L.lanes[which]);
-    if (scatter) scatter_kernel<T><<<air_counted(grid_cap(S.m, 256)), 256, 0, s>>>(S.m, S.rows, tmp, x);
-}
-
-// One Jacobi sweep over the point set `which` from x into the full vector y:
+// One Jacobi sweep over the point set `which` (0 = F, 1 = C) from x into the full vector y:
 // the set's rows get their new values, the other set's rows (when copy) their
 // values in x, in the same launch.
 template <typename TV, typename T>
-void jacobi_full_dispatch(const AirLevel &L, const T *diag, const T *dinv, int which, T omega, const T *b,
+void jacobi_dispatch(const AirLevel &L, const T *diag, const T *dinv, int which, T omega, const T *b,
                           const T *x, T *y, bool copy, cudaStream_t s) {
     const Sell &S = L.sset[which], &O = L.sset[1 - which];
     const int64_t mc = copy ? O.m : 0;
@@ -761,7 +717,7 @@ void jacobi_full_dispatch(const AirLevel &L, const T *diag, const T *dinv, int w
         if (mc > 0) {
             SellArgs<TV, T> a{};
             a.m = 0; a.x = x; a.y = y; a.mc = mc; a.crows = O.rows; a.sweep_blocks = 0;
-            sell_kernel<8, TV, T, ROW_JACOBI_FULL><<<air_counted((unsigned)copy_blocks(mc)), 256, 0, s>>>(a);
+            sell_kernel<8, TV, T, ROW_JACOBI><<<air_counted((unsigned)copy_blocks(mc)), 256, 0, s>>>(a);
         }
         return;
     }
@@ -769,28 +725,13 @@ void jacobi_full_dispatch(const AirLevel &L, const T *diag, const T *dinv, int w
         BSellArgs<TV, T> ba{};
         ba.m = S.m; ba.ptr = S.ptr; ba.bc = S.bc; ba.v = (const TV *)S.v; ba.dv = (const T *)S.dv; ba.rows = S.rows;
         ba.x = x; ba.y = y; ba.b = b; ba.dinv = dinv; ba.omega = omega; ba.mc = mc; ba.crows = O.rows;
-        bsell_launch<TV, T, ROW_JACOBI_FULL>(S.b, ba, s);
+        bsell_launch<TV, T, ROW_JACOBI>(S.b, ba, s);
         return;
     }
     SellArgs<TV, T> a{};
     a.m = S.m; a.ptr = S.ptr; a.ci = S.ci; a.v = (const TV *)S.v; a.rows = S.rows;
     a.x = x; a.y = y; a.b = b; a.dinv = dinv; a.diag = diag; a.omega = omega; a.mc = mc; a.crows = O.rows;
-    sell_launch<TV, T, ROW_JACOBI_FULL>(a, s, L.lanes[which]);
-}
-
-// One Jacobi sweep over all points: both point sets from the same old x into
-// the two halves of tmp, then both scatters.
-template <typename TV, typename T>
-void jacobi_all_dispatch(const AirLevel &L, const T *diag, const T *dinv, T omega, const T *b, T *x, T *tmp,
-                         cudaStream_t s) {
-    T *tf = tmp, *tc = tmp + L.sset[0].m;
-    jacobi_dispatch<TV, T>(L, diag, dinv, 0, omega, b, x, tf, s, false);
-    jacobi_dispatch<TV, T>(L, diag, dinv, 1, omega, b, x, tc, s, false);
-    for (int w = 0; w < 2; ++w) {
-        const Sell &S = L.sset[w];
-        if (S.m > 0)
-            scatter_kernel<T><<<air_counted(grid_cap(S.m, 256)), 256, 0, s>>>(S.m, S.rows, w == 0 ? tf : tc, x);
-    }
+    sell_launch<TV, T, ROW_JACOBI>(a, s, L.lanes[which]);
 }
 
 // The separate FP32 diagonal (BF16 storage only) and 1/a_ii in the vector
@@ -836,38 +777,23 @@ int vcycle_t(const air_hierarchy *H, const T *b0, T *x0, cudaStream_t s) {
         const T *xc = (const T *)H->lev[l + 1].x;
         const T *diag = (const T *)lvl_diag<TV>(A);
         const T *dinv = lvl_dinv<T>(A);
-        bool gs = false;
-        for (int q = 0; q < ns; ++q) gs = gs || relax[q] >= 'a';
-        if (!gs) {
-            // x = P x_c, then Jacobi sweeps alternating between out and alt,
-            // starting in whichever of the two makes the last sweep end in out
-            T *cur = ns % 2 == 1 ? alt : out, *nxt = ns % 2 == 1 ? out : alt;
-            interp_kernel<T><<<air_counted(grid_cap(A.n, 256)), 256, 0, s>>>(A.n, A.pcol, xc, cur);
-            for (int q = 0; q < ns; ++q) {
-                const char c = relax[q];
-                if (c == 'A') {
-                    jacobi_full_dispatch<TV, T>(A, diag, dinv, 0, omega, bl, cur, nxt, false, s);
-                    jacobi_full_dispatch<TV, T>(A, diag, dinv, 1, omega, bl, cur, nxt, false, s);
-                } else {
-                    jacobi_full_dispatch<TV, T>(A, diag, dinv, c == 'C' ? 1 : 0, omega, bl, cur, nxt, true, s);
-                }
-                T *t = cur;
-                cur = nxt;
-                nxt = t;
-            }
-            continue;
-        }
-        // x = P x_c, then the sweeps in place
-        interp_kernel<T><<<air_counted(grid_cap(A.n, 256)), 256, 0, s>>>(A.n, A.pcol, xc, out);
+        // x = P x_c, then the sweeps alternate between out and alt, starting in
+        // whichever of the two makes the last one end in out
+        T *cur = ns % 2 == 1 ? alt : out, *nxt = ns % 2 == 1 ? out : alt;
+        interp_kernel<T><<<air_counted(grid_cap(A.n, 256)), 256, 0, s>>>(A.n, A.pcol, xc, cur);
         for (int q = 0; q < ns; ++q) {
             const char c = relax[q];
-            if (c == 'F' || c == 'C') {
-                jacobi_dispatch<TV, T>(A, diag, dinv, c == 'C' ? 1 : 0, omega, bl, out, alt, s);
-            } else if (c == 'A') {
-                jacobi_all_dispatch<TV, T>(A, diag, dinv, omega, bl, out, alt, s);
+            if (c == 'A') {
+                jacobi_dispatch<TV, T>(A, diag, dinv, 0, omega, bl, cur, nxt, false, s);
+                jacobi_dispatch<TV, T>(A, diag, dinv, 1, omega, bl, cur, nxt, false, s);
+            } else if (c == 'F' || c == 'C') {
+                jacobi_dispatch<TV, T>(A, diag, dinv, c == 'C' ? 1 : 0, omega, bl, cur, nxt, true, s);
             } else {                                   // 'f', 'c', 'a': forward Gauss-Seidel
-                AIR_TRY(air_gs_sweep<T>(A, c == 'f' ? 0 : (c == 'c' ? 1 : 2), omega, bl, out, alt, s));
+                AIR_TRY(air_gs_sweep<T>(A, c == 'f' ? 0 : (c == 'c' ? 1 : 2), omega, bl, cur, nxt, H->d_err, s));
             }
+            T *t = cur;
+            cur = nxt;
+            nxt = t;
         }
     }
     AIR_LAUNCH();
@@ -1155,7 +1081,7 @@ int tune_set(const AirLevel &Lv, const Sell &S, const Sell *other, bool jacobi, 
         if (c > 1 && (avg / c < 1.0 || (S.m >= 2000000 && c > 2))) continue;
         for (int rep = 0; rep < 4; ++rep) {
             if (rep == 1) cudaEventRecord(e0, s);
-            if (jacobi) sell_launch<TV, T, ROW_JACOBI_FULL>(a, s, c);
+            if (jacobi) sell_launch<TV, T, ROW_JACOBI>(a, s, c);
             else sell_launch<TV, T, ROW_SPMV>(a, s, c);
         }
         cudaEventRecord(e1, s);
