@@ -400,12 +400,9 @@ int air_setup_end(air_hierarchy *H, cudaStream_t s) {
     PhaseTimer T(H, s);
     T.start(6);
     {
-        double *work = nullptr;
-        int64_t n = Lc.n;
+        const int64_t n = Lc.n;
         AIR_TRY(dalloc(&H->cinv, n * n));
-        AIR_CUDA(cudaMallocAsync((void **)&work, (size_t)(2 * n * n + n + 1) * sizeof(double), s));
-        AIR_TRY(air_coarse_inverse(n, Lc.rp, Lc.ci, Lc.v, H->cinv, work, H->d_err, s));
-        cudaFreeAsync(work, s);
+        AIR_TRY(air_coarse_inverse(n, Lc.rp, Lc.ci, Lc.v, H->cinv, H->d_err, s));
         AIR_TRY(check_err(H, s));
     }
     {

@@ -291,8 +291,10 @@ int air_onepoint_P(const AirLevel &L, double theta, cudaStream_t s);
 int air_rap(const AirLevel &L, int64_t *acrp, int32_t *acci, double *acv, int32_t *cnt, int fill,
             int32_t max_terms, const int32_t *terms, int *d_err, cudaStream_t s);
 int air_rap_terms(const AirLevel &L, int32_t *terms, cudaStream_t s);
-int air_coarse_inverse(int64_t n, const int64_t *rp, const int32_t *ci, const double *v, double *inv,
-                       double *work, int *d_err, cudaStream_t s);
+// coarse_inverse.cu: the dense inverse of a CSR matrix (AIR_DEVERR_SINGULAR in d_err: no pivot above 1e-14 of the
+// largest entry)
+int air_coarse_inverse(int64_t n, const int64_t *rp, const int32_t *ci, const double *v, double *inv, int *d_err,
+                       cudaStream_t s);
 
 // adjoint.cu
 int air_csr_transpose_impl(int64_t n, int64_t ncols, int64_t nnz, const int64_t *rp, const int32_t *ci,
