@@ -58,15 +58,45 @@ __device__ __forceinline__ A seg_sum(A s) {
 // (crows), so that the sweeps alternate between two vectors.
 enum { ROW_SPMV = 0, ROW_JACOBI = 1 };
 
-// Block blk of the copy part of a ROW_JACOBI launch.
+// The V-cycle's kernels are launched with programmatic dependence: a grid may
+// start while the one before it still runs, reads what no V-cycle writes (the
+// matrix, row lists, 1 / a_ii) and only then waits for it.  Between kernels of
+// a few microseconds that hides the launch and the first load latencies.  A
+// kernel reads vectors and writes only after dep_wait, which at least one thread
+// of every grid reaches, so the end of a grid also is the end of all before it.
+__device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename Args>
+void launch_dependent(void (*kernel)(Args), unsigned grid, const Args &a, cudaStream_t s) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = air_counted(grid);
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, a);
+}
+
+// Block blk of the copy part of a ROW_JACOBI launch: COPY_R rows per thread.
+constexpr int COPY_R = 4;
 template <typename TX>
-__device__ __forceinline__ void copy_rows(int64_t mc, const int32_t *__restrict__ crows, const TX *__restrict__ x,
-                                          TX *__restrict__ y, int64_t blk) {
-    const int64_t p = blk * blockDim.x + threadIdx.x;
-    if (p < mc) {
-        const int32_t r = crows[p];
-        y[r] = x[r];
-    }
+__device__ __forceinline__ void copy_rows(int64_t mc, const int32_t *crows, const TX *x, TX *y, int64_t blk) {
+    const int64_t p0 = blk * blockDim.x * COPY_R + threadIdx.x;
+    int32_t r[COPY_R];
+#pragma unroll
+    for (int u = 0; u < COPY_R; ++u) r[u] = p0 + u * blockDim.x < mc ? crows[p0 + u * blockDim.x] : -1;
+    dep_wait();
+    TX v[COPY_R];
+#pragma unroll
+    for (int u = 0; u < COPY_R; ++u)
+        if (r[u] >= 0) v[u] = x[r[u]];
+#pragma unroll
+    for (int u = 0; u < COPY_R; ++u)
+        if (r[u] >= 0) y[r[u]] = v[u];
 }
 
 template <typename TV, typename TX>
@@ -112,26 +142,64 @@ __global__ void __launch_bounds__(256) row_kernel(RowArgs<TV, TX> a) {
     }
 }
 
+constexpr int INTERP_R = 4;
 template <typename T>
-__global__ void interp_kernel(int64_t n, const int32_t *pcol, const T *xc, T *x) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        int32_t pc = pcol[i];
-        x[i] = pc >= 0 ? xc[pc] : (T)0;
-    }
+struct InterpArgs {
+    int64_t n;
+    const int32_t *pcol;
+    const T *xc;
+    T *x;
+};
+template <typename T>
+__global__ void __launch_bounds__(256) interp_kernel(InterpArgs<T> a) {
+    dep_launch();
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x * INTERP_R + threadIdx.x;
+    int32_t p[INTERP_R];
+#pragma unroll
+    for (int u = 0; u < INTERP_R; ++u) p[u] = i0 + u * blockDim.x < a.n ? a.pcol[i0 + u * blockDim.x] : -1;
+    dep_wait();
+    T v[INTERP_R];
+#pragma unroll
+    for (int u = 0; u < INTERP_R; ++u) v[u] = p[u] >= 0 ? a.xc[p[u]] : (T)0;
+#pragma unroll
+    for (int u = 0; u < INTERP_R; ++u)
+        if (i0 + u * blockDim.x < a.n) a.x[i0 + u * blockDim.x] = v[u];
 }
 
-// x = Cinv b, dense row-major, one warp per row
+// x = Cinv b, dense row-major, one warp per row; a lane's entries are loaded GEMV_U at a time, the first before the wait
+constexpr int GEMV_U = 16;
 template <typename T>
-__global__ void dense_gemv_kernel(int64_t n, const T *__restrict__ Ci, const T *__restrict__ b, T *__restrict__ x) {
-    int lane = threadIdx.x & 31;
-    int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t r = w; r < n; r += nw) {
-        T s = 0;
-        for (int64_t c = lane; c < n; c += 32) s += Ci[r * n + c] * b[c];
-        s = seg_sum<32, T>(s);
-        if (lane == 0) x[r] = s;
+struct GemvArgs {
+    int64_t n;
+    const T *Ci, *b;
+    T *x;
+};
+template <typename T>
+__global__ void __launch_bounds__(256) dense_gemv_kernel(GemvArgs<T> a) {
+    dep_launch();
+    const int lane = threadIdx.x & 31;
+    const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const bool valid = r < a.n;
+    const T *row = a.Ci + r * a.n;
+    T m[GEMV_U], s = 0;
+#pragma unroll
+    for (int u = 0; u < GEMV_U; ++u) m[u] = valid && lane + 32 * u < a.n ? row[lane + 32 * u] : (T)0;
+    dep_wait();
+    if (!valid) return;                              // a whole warp
+    for (int64_t c0 = lane; c0 < a.n; c0 += 32 * GEMV_U) {
+        T x[GEMV_U];
+#pragma unroll
+        for (int u = 0; u < GEMV_U; ++u) {
+            const int64_t c = c0 + 32 * u;
+            x[u] = c < a.n ? a.b[c] : (T)0;
+            if (c0 > lane) m[u] = c < a.n ? row[c] : (T)0;
+        }
+#pragma unroll
+        for (int u = 0; u < GEMV_U; ++u)
+            if (c0 + 32 * u < a.n) s += m[u] * x[u];
     }
+    s = seg_sum<32, T>(s);
+    if (lane == 0) a.x[r] = s;
 }
 
 __global__ void d2f_kernel(const double *in, float *out, int64_t n) {
@@ -252,43 +320,95 @@ struct SellArgs {
     int64_t sweep_blocks;
 };
 
-// One thread per row: entry k of the 32 rows of a slice is one coalesced
-// load; UN entries are loaded before their x gathers.
-template <int UN, typename TV, typename TX, int MODE>
+// VL lanes per row (VL divides 32): lane j of a row takes the row's stored
+// entries j, j + VL, ..., U at a time, then the lanes sum their partial
+// results; VL = 1 is one thread per row, entry k of a slice's rows one
+// coalesced load.  More lanes are for levels whose rows are long (Galerkin
+// fill) and few: the row's latency chain is VL times shorter.  The entries
+// past the last full batch are loaded together too, under predicates (full
+// batches under predicates cost 35% at 3.4 M rows).  U: with one or two lanes an
+// FP32 row has 17 to 40 entries per lane, and 12 in flight are best (V-cycle at
+// 7.9 M unknowns: 4 1403, 8 1349, 12 1313, 16 1377 us); with more lanes 8 hold
+// a row.
+template <int VL, int U, typename TV, typename TX, int MODE>
 __global__ void __launch_bounds__(256) sell_kernel(SellArgs<TV, TX> a) {
     using A = typename Acc<TX>::type;
-    if (MODE == ROW_JACOBI && (int64_t)blockIdx.x >= a.sweep_blocks) {
+    dep_launch();
+    if (MODE == ROW_JACOBI && (int64_t)blockIdx.x >= a.sweep_blocks) {   // whole blocks: no lane is left in a shuffle
         copy_rows(a.mc, a.crows, a.x, a.y, (int64_t)blockIdx.x - a.sweep_blocks);
         return;
     }
-    const int64_t pos = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (pos >= a.m) return;
-    const int64_t sl = pos >> 5;
-    const int l = (int)(pos & 31);
-    const int64_t base = a.ptr[sl];
-    const int w = (int)((a.ptr[sl + 1] - base) >> 5);
-    const int32_t *cp = a.ci + base + l;
-    const TV *vp = a.v + base + l;
-    A acc = 0;
-    int k = 0;
-    for (; k + UN <= w; k += UN) {
-        int32_t c[UN];
-        TV vv[UN];
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t pos = t / VL;
+    const int j = (int)(t % VL);
+    const bool valid = pos < a.m;                 // whole groups of VL lanes share validity
+    int w = 0;
+    int64_t row = 0;
+    TX di = 0;
+    const int32_t *cp = a.ci;
+    const TV *vp = a.v;
+    if (valid) {
+        const int64_t sl = pos >> 5;
+        const int64_t base = a.ptr[sl];
+        w = (int)((a.ptr[sl + 1] - base) >> 5);
+        cp += base + (pos & 31);
+        vp += base + (pos & 31);
+        row = a.rows[pos];
+        if (MODE == ROW_JACOBI) di = a.dinv[row];
+    }
+    int32_t c[U];
+    TV vv[U];
 #pragma unroll
-        for (int u = 0; u < UN; ++u) {
-            c[u] = __ldg(cp + 32 * (k + u));
-            vv[u] = vp[32 * (k + u)];
+    for (int u = 0; u < U; ++u) {
+        const int k = j + u * VL;
+        c[u] = k < w ? __ldg(cp + 32 * k) : 0;
+        vv[u] = k < w ? vp[32 * k] : (TV)0;
+    }
+    dep_wait();
+    TX bi = 0, xi = 0;
+    if (valid && j == 0) {
+        if (MODE == ROW_JACOBI) xi = a.x[row];
+        if (MODE == ROW_JACOBI || a.b) bi = a.b[row];
+    }
+    A acc = 0;
+    int k0 = j;
+    TX x[U];
+    for (; k0 + (U - 1) * VL < w; k0 += U * VL) {     // full batches
+        if (k0 > j) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                c[u] = __ldg(cp + 32 * (k0 + u * VL));
+                vv[u] = vp[32 * (k0 + u * VL)];
+            }
         }
 #pragma unroll
-        for (int u = 0; u < UN; ++u) acc += to_acc<A, TV>(vv[u]) * (A)__ldg(a.x + c[u]);
+        for (int u = 0; u < U; ++u) x[u] = a.x[c[u]];
+#pragma unroll
+        for (int u = 0; u < U; ++u) acc += to_acc<A, TV>(vv[u]) * (A)x[u];
     }
-    for (; k < w; ++k) acc += to_acc<A, TV>(vp[32 * k]) * (A)__ldg(a.x + cp[32 * k]);
-    const int64_t row = a.rows[pos];
+    if (k0 < w) {                                     // the rest, together
+        if (k0 > j) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int k = k0 + u * VL;
+                c[u] = k < w ? __ldg(cp + 32 * k) : 0;
+                vv[u] = k < w ? vp[32 * k] : (TV)0;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) x[u] = k0 + u * VL < w ? a.x[c[u]] : (TX)0;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (k0 + u * VL < w) acc += to_acc<A, TV>(vv[u]) * (A)x[u];
+    }
+#pragma unroll
+    for (int o = VL / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o, VL);
+    if (!valid || j != 0) return;
     if (MODE == ROW_SPMV) {
-        a.y[row] = a.b ? (TX)((A)a.b[row] - acc) : (TX)acc;
+        a.y[row] = a.b ? (TX)((A)bi - acc) : (TX)acc;
     } else {
-        if (a.diag) acc += (A)a.diag[row] * (A)a.x[row];
-        const TX nv = (TX)(a.x[row] + a.omega * ((TX)((A)a.b[row] - acc)) * a.dinv[row]);
+        if (a.diag) acc += (A)a.diag[row] * (A)xi;
+        const TX nv = (TX)(xi + a.omega * ((TX)((A)bi - acc)) * di);
         a.y[row] = nv;
     }
 }
@@ -318,14 +438,14 @@ __device__ __forceinline__ void pair_to<float, __nv_bfloat16>(const __nv_bfloat1
 }
 
 template <int B, bool PAIRS, typename A, typename T>
-__device__ __forceinline__ void load_run(const T *__restrict__ p, A (&out)[B]) {
+__device__ __forceinline__ void load_run(const T *p, A (&out)[B]) {
     if constexpr (PAIRS && B % 2 == 0) {
         const typename Pair<T>::type *q = reinterpret_cast<const typename Pair<T>::type *>(p);
 #pragma unroll
-        for (int j = 0; j < B / 2; ++j) pair_to<A, T>(__ldg(q + j), out[2 * j], out[2 * j + 1]);
+        for (int j = 0; j < B / 2; ++j) pair_to<A, T>(q[j], out[2 * j], out[2 * j + 1]);
     } else {
 #pragma unroll
-        for (int j = 0; j < B; ++j) out[j] = to_acc<A, T>(__ldg(p + j));
+        for (int j = 0; j < B; ++j) out[j] = to_acc<A, T>(p[j]);
     }
 }
 
@@ -347,11 +467,15 @@ struct BSellArgs {
     int64_t sweep_blocks;
 };
 
-// One thread per row: the row's blocks two at a time, each block's b values
-// and b entries of x as runs of consecutive elements.
+// One thread per row: the row's blocks G at a time, each block's b values and
+// b entries of x as runs of consecutive elements.  FP32 takes one block at a
+// time in 32 registers with every warp slot in use (V-cycle at 7.9 M unknowns
+// 1327 us, two blocks 1349, three 1364); FP64 two, its row product is bound by
+// FP64 issue.
 template <int B, bool PAIRS, typename TV, typename TX, int MODE>
 __global__ void __launch_bounds__(256) bsell_kernel(BSellArgs<TV, TX> a) {
     using A = typename Acc<TX>::type;
+    dep_launch();
     if (MODE == ROW_JACOBI && (int64_t)blockIdx.x >= a.sweep_blocks) {
         copy_rows(a.mc, a.crows, a.x, a.y, (int64_t)blockIdx.x - a.sweep_blocks);
         return;
@@ -363,45 +487,54 @@ __global__ void __launch_bounds__(256) bsell_kernel(BSellArgs<TV, TX> a) {
     const int64_t base = a.ptr[sl];
     const int w = (int)((a.ptr[sl + 1] - base) >> 5);
     const int64_t row = a.rows[pos];
-    A acc = (A)a.dv[pos] * (A)a.x[row];
+    const A d = (A)a.dv[pos];
+    const TX di = MODE == ROW_JACOBI ? a.dinv[row] : (TX)0;
+    dep_wait();
+    const TX xi = a.x[row];
+    const TX bi = MODE == ROW_JACOBI || a.b ? a.b[row] : (TX)0;
+    A acc = d * (A)xi;
+    constexpr int G = sizeof(TX) == 4 ? 1 : 2;
+    A v[G][B], x[G][B];
     int t = 0;
-    for (; t + 2 <= w; t += 2) {
-        const int64_t i0 = base + 32 * t + l, i1 = i0 + 32;
-        const int32_t c0 = __ldg(a.bc + i0), c1 = __ldg(a.bc + i1);
-        A v0[B], v1[B], x0[B], x1[B];
-        load_run<B, PAIRS>(a.v + i0 * B, v0);
-        load_run<B, PAIRS>(a.v + i1 * B, v1);
-        load_run<B, PAIRS>(a.x + c0, x0);
-        load_run<B, PAIRS>(a.x + c1, x1);
+    for (; t + G <= w; t += G) {
+        int32_t c[G];
 #pragma unroll
-        for (int j = 0; j < B; ++j) acc += v0[j] * x0[j];
+        for (int u = 0; u < G; ++u) {
+            const int64_t i = base + 32 * (t + u) + l;
+            c[u] = __ldg(a.bc + i);
+            load_run<B, PAIRS>(a.v + i * B, v[u]);
+        }
 #pragma unroll
-        for (int j = 0; j < B; ++j) acc += v1[j] * x1[j];
+        for (int u = 0; u < G; ++u) load_run<B, PAIRS>(a.x + c[u], x[u]);
+#pragma unroll
+        for (int u = 0; u < G; ++u)
+#pragma unroll
+            for (int j = 0; j < B; ++j) acc += v[u][j] * x[u][j];
     }
-    if (t < w) {
-        const int64_t i0 = base + 32 * t + l;
-        const int32_t c0 = __ldg(a.bc + i0);
-        A v0[B], x0[B];
-        load_run<B, PAIRS>(a.v + i0 * B, v0);
-        load_run<B, PAIRS>(a.x + c0, x0);
+    if (t < w) {                                      // G = 2: the last of an odd number
+        const int64_t i = base + 32 * t + l;
+        load_run<B, PAIRS>(a.v + i * B, v[0]);
+        load_run<B, PAIRS>(a.x + __ldg(a.bc + i), x[0]);
 #pragma unroll
-        for (int j = 0; j < B; ++j) acc += v0[j] * x0[j];
+        for (int j = 0; j < B; ++j) acc += v[0][j] * x[0][j];
     }
     if (MODE == ROW_SPMV) {
-        a.y[row] = a.b ? (TX)((A)a.b[row] - acc) : (TX)acc;
+        a.y[row] = a.b ? (TX)((A)bi - acc) : (TX)acc;
     } else {
-        const TX nv = (TX)(a.x[row] + a.omega * ((TX)((A)a.b[row] - acc)) * a.dinv[row]);
+        const TX nv = (TX)(xi + a.omega * ((TX)((A)bi - acc)) * di);
         a.y[row] = nv;
     }
 }
+
+// Blocks of the copy part of a ROW_JACOBI launch.
+inline int64_t copy_blocks(int64_t mc) { return (mc + 256 * COPY_R - 1) / (256 * COPY_R); }
 
 template <int B, typename TV, typename TX, int MODE>
 void bsell_launch_b(const BSellArgs<TV, TX> &a0, bool pairs, cudaStream_t s) {
     BSellArgs<TV, TX> a = a0;
     a.sweep_blocks = (a.m + 255) / 256;
-    const unsigned g = (unsigned)(a.sweep_blocks + (MODE == ROW_JACOBI ? (a.mc + 255) / 256 : 0));
-    if (pairs) bsell_kernel<B, true, TV, TX, MODE><<<air_counted(g), 256, 0, s>>>(a);
-    else bsell_kernel<B, false, TV, TX, MODE><<<air_counted(g), 256, 0, s>>>(a);
+    const unsigned g = (unsigned)(a.sweep_blocks + (MODE == ROW_JACOBI ? copy_blocks(a.mc) : 0));
+    launch_dependent(pairs ? bsell_kernel<B, true, TV, TX, MODE> : bsell_kernel<B, false, TV, TX, MODE>, g, a, s);
 }
 
 // pairs are safe when x starts on a pair boundary (the values always do)
@@ -418,83 +551,25 @@ void bsell_launch(int b, const BSellArgs<TV, TX> &a, cudaStream_t s) {
     }
 }
 
-// VL lanes per row (VL divides 32): lane j of a row takes the row's stored
-// entries j, j + VL, ..., four at a time, then the lanes sum their partial
-// results.  For levels whose rows are long (Galerkin fill) and few, the row's
-// latency chain is VL times shorter.
-template <int VL, typename TV, typename TX, int MODE>
-__global__ void __launch_bounds__(256) sell_lanes_kernel(SellArgs<TV, TX> a) {
-    using A = typename Acc<TX>::type;
-    if (MODE == ROW_JACOBI && (int64_t)blockIdx.x >= a.sweep_blocks) {   // whole blocks: no lane is left in a shuffle
-        copy_rows(a.mc, a.crows, a.x, a.y, (int64_t)blockIdx.x - a.sweep_blocks);
-        return;
-    }
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t pos = t / VL;
-    const int j = (int)(t % VL);
-    const bool valid = pos < a.m;                 // whole groups of VL lanes share validity
-    A acc = 0;
-    int64_t row = 0;
-    if (valid) {
-        const int64_t sl = pos >> 5;
-        const int l = (int)(pos & 31);
-        const int64_t base = a.ptr[sl];
-        const int w = (int)((a.ptr[sl + 1] - base) >> 5);
-        const int32_t *cp = a.ci + base + l;
-        const TV *vp = a.v + base + l;
-        int k = j;
-        for (; k + 3 * VL < w; k += 4 * VL) {
-            int32_t c[4];
-            TV vv[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                c[u] = __ldg(cp + 32 * (k + u * VL));
-                vv[u] = vp[32 * (k + u * VL)];
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) acc += to_acc<A, TV>(vv[u]) * (A)__ldg(a.x + c[u]);
-        }
-        for (; k < w; k += VL) acc += to_acc<A, TV>(vp[32 * k]) * (A)__ldg(a.x + cp[32 * k]);
-        row = a.rows[pos];
-    }
-#pragma unroll
-    for (int o = VL / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o, VL);
-    if (!valid || j != 0) return;
-    if (MODE == ROW_SPMV) {
-        a.y[row] = a.b ? (TX)((A)a.b[row] - acc) : (TX)acc;
-    } else {
-        if (a.diag) acc += (A)a.diag[row] * (A)a.x[row];
-        const TX nv = (TX)(a.x[row] + a.omega * ((TX)((A)a.b[row] - acc)) * a.dinv[row]);
-        a.y[row] = nv;
-    }
-}
-
-// Blocks of the copy part of a ROW_JACOBI launch.
-inline int64_t copy_blocks(int64_t mc) { return (mc + 255) / 256; }
-
 template <int VL, typename TV, typename TX, int MODE>
 void sell_lanes_launch(const SellArgs<TV, TX> &a0, cudaStream_t s) {
     SellArgs<TV, TX> a = a0;
     a.sweep_blocks = (a.m * VL + 255) / 256;
     const int64_t g = a.sweep_blocks + (MODE == ROW_JACOBI ? copy_blocks(a.mc) : 0);
-    sell_lanes_kernel<VL, TV, TX, MODE><<<air_counted((unsigned)g), 256, 0, s>>>(a);
+    launch_dependent(sell_kernel<VL, (VL <= 2 && sizeof(TX) == 4 ? 12 : 8), TV, TX, MODE>, (unsigned)g, a, s);
 }
 
 template <typename TV, typename TX, int MODE>
 void sell_launch(const SellArgs<TV, TX> &a, cudaStream_t s, int lanes = 1) {
-    if (a.m <= 0) return;
+    if (a.m <= 0 && !(MODE == ROW_JACOBI && a.mc > 0)) return;
     switch (lanes) {
     case 2: sell_lanes_launch<2, TV, TX, MODE>(a, s); return;
     case 4: sell_lanes_launch<4, TV, TX, MODE>(a, s); return;
     case 8: sell_lanes_launch<8, TV, TX, MODE>(a, s); return;
     case 16: sell_lanes_launch<16, TV, TX, MODE>(a, s); return;
     case 32: sell_lanes_launch<32, TV, TX, MODE>(a, s); return;
-    default: break;
+    default: sell_lanes_launch<1, TV, TX, MODE>(a, s); return;
     }
-    SellArgs<TV, TX> b = a;
-    b.sweep_blocks = (a.m + 255) / 256;
-    const int64_t g = b.sweep_blocks + (MODE == ROW_JACOBI ? copy_blocks(a.mc) : 0);
-    sell_kernel<8, TV, TX, MODE><<<air_counted((unsigned)g), 256, 0, s>>>(b);
 }
 
 __global__ void f2d_kernel(const float *in, double *out, int64_t n) {
@@ -713,14 +788,6 @@ void jacobi_dispatch(const AirLevel &L, const T *diag, const T *dinv, int which,
                           const T *x, T *y, bool copy, cudaStream_t s) {
     const Sell &S = L.sset[which], &O = L.sset[1 - which];
     const int64_t mc = copy ? O.m : 0;
-    if (S.m == 0) {
-        if (mc > 0) {
-            SellArgs<TV, T> a{};
-            a.m = 0; a.x = x; a.y = y; a.mc = mc; a.crows = O.rows; a.sweep_blocks = 0;
-            sell_kernel<8, TV, T, ROW_JACOBI><<<air_counted((unsigned)copy_blocks(mc)), 256, 0, s>>>(a);
-        }
-        return;
-    }
     if (S.b > 0) {
         BSellArgs<TV, T> ba{};
         ba.m = S.m; ba.ptr = S.ptr; ba.bc = S.bc; ba.v = (const TV *)S.v; ba.dv = (const T *)S.dv; ba.rows = S.rows;
@@ -765,8 +832,7 @@ int vcycle_t(const air_hierarchy *H, const T *b0, T *x0, cudaStream_t s) {
         const T *bl = L == 1 ? b0 : (const T *)C.b;
         T *xl = L == 1 ? x0 : (T *)C.x;
         const T *Ci = std::is_same<T, double>::value ? (const T *)H->cinv : (const T *)H->cinv32;
-        unsigned g = grid_cap(C.n * 32, 256, 152 * 8);
-        dense_gemv_kernel<T><<<air_counted(g), 256, 0, s>>>(C.n, Ci, bl, xl);
+        launch_dependent(dense_gemv_kernel<T>, (unsigned)((C.n + 7) / 8), GemvArgs<T>{C.n, Ci, bl, xl}, s);
     }
     // interpolation and relaxation back up
     for (int l = L - 2; l >= 0; --l) {
@@ -780,7 +846,8 @@ int vcycle_t(const air_hierarchy *H, const T *b0, T *x0, cudaStream_t s) {
         // x = P x_c, then the sweeps alternate between out and alt, starting in
         // whichever of the two makes the last one end in out
         T *cur = ns % 2 == 1 ? alt : out, *nxt = ns % 2 == 1 ? out : alt;
-        interp_kernel<T><<<air_counted(grid_cap(A.n, 256)), 256, 0, s>>>(A.n, A.pcol, xc, cur);
+        launch_dependent(interp_kernel<T>, (unsigned)((A.n + 256 * INTERP_R - 1) / (256 * INTERP_R)),
+                         InterpArgs<T>{A.n, A.pcol, xc, cur}, s);
         for (int q = 0; q < ns; ++q) {
             const char c = relax[q];
             if (c == 'A') {
