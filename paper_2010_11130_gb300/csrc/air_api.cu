@@ -615,9 +615,9 @@ int air_gmres_step(AirGmres &g) {
     AIR_TRY(air_sell_spmv_f64(H->a0, zj, w, nullptr, g.s));
     AIR_TRY(air_dot_partials(n, H->V, n, j + 1, w, H->partials, nblk, g.s));
     AIR_TRY(air_reduce_partials(j + 1, H->partials, nblk, h1, g.s));
-    AIR_TRY(air_update_dot_partials(n, H->V, n, j + 1, h1, w, H->partials, nblk, j + 1, g.s));
+    AIR_TRY(air_update_dot_partials(n, H->V, n, j + 1, h1, w, H->partials, nblk, true, g.s));
     AIR_TRY(air_reduce_partials(j + 1, H->partials, nblk, h2, g.s));
-    AIR_TRY(air_update_dot_partials(n, H->V, n, j + 1, h2, w, H->partials, nblk, -1, g.s));
+    AIR_TRY(air_update_dot_partials(n, H->V, n, j + 1, h2, w, H->partials, nblk, false, g.s));
     AIR_TRY(air_reduce_partials(1, H->partials, nblk, sc + 4, g.s));
     AIR_TRY(air_arnoldi_givens(j, m, h1, h2, sc + 4, H->Hm, H->cs, H->sn, H->gvec, sc, g.bnorm, g.s));
     AIR_TRY(air_scale_vec(n, w, w, sc + 2, 0, g.s));

@@ -355,7 +355,7 @@ int air_diag_inverse(int64_t n, const int64_t *rp, const int32_t *ci, const doub
 int air_dot_partials(int64_t n, const double *V, int64_t ldv, int k, const double *w, double *partials,
                      int nblk, cudaStream_t s);
 int air_update_dot_partials(int64_t n, const double *V, int64_t ldv, int k, const double *h, double *w,
-                            double *partials, int nblk, int dots, cudaStream_t s);
+                            double *partials, int nblk, bool dots, cudaStream_t s);
 int air_reduce_partials(int k, const double *partials, int nblk, double *out, cudaStream_t s);
 int air_scale_vec(int64_t n, const double *in, double *out, const double *d_norm, int sqrt_of, cudaStream_t s);
 int air_arnoldi_givens(int j, int m, const double *h1, const double *h2, const double *nrm2, double *Hm,

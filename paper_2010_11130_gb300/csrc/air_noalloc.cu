@@ -145,9 +145,9 @@ extern "C" int air_gmres_solve_noalloc(const air_csr *A, const air_hierarchy *H,
             AIR_TRY(air_spmv_f64(n, A0.rp, A0.ci, A0.v, zj, wj, nullptr, s, A0.nnz, A0.maxrow));
             AIR_TRY(air_dot_partials(n, w.V, n, j + 1, wj, w.partials, nblk, s));
             AIR_TRY(air_reduce_partials(j + 1, w.partials, nblk, w.h1, s));
-            AIR_TRY(air_update_dot_partials(n, w.V, n, j + 1, w.h1, wj, w.partials, nblk, j + 1, s));
+            AIR_TRY(air_update_dot_partials(n, w.V, n, j + 1, w.h1, wj, w.partials, nblk, true, s));
             AIR_TRY(air_reduce_partials(j + 1, w.partials, nblk, w.h2, s));
-            AIR_TRY(air_update_dot_partials(n, w.V, n, j + 1, w.h2, wj, w.partials, nblk, -1, s));
+            AIR_TRY(air_update_dot_partials(n, w.V, n, j + 1, w.h2, wj, w.partials, nblk, false, s));
             AIR_TRY(air_reduce_partials(1, w.partials, nblk, w.sc + 4, s));
             AIR_TRY(air_arnoldi_givens(j, m, w.h1, w.h2, w.sc + 4, w.Hm, w.cs, w.sn, w.g, w.sc, bnorm, s));
             AIR_TRY(air_scale_vec(n, wj, wj, w.sc + 2, 0, s));

@@ -593,79 +593,132 @@ __global__ void diag_inverse_kernel(int64_t n, const int64_t *rp, const int32_t 
 constexpr int RT = 256;          // threads of the reduction kernels
 constexpr int MAXK = AIR_MAX_RESTART + 1;
 
-// partials[i * nblk + blk] = sum over this block's slice of V_i . w   (i < k)
-template <int KB>
-__global__ void __launch_bounds__(RT) dot_partials_kernel(int64_t n, const double *__restrict__ V, int64_t ldv,
-                                                          int k0, int k, const double *__restrict__ w,
-                                                          double *__restrict__ partials, int nblk) {
-    __shared__ double red[RT / 32][KB];
-    double acc[KB];
+// The dot kernels are compiled for every number of vectors: all loads of an
+// element then are in flight together (under a run-time bound each waited for
+// the one before it) and no FP64 instruction is spent on a vector that is not
+// there.  Bound: FP64 issue, two lanes per SM and clock (K multiply-adds per
+// element for the dots, 2 K for the update with dots), close to the HBM time of
+// the vectors.  4.6 M unknowns, 16 vectors: dots 133 us (388 with run-time
+// bounds), update with dots 245 us, update with norm 138 us.
+
+// Sums over the warp of x[0] .. x[K - 1], left in lane-dependent places: the lane returns the index whose sum it has in
+// x[0], or -1 for a place that pads an odd count (first: index of x[0], count: entries that are not padding).  The sums are those of a butterfly over lane distances 16, 8, 4, 2, 1, but every step adds only the half of the
+// values that the lane keeps: K + 4 additions instead of 5 K.
+template <int K>
+__device__ __forceinline__ int warp_sums(double (&x)[K], int o, int first, int count) {
+    const int lane = threadIdx.x & 31;
+    if constexpr (K == 1) {
+        for (; o > 0; o >>= 1) x[0] += __shfl_xor_sync(FULL, x[0], o);
+        return count > 0 ? first : -1;
+    } else {
+        constexpr int H = (K + 1) / 2;
+        const bool up = lane & o;
+        double y[H];
 #pragma unroll
-    for (int i = 0; i < KB; ++i) acc[i] = 0.0;
-    for (int64_t t = (int64_t)blockIdx.x * RT + threadIdx.x; t < n; t += (int64_t)gridDim.x * RT) {
-        double wt = w[t];
-#pragma unroll
-        for (int i = 0; i < KB; ++i)
-            if (k0 + i < k) acc[i] += V[(int64_t)(k0 + i) * ldv + t] * wt;
-    }
-    int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int i = 0; i < KB; ++i) {
-        double s = acc[i];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
-        if (lane == 0) red[wid][i] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x < KB && k0 + (int)threadIdx.x < k) {
-        double s = 0.0;
-        for (int q = 0; q < RT / 32; ++q) s += red[q][threadIdx.x];
-        partials[(int64_t)(k0 + threadIdx.x) * nblk + blockIdx.x] = s;
+        for (int i = 0; i < H; ++i) {
+            const double hi = i + H < K ? x[i + H < K ? i + H : 0] : 0.0;
+            const double keep = up ? hi : x[i], give = up ? x[i] : hi;
+            y[i] = keep + __shfl_xor_sync(FULL, give, o);
+        }
+        const int r = warp_sums<H>(y, o >> 1, up ? first + H : first, up ? count - H : (count < H ? count : H));
+        x[0] = y[0];
+        return r;
     }
 }
 
-// w -= sum_i h_i V_i (i < k); then partial dots of the updated w with V_i
-// (i < dots) or, if dots == -1, the partial squared norm of w into row 0.
-template <int KB>
-__global__ void __launch_bounds__(RT) update_dot_kernel(int64_t n, const double *__restrict__ V, int64_t ldv, int k,
-                                                        const double *__restrict__ h, double *__restrict__ w,
-                                                        double *__restrict__ partials, int nblk, int dots) {
-    __shared__ double red[RT / 32][KB];
-    __shared__ double hs[KB];
-    if (threadIdx.x < KB) hs[threadIdx.x] = (int)threadIdx.x < k ? h[threadIdx.x] : 0.0;
+// The block's sums of K per-thread values into partials[i nblk + block], i < K
+template <int K>
+__device__ __forceinline__ void block_sums(double (&acc)[K], double *partials, int nblk) {
+    __shared__ double red[RT / 32][K];
+    const int i = warp_sums<K>(acc, 16, 0, K);
+    if (i >= 0) red[threadIdx.x >> 5][i] = acc[0];    // several lanes may hold the same sum
     __syncthreads();
-    double acc[KB];
-#pragma unroll
-    for (int i = 0; i < KB; ++i) acc[i] = 0.0;
-    for (int64_t t = (int64_t)blockIdx.x * RT + threadIdx.x; t < n; t += (int64_t)gridDim.x * RT) {
-        double vt[KB];
-        double wt = w[t];
-#pragma unroll
-        for (int i = 0; i < KB; ++i) {
-            vt[i] = i < k ? V[(int64_t)i * ldv + t] : 0.0;
-            wt -= hs[i] * vt[i];
-        }
-        w[t] = wt;
-        if (dots < 0) {
-            acc[0] += wt * wt;
-        } else {
-#pragma unroll
-            for (int i = 0; i < KB; ++i) acc[i] += vt[i] * wt;
-        }
-    }
-    int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int nd = dots < 0 ? 1 : dots;
-#pragma unroll
-    for (int i = 0; i < KB; ++i) {
-        double s = acc[i];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
-        if (lane == 0) red[wid][i] = s;
-    }
-    __syncthreads();
-    if ((int)threadIdx.x < nd && (int)threadIdx.x < KB) {
+    if (threadIdx.x < K) {
         double s = 0.0;
         for (int q = 0; q < RT / 32; ++q) s += red[q][threadIdx.x];
         partials[(int64_t)threadIdx.x * nblk + blockIdx.x] = s;
     }
+}
+
+// partials[i * nblk + blk] = sum over this block's slice of V_i . w   (i < K)
+template <int K>
+__global__ void __launch_bounds__(RT) dot_partials_kernel(int64_t n, const double *__restrict__ V, int64_t ldv,
+                                                          const double *__restrict__ w,
+                                                          double *__restrict__ partials, int nblk) {
+    constexpr int T = K <= 2 ? 4 : (K <= 6 ? 2 : 1);   // elements in flight
+    const int64_t step = (int64_t)gridDim.x * RT;
+    double acc[K];
+#pragma unroll
+    for (int i = 0; i < K; ++i) acc[i] = 0.0;
+    int64_t t = (int64_t)blockIdx.x * RT + threadIdx.x;
+    for (; t + (T - 1) * step < n; t += T * step) {
+        double wt[T], vt[T][K];
+#pragma unroll
+        for (int u = 0; u < T; ++u) {
+            wt[u] = w[t + u * step];
+#pragma unroll
+            for (int i = 0; i < K; ++i) vt[u][i] = V[i * ldv + t + u * step];
+        }
+#pragma unroll
+        for (int u = 0; u < T; ++u)
+#pragma unroll
+            for (int i = 0; i < K; ++i) acc[i] += vt[u][i] * wt[u];
+    }
+    for (; t < n; t += step) {
+        const double wt = w[t];
+#pragma unroll
+        for (int i = 0; i < K; ++i) acc[i] += V[i * ldv + t] * wt;
+    }
+    block_sums<K>(acc, partials, nblk);
+}
+
+// w -= sum_i h_i V_i (i < K); then partial dots of the updated w with V_i (DOTS) or the partial squared norm of w.
+template <int K, bool DOTS>
+__global__ void __launch_bounds__(RT) update_dot_kernel(int64_t n, const double *V, int64_t ldv,
+                                                        const double *__restrict__ h, double *w,
+                                                        double *__restrict__ partials, int nblk) {
+    constexpr int KA = DOTS ? K : 1;
+    // Elements in flight.  The warp meets between the loads and the chain of dependent subtractions: where nothing else
+    // keeps the loaded values (no dots), the loads were issued one by one along that chain (29 vectors: 757 us, now
+    // 242 us).
+    constexpr int T = DOTS ? (K <= 8 ? 2 : 1) : 2;
+    __shared__ double hs[K];
+    if (threadIdx.x < K) hs[threadIdx.x] = h[threadIdx.x];
+    __syncthreads();
+    const int64_t step = (int64_t)gridDim.x * RT;
+    double acc[KA];
+#pragma unroll
+    for (int i = 0; i < KA; ++i) acc[i] = 0.0;
+    for (int64_t t0 = (int64_t)blockIdx.x * RT; t0 < n; t0 += T * step) {      // whole warps: they meet below
+        const int64_t t = t0 + threadIdx.x;
+        double vt[T][K], wt[T];
+        bool on[T];
+#pragma unroll
+        for (int u = 0; u < T; ++u) {
+            on[u] = t + u * step < n;
+            const int64_t at = on[u] ? t + u * step : 0;
+            wt[u] = w[at];
+#pragma unroll
+            for (int i = 0; i < K; ++i) vt[u][i] = V[i * ldv + at];
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < K; ++i)
+#pragma unroll
+            for (int u = 0; u < T; ++u) wt[u] -= hs[i] * vt[u][i];
+#pragma unroll
+        for (int u = 0; u < T; ++u) {
+            if (!on[u]) continue;
+            w[t + u * step] = wt[u];
+            if (DOTS) {
+#pragma unroll
+                for (int i = 0; i < KA; ++i) acc[i] += vt[u][i] * wt[u];
+            } else {
+                acc[0] += wt[u] * wt[u];
+            }
+        }
+    }
+    block_sums<KA>(acc, partials, nblk);
 }
 
 __global__ void reduce_partials_kernel(const double *partials, int nblk, double *out) {
@@ -1318,24 +1371,40 @@ int air_reduce_nblk(int64_t n) {
     return (int)b;
 }
 
+namespace {
+
+template <int K>
+void dot_launch(int k, int64_t n, const double *V, int64_t ldv, const double *w, double *partials, int nblk,
+                cudaStream_t s) {
+    if (k == K) dot_partials_kernel<K><<<air_counted(nblk), RT, 0, s>>>(n, V, ldv, w, partials, nblk);
+    else if constexpr (K > 1) dot_launch<K - 1>(k, n, V, ldv, w, partials, nblk, s);
+}
+
+template <int K>
+void update_launch(int k, bool dots, int64_t n, const double *V, int64_t ldv, const double *h, double *w,
+                   double *partials, int nblk, cudaStream_t s) {
+    if (k == K) {
+        if (dots) update_dot_kernel<K, true><<<air_counted(nblk), RT, 0, s>>>(n, V, ldv, h, w, partials, nblk);
+        else update_dot_kernel<K, false><<<air_counted(nblk), RT, 0, s>>>(n, V, ldv, h, w, partials, nblk);
+    } else if constexpr (K > 1) {
+        update_launch<K - 1>(k, dots, n, V, ldv, h, w, partials, nblk, s);
+    }
+}
+
+}  // namespace
+
 int air_dot_partials(int64_t n, const double *V, int64_t ldv, int k, const double *w, double *partials, int nblk,
                      cudaStream_t s) {
-    for (int k0 = 0; k0 < k; k0 += 16) {
-        if (k - k0 <= 4) dot_partials_kernel<4><<<air_counted(nblk), RT, 0, s>>>(n, V, ldv, k0, k, w, partials, nblk);
-        else if (k - k0 <= 8) dot_partials_kernel<8><<<air_counted(nblk), RT, 0, s>>>(n, V, ldv, k0, k, w, partials, nblk);
-        else dot_partials_kernel<16><<<air_counted(nblk), RT, 0, s>>>(n, V, ldv, k0, k, w, partials, nblk);
-    }
+    for (int k0 = 0; k0 < k; k0 += 16)
+        dot_launch<16>(k - k0 < 16 ? k - k0 : 16, n, V + (int64_t)k0 * ldv, ldv, w, partials + (int64_t)k0 * nblk, nblk, s);
     AIR_LAUNCH();
     return AIR_OK;
 }
 
 int air_update_dot_partials(int64_t n, const double *V, int64_t ldv, int k, const double *h, double *w,
-                            double *partials, int nblk, int dots, cudaStream_t s) {
-    if (k <= 4) update_dot_kernel<4><<<air_counted(nblk), RT, 0, s>>>(n, V, ldv, k, h, w, partials, nblk, dots);
-    else if (k <= 8) update_dot_kernel<8><<<air_counted(nblk), RT, 0, s>>>(n, V, ldv, k, h, w, partials, nblk, dots);
-    else if (k <= 16) update_dot_kernel<16><<<air_counted(nblk), RT, 0, s>>>(n, V, ldv, k, h, w, partials, nblk, dots);
-    else if (k <= 32) update_dot_kernel<32><<<air_counted(nblk), RT, 0, s>>>(n, V, ldv, k, h, w, partials, nblk, dots);
-    else return AIR_ERR_UNSUPPORTED;
+                            double *partials, int nblk, bool dots, cudaStream_t s) {
+    if (k < 1 || k > 32) return AIR_ERR_UNSUPPORTED;
+    update_launch<32>(k, dots, n, V, ldv, h, w, partials, nblk, s);
     AIR_LAUNCH();
     return AIR_OK;
 }
