@@ -2,7 +2,8 @@
 // settings, whose details the paper leaves to its library): the points are cut
 // into consecutive index blocks of `block` points; the first pass of
 // Ruge-Stueben runs in every block at once on the strength graph restricted to
-// the block, one warp per block with the block's measures in shared memory;
+// the block, one warp per block with the block's measures and graph in shared
+// memory;
 // then the interface points that ended F with strong connections but no
 // strong C point are fixed by rounds of a parallel independent set.
 //
@@ -15,7 +16,13 @@
 // point of the block in S_i loses one; stop when the largest measure is 0 (the
 // rest become F).  The maximum is found through two levels of upper bounds
 // (per 32 points and per 1024 points) that increments raise and searches
-// repair when they meet a stale one.
+// repair when they meet a stale one.  What bounds it is the chain of picks of
+// one block (a block of 8192 points has 2,000 to 3,600; blocks run side by
+// side): a pick is about a dozen dependent accesses, in shared memory 30 cycles
+// each, in the L2 300 to 600.  The block's graph, 16-bit local indices both ways,
+// is therefore gathered into shared memory first, and the strong connections of
+// four new F points are raised together.  All levels at 2.3 M unknowns: 17.5 ms
+// (40.8 ms with the graph in global memory and one F point after the other).
 //
 // Interface rounds: U = F points with S_i non-empty, no C point in S_i and a
 // strong connection (either way) to another block.  Weight
@@ -28,7 +35,7 @@
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
-constexpr int FWARPS = 4;            // blocks of points (warps) per CTA
+constexpr int LT = 256;              // threads per block of points: all gather its graph, one warp picks
 constexpr int NEWF_CAP = 1024;       // new F points of one pick
 constexpr int LAM_F = -1, LAM_C = -2;
 constexpr int8_t CF_F = 0, CF_C = 1;
@@ -39,12 +46,6 @@ __device__ __forceinline__ unsigned lanemask_lt() {
     return m;
 }
 
-__device__ __forceinline__ int warp_max_i(int v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(FULL, v, o));
-    return v;
-}
-
 unsigned grid_for(int64_t items, int threads) {
     int64_t b = (items + threads - 1) / threads;
     if (b < 1) b = 1;
@@ -52,95 +53,97 @@ unsigned grid_for(int64_t items, int threads) {
     return (unsigned)b;
 }
 
-// Shared memory of one warp: lam[block] (int32), g1[block / 32], g2[block / 1024], newF[NEWF_CAP].
-__global__ void __launch_bounds__(FWARPS * 32) local_pass_kernel(int64_t n, int64_t block, const int64_t *srp,
-                                                                 const int32_t *sci, const int64_t *strp,
-                                                                 const int32_t *stci, int8_t *cf, int *err) {
-    extern __shared__ int32_t fsm[];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t nblk = (n + block - 1) / block;
-    const int64_t b = (int64_t)blockIdx.x * FWARPS + w;
-    if (b >= nblk) return;
-    const int64_t lo = b * block, hi = lo + block < n ? lo + block : n;
-    const int m = (int)(hi - lo);
-    const int ng1 = (int)((block + 31) / 32), ng2 = (int)((block + 1023) / 1024);
-    int32_t *lam = fsm + (size_t)w * (block + ng1 + ng2 + NEWF_CAP);
-    int32_t *g1 = lam + block, *g2 = g1 + ng1, *newF = g2 + ng2;
-    // measures inside the block
-    for (int t = lane; t < (int)block; t += 32) {
-        int v = LAM_F;
-        if (t < m) {
-            const int64_t i = lo + t;
-            int cnt = 0, ns = 0;
-            for (int64_t a = strp[i]; a < strp[i + 1]; ++a) cnt += (stci[a] >= lo && stci[a] < hi);
-            for (int64_t a = srp[i]; a < srp[i + 1]; ++a) ns += (sci[a] >= lo && sci[a] < hi);
-            v = (cnt == 0 && ns == 0) ? LAM_F : cnt;
+// Shared memory of one block of points: lam[block], g1[block / 32], g2[block / 1024], newF[NEWF_CAP] (int32), then 16
+// bits each: row starts of S and of S^T (block + 1, padded to even), their entries (cap each).
+struct LocalGraph {
+    int64_t lo;                       // first point and number of points
+    int m;
+    const int64_t *srp, *strp;        // the whole graph, for blocks whose own part does not fit
+    const int32_t *sci, *stci;
+    const uint16_t *sp, *tp, *se, *te;
+};
+
+// Rows of S (T = false) or S^T of a local point, restricted to the block: entry numbers first .. last, at(e) the local
+// neighbour or -1 outside the block.
+template <bool SMEM, bool T>
+struct Row {
+    int64_t first, last;
+    __device__ __forceinline__ Row(const LocalGraph &g, int j) {
+        if (SMEM) {
+            const uint16_t *p = T ? g.tp : g.sp;
+            first = p[j];
+            last = p[j + 1];
+        } else {
+            const int64_t *p = T ? g.strp : g.srp;
+            first = p[g.lo + j];
+            last = p[g.lo + j + 1];
         }
-        lam[t] = v;
     }
-    __syncwarp();
-    for (int gidx = lane; gidx < ng1; gidx += 32) {
-        int mx = LAM_C;
-        for (int t = 0; t < 32; ++t) mx = max(mx, lam[gidx * 32 + t]);
-        g1[gidx] = mx;
+    __device__ __forceinline__ int at(const LocalGraph &g, int64_t e) const {
+        if (SMEM) return (T ? g.te : g.se)[e];
+        const int64_t k = (T ? g.stci : g.sci)[e] - g.lo;
+        return k >= 0 && k < g.m ? (int)k : -1;
     }
-    __syncwarp();
-    for (int h = lane; h < ng2; h += 32) {
-        int mx = LAM_C;
-        for (int t = 0; t < 32 && h * 32 + t < ng1; ++t) mx = max(mx, g1[h * 32 + t]);
-        g2[h] = mx;
-    }
-    __syncwarp();
-    const int64_t cap = 64 * (int64_t)m + 1024;  // picks plus repairs of stale bounds (a safety net)
+};
+
+// The picks of one block, by one warp.
+template <bool SMEM>
+__device__ void local_picks(const LocalGraph &g, int ng1, int ng2, int32_t *lam, int32_t *g1, int32_t *g2,
+                            int32_t *newF, int *err) {
+    const int lane = threadIdx.x & 31;
+    const int64_t cap = 64 * (int64_t)g.m + 1024;  // picks plus repairs of stale bounds (a safety net)
     for (int64_t step = 0;; ++step) {
         if (step > cap) {
             if (lane == 0) atomicOr(err, AIR_DEVERR_RS_CAP);
             break;
         }
-        // level 2: the largest bound and its first 1024-point range
-        int v2 = lane < ng2 ? g2[lane] : LAM_C;
-        for (int h = lane + 32; h < ng2; h += 32) v2 = max(v2, g2[h]);
-        const int top = warp_max_i(v2);
+        // level 2 (at most 8 ranges): the largest bound and its first 1024-point range
+        const int v2 = lane < ng2 ? g2[lane] : LAM_C;
+        const int top = __reduce_max_sync(FULL, v2);
         if (top < 1) break;
-        int h = -1;
-        for (int h0 = 0; h0 < ng2 && h < 0; h0 += 32) {
-            const unsigned bal = __ballot_sync(FULL, h0 + lane < ng2 && g2[h0 + lane] == top);
-            if (bal) h = h0 + __ffs(bal) - 1;
-        }
+        const int h = __ffs(__ballot_sync(FULL, v2 == top)) - 1;
         // level 1: the first 32-point group of that range with the bound
         const int gi = h * 32 + lane;
         const int b1 = gi < ng1 ? g1[gi] : LAM_C;
         const unsigned bal1 = __ballot_sync(FULL, b1 == top);
         if (!bal1) {                                   // stale range bound: repair it
-            const int mx = warp_max_i(b1);
+            const int mx = __reduce_max_sync(FULL, b1);
             if (lane == 0) g2[h] = mx;
             __syncwarp();
             continue;
         }
-        const int g = h * 32 + __ffs(bal1) - 1;
-        const int lv = lam[g * 32 + lane];
+        const int q1 = h * 32 + __ffs(bal1) - 1;
+        const int lv = lam[q1 * 32 + lane];
         const unsigned bal0 = __ballot_sync(FULL, lv == top);
         if (!bal0) {                                   // stale group bound: repair it
-            const int mx = warp_max_i(lv);
-            if (lane == 0) g1[g] = mx;
+            const int mx = __reduce_max_sync(FULL, lv);
+            if (lane == 0) g1[q1] = mx;
             __syncwarp();
             continue;
         }
-        const int li = g * 32 + __ffs(bal0) - 1;
-        const int64_t i = lo + li;
-        if (lane == 0) lam[li] = LAM_C;
+        const int i = q1 * 32 + __ffs(bal0) - 1;
+        const Row<SMEM, true> dep(g, i);
+        const Row<SMEM, false> own(g, i);
+        // i leaves its group and range: their exact bounds now cost less than meeting stale ones later
+        const int picked = __ffs(bal0) - 1;
+        const int m1 = __reduce_max_sync(FULL, lane == picked ? LAM_C : lv);
+        const int m2 = __reduce_max_sync(FULL, lane == (q1 & 31) ? m1 : b1);
+        if (lane == 0) {
+            lam[i] = LAM_C;
+            g1[q1] = m1;
+            g2[h] = m2;
+        }
         __syncwarp();
         // undecided strong dependants of i in the block become F
         int nf = 0;
-        for (int64_t a0 = strp[i]; a0 < strp[i + 1]; a0 += 32) {
-            const int64_t a = a0 + lane;
-            int32_t j = a < strp[i + 1] ? stci[a] : -1;
-            const bool f = j >= lo && j < hi && lam[j - lo] >= 0;
+        for (int64_t a0 = dep.first; a0 < dep.last; a0 += 32) {
+            const int j = a0 + lane < dep.last ? dep.at(g, a0 + lane) : -1;
+            const bool f = j >= 0 && lam[j] >= 0;
             const unsigned bal = __ballot_sync(FULL, f);
             if (f) {
                 const int p = nf + __popc(bal & lanemask_lt());
                 if (p < NEWF_CAP) newF[p] = j;
-                lam[j - lo] = LAM_F;
+                lam[j] = LAM_F;
             }
             nf += __popc(bal);
         }
@@ -149,28 +152,98 @@ __global__ void __launch_bounds__(FWARPS * 32) local_pass_kernel(int64_t n, int6
             break;
         }
         __syncwarp();
-        // every undecided point of the block in S_j of a new F point j gains one
-        for (int q = 0; q < nf; ++q) {
-            const int32_t j = newF[q];
-            for (int64_t a = srp[j] + lane; a < srp[j + 1]; a += 32) {
-                const int32_t k = sci[a];
-                if (k >= lo && k < hi && lam[k - lo] >= 0) {
-                    const int nv = atomicAdd(&lam[k - lo], 1) + 1;
-                    atomicMax(&g1[(k - lo) >> 5], nv);
-                    atomicMax(&g2[(k - lo) >> 10], nv);
+        // every undecided point of the block in S_j of a new F point j gains one: eight lanes per j
+        for (int q = lane >> 3; q < nf; q += 4) {
+            const Row<SMEM, false> r(g, newF[q]);
+            for (int64_t a = r.first + (lane & 7); a < r.last; a += 8) {
+                const int k = r.at(g, a);
+                if (k >= 0 && lam[k] >= 0) {
+                    const int nv = atomicAdd(&lam[k], 1) + 1;
+                    atomicMax(&g1[k >> 5], nv);
+                    atomicMax(&g2[k >> 10], nv);
                 }
             }
         }
-        __syncwarp();
-        // every undecided point of the block in S_i loses one (bounds stay upper bounds)
-        for (int64_t a = srp[i] + lane; a < srp[i + 1]; a += 32) {
-            const int32_t k = sci[a];
-            if (k >= lo && k < hi && lam[k - lo] >= 0) atomicSub(&lam[k - lo], 1);
+        // every undecided point of the block in S_i loses one (bounds stay upper bounds, also beside the gains)
+        for (int64_t a = own.first + lane; a < own.last; a += 32) {
+            const int k = own.at(g, a);
+            if (k >= 0 && lam[k] >= 0) atomicSub(&lam[k], 1);
         }
         __syncwarp();
     }
     __syncwarp();
-    for (int t = lane; t < m; t += 32) cf[lo + t] = lam[t] == LAM_C ? CF_C : CF_F;
+}
+
+__global__ void __launch_bounds__(LT) local_pass_kernel(int64_t n, int64_t block, int cap, const int64_t *srp,
+                                                        const int32_t *sci, const int64_t *strp, const int32_t *stci,
+                                                        int8_t *cf, int *err) {
+    extern __shared__ int32_t fsm[];
+    __shared__ int sum[2][LT];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int64_t lo = blockIdx.x * block, hi = lo + block < n ? lo + block : n;
+    const int m = (int)(hi - lo), ng1 = (int)(block / 32), ng2 = (int)(block / 1024), nb = (int)block;
+    int32_t *lam = fsm, *g1 = lam + block, *g2 = g1 + ng1, *newF = g2 + ng2;
+    uint16_t *sp = (uint16_t *)(newF + NEWF_CAP), *tp = sp + block + 2, *se = tp + block + 2, *te = se + cap;
+    // a thread's consecutive points: entries inside the block, counted, then gathered
+    const int per = nb / LT, t0 = tid * per;
+    int s_sum = 0, t_sum = 0;
+    for (int t = t0; t < t0 + per; ++t) {
+        int cnt = 0, ns = 0;
+        if (t < m) {
+            const int64_t i = lo + t;
+            for (int64_t a = strp[i]; a < strp[i + 1]; ++a) cnt += (stci[a] >= lo && stci[a] < hi);
+            for (int64_t a = srp[i]; a < srp[i + 1]; ++a) ns += (sci[a] >= lo && sci[a] < hi);
+        }
+        lam[t] = cnt == 0 && ns == 0 ? LAM_F : cnt;
+        s_sum += ns;
+        t_sum += cnt;
+    }
+    sum[0][tid] = s_sum;
+    sum[1][tid] = t_sum;
+    __syncthreads();
+    int s_at = 0, t_at = 0, total = 0;
+    for (int u = 0; u < LT; ++u) {                     // the same order for every thread: broadcasts
+        if (u < tid) {
+            s_at += sum[0][u];
+            t_at += sum[1][u];
+        }
+        total += sum[0][u];                            // = the entries of S^T inside the block
+    }
+    const bool fits = total <= cap;
+    if (fits) {
+        for (int t = t0; t < t0 + per; ++t) {
+            sp[t] = (uint16_t)s_at;
+            tp[t] = (uint16_t)t_at;
+            if (t < m) {
+                const int64_t i = lo + t;
+                for (int64_t a = srp[i]; a < srp[i + 1]; ++a)
+                    if (sci[a] >= lo && sci[a] < hi) se[s_at++] = (uint16_t)(sci[a] - lo);
+                for (int64_t a = strp[i]; a < strp[i + 1]; ++a)
+                    if (stci[a] >= lo && stci[a] < hi) te[t_at++] = (uint16_t)(stci[a] - lo);
+            }
+        }
+        if (tid == LT - 1) {
+            sp[nb] = (uint16_t)s_at;
+            tp[nb] = (uint16_t)t_at;
+        }
+    }
+    for (int q = tid >> 5; q < ng1; q += LT / 32) {
+        const int mx = __reduce_max_sync(FULL, lam[q * 32 + lane]);
+        if (lane == 0) g1[q] = mx;
+    }
+    __syncthreads();
+    for (int q = tid >> 5; q < ng2; q += LT / 32) {
+        const int mx = __reduce_max_sync(FULL, g1[q * 32 + lane]);
+        if (lane == 0) g2[q] = mx;
+    }
+    __syncthreads();
+    if (tid < 32) {
+        const LocalGraph g{lo, m, srp, strp, sci, stci, sp, tp, se, te};
+        if (fits) local_picks<true>(g, ng1, ng2, lam, g1, g2, newF, err);
+        else local_picks<false>(g, ng1, ng2, lam, g1, g2, newF, err);
+    }
+    __syncthreads();
+    for (int t = tid; t < m; t += LT) cf[lo + t] = lam[t] == LAM_C ? CF_C : CF_F;
 }
 
 __device__ __forceinline__ double hash_frac(uint64_t x) {
@@ -256,12 +329,16 @@ int air_falgout_split(int64_t n, int64_t block, const int64_t *srp, const int32_
                       const int32_t *stci, int8_t *cf, int *d_err, cudaStream_t s) {
     if (block < 32 || block % 1024 != 0) return AIR_ERR_INVALID_ARG;
     const int64_t nblk = (n + block - 1) / block;
-    const int64_t ng1 = (block + 31) / 32, ng2 = (block + 1023) / 1024;
-    const size_t per_warp = (size_t)(block + ng1 + ng2 + NEWF_CAP) * sizeof(int32_t);
-    if (per_warp * FWARPS > AIR_SMEM_OPTIN) return AIR_ERR_UNSUPPORTED;     // block <= 8192 points
+    // entries of a block's graph in shared memory: six per point (HDG levels hold two to five inside a block), up to
+    // what the shared memory and 16-bit row starts allow; other blocks read the graph from global memory
+    const size_t fixed = (size_t)(block + block / 32 + block / 1024 + NEWF_CAP) * sizeof(int32_t) +
+                         2 * (size_t)(block + 2) * sizeof(uint16_t);
+    if (block > 8192) return AIR_ERR_UNSUPPORTED;
+    int64_t cap = (int64_t)((AIR_SMEM_OPTIN - 2048 - fixed) / (2 * sizeof(uint16_t)));   // 2048: the static arrays
+    if (cap > 6 * block) cap = 6 * block;
+    const size_t smem = fixed + 2 * (size_t)cap * sizeof(uint16_t);
     AIR_CUDA(air_smem_optin(local_pass_kernel));
-    local_pass_kernel<<<air_counted((unsigned)((nblk + FWARPS - 1) / FWARPS)), FWARPS * 32, per_warp * FWARPS, s>>>(
-        n, block, srp, sci, strp, stci, cf, d_err);
+    local_pass_kernel<<<air_counted((unsigned)nblk), LT, smem, s>>>(n, block, (int)cap, srp, sci, strp, stci, cf, d_err);
     AIR_LAUNCH();
     int8_t *inU = nullptr, *sel = nullptr;
     unsigned long long *count = nullptr;
