@@ -1130,14 +1130,38 @@ __global__ void rap_terms_kernel(int64_t nc, const int64_t *rrp, const int32_t *
     }
 }
 
-// One warp per coarse row i.  Stage 1: (RA)_ij over R entries k ascending and
-// A row k, accumulated into a per-warp hash table (within one k the columns j
-// are distinct, so no two lanes touch one slot).  Stage 2: keys (P(j), j)
-// sorted by a bitonic network, then every coarse column sums its terms in
-// ascending j.  COUNT mode only counts the coarse columns.  The table lives in
-// shared memory, or (GMEM, for rows with more terms than fit there) in a
-// global scratch area of HS x 20 bytes per warp of the grid.  rows (if not
-// NULL) lists the nrows coarse rows to process.
+// One warp per coarse row i; T = its number of terms r_ik a_kj, HS >= 2 T slots.
+//
+// FILL: (RA)_ij, k ascending, is accumulated per fine column j: a hash table of
+// HS slots finds the column's place in a dense list (within one k the columns
+// are distinct, so no two lanes touch one place).  Then the places are chained
+// by coarse column J = P(j) through a second table of HS / 2 slots in the same
+// memory, every coarse column finds its position in the row by counting the
+// smaller ones, and one lane per coarse column sums its chain in ascending j.
+// COUNT: the distinct coarse columns of the terms, from one table.
+// What bounds it: shared-memory latency and instructions, 16 to 24 warps per SM.
+// Sorting all (J, j) pairs by a bitonic network took twice as long: all
+// levels at 2.3 M unknowns, count 1.7 ms and fill 9.3 ms (8.5 and 17.5 ms).
+// Tables live in shared memory, or (GMEM, for rows with more terms than fit
+// there) in a global scratch area per warp of the grid.  rows (if not NULL)
+// lists the nrows coarse rows to process.
+__host__ __device__ constexpr size_t rap_slot_bytes(bool fill, bool gmem) { return fill ? (gmem ? 16 : 14) : 4; }
+
+__device__ __forceinline__ unsigned rap_hash(int32_t j, int bits) { return ((unsigned)j * 2654435761u) >> (32 - bits); }
+
+// Slot of key in the open-addressed table; fresh: it was not there.  -1: the table is full (cannot happen).
+__device__ __forceinline__ int rap_insert(int32_t *keys, int bits, int32_t key, bool &fresh) {
+    const int mask = (1 << bits) - 1;
+    unsigned h = rap_hash(key, bits);
+    for (int probe = 0; probe <= mask; ++probe) {
+        const int32_t old = atomicCAS(&keys[h], -1, key);
+        if (old == -1) { fresh = true; return (int)h; }
+        if (old == key) return (int)h;
+        h = (h + 1) & mask;
+    }
+    return -1;
+}
+
 template <bool FILL, bool GMEM>
 __global__ void rap_kernel(int64_t nrows, const int32_t *rows, const int64_t *rrp, const int32_t *rci,
                            const double *rv, const int64_t *rp, const int32_t *ci, const double *v,
@@ -1145,112 +1169,118 @@ __global__ void rap_kernel(int64_t nrows, const int32_t *rows, const int64_t *rr
                            const int64_t *acrp, int32_t *acci, double *acv, int *err) {
     extern __shared__ unsigned char rsm[];
     const int HS = 1 << hs_bits, HH = HS >> 1;
-    int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    unsigned char *base = GMEM ? gscratch + (size_t)global_warp() * (size_t)HS * 20
-                               : rsm + (size_t)wib * (size_t)HS * 20;
-    double *vals = (double *)base;                          // HS
-    unsigned long long *skey = (unsigned long long *)(vals + HS);   // HH
-    double *sval = (double *)(skey + HH);                   // HH
-    int32_t *keys = (int32_t *)(sval + HH);                 // HS
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const size_t per_warp = (size_t)HS * rap_slot_bytes(FILL, GMEM);
+    unsigned char *base = GMEM ? gscratch + (size_t)global_warp() * per_warp : rsm + (size_t)wib * per_warp;
+    // FILL: values and columns of the places (HH each), the table (HS keys, HS places) and the chains (HH); then in the
+    // keys' memory the coarse keys and chain heads (HH each), in the places' the coarse columns' slots (HH)
+    using Place = typename std::conditional<GMEM, int32_t, uint16_t>::type;
+    double *dval = (double *)base;
+    int32_t *keys = FILL ? (int32_t *)(dval + HH) : (int32_t *)base;
+    int32_t *dj = keys + HS;
+    Place *place = (Place *)(dj + HH);
+    int32_t *chain = (int32_t *)(place + HS);
     for (int64_t u = global_warp(); u < nrows; u += warp_count()) {
         const int64_t t = rows ? (int64_t)rows[u] : u;
         for (int s = lane; s < HS; s += 32) keys[s] = -1;
         __syncwarp();
-        for (int64_t q = rrp[t]; q < rrp[t + 1]; ++q) {
-            int32_t k = rci[q];
-            double rik = FILL ? rv[q] : 0.0;
-            for (int64_t e = rp[k] + lane; e < rp[k + 1]; e += 32) {
-                int32_t j = ci[e];
-                unsigned h = ((unsigned)j * 2654435761u) >> (32 - hs_bits);
-                bool placed = false;
-                for (int probe = 0; probe < HS; ++probe) {      // the table holds twice the row's terms
-                    int32_t old = atomicCAS(&keys[h], -1, j);
-                    if (old == -1) { if (FILL) vals[h] = 0.0; placed = true; break; }
-                    if (old == j) { placed = true; break; }
-                    h = (h + 1) & (HS - 1);
+        int n = 0;                                      // FILL: places in use; COUNT: coarse columns
+        for (int64_t q0 = rrp[t]; q0 < rrp[t + 1]; q0 += 32) {
+            // the rows of A that this chunk of R's row meets: bounds and factors of 32 at once
+            const int64_t ql = q0 + lane, qe = rrp[t + 1];
+            const int32_t k = ql < qe ? rci[ql] : 0;
+            const int64_t rs = ql < qe ? rp[k] : 0;
+            const int len = ql < qe ? (int)(rp[k + 1] - rs) : 0;
+            const double rk = FILL && ql < qe ? rv[ql] : 0.0;
+            const int nq = qe - q0 < 32 ? (int)(qe - q0) : 32;
+            for (int q = 0; q < nq; ++q) {
+                const int64_t b = __shfl_sync(FULL, rs, q);
+                const int l = __shfl_sync(FULL, len, q);
+                const double rik = FILL ? __shfl_sync(FULL, rk, q) : 0.0;
+                for (int e0 = 0; e0 < l; e0 += 32) {
+                    const bool on = e0 + lane < l;
+                    bool fresh = false;
+                    int at = -1;
+                    int32_t j = -1;
+                    double x = 0.0;
+                    if (on) {
+                        j = ci[b + e0 + lane];
+                        if (FILL) x = __dmul_rn(rik, v[b + e0 + lane]);
+                        else j = pcol[j];
+                        if (j >= 0) {
+                            at = rap_insert(keys, hs_bits, j, fresh);
+                            if (at < 0) atomicOr(err, AIR_DEVERR_CAP);
+                        }
+                    }
+                    const unsigned bal = __ballot_sync(FULL, fresh);
+                    if (FILL && at >= 0) {
+                        int p;
+                        if (fresh) {
+                            p = n + __popc(bal & lanemask_lt());
+                            place[at] = (Place)p;
+                            dj[p] = j;
+                            dval[p] = __dadd_rn(0.0, x);
+                        } else {
+                            p = (int)place[at];
+                            dval[p] = __dadd_rn(dval[p], x);
+                        }
+                    }
+                    n += __popc(bal);
+                    __syncwarp();
                 }
-                if (!placed) { atomicOr(err, AIR_DEVERR_CAP); continue; }
-                if (FILL) vals[h] = __dadd_rn(vals[h], __dmul_rn(rik, v[e]));
             }
-            __syncwarp();
         }
         if (!FILL) {
-            // COUNT: the number of distinct coarse columns P(j), from a second hash table
-            int32_t *jt = (int32_t *)skey;                  // HS slots (the sort area, unused here)
-            for (int s = lane; s < HS; s += 32) jt[s] = -1;
-            __syncwarp();
-            int heads = 0;
-            for (int s0 = 0; s0 < HS; s0 += 32) {
-                const int32_t j = keys[s0 + lane];
-                const int32_t J = j >= 0 ? pcol[j] : -1;
-                bool fresh = false;
-                if (J >= 0) {
-                    unsigned h = ((unsigned)J * 2654435761u) >> (32 - hs_bits);
-                    bool placed = false;
-                    for (int probe = 0; probe < HS; ++probe) {
-                        const int32_t old = atomicCAS(&jt[h], -1, J);
-                        if (old == -1) { fresh = true; placed = true; break; }
-                        if (old == J) { placed = true; break; }
-                        h = (h + 1) & (HS - 1);
-                    }
-                    if (!placed) atomicOr(err, AIR_DEVERR_CAP);
-                }
-                heads += __popc(__ballot_sync(FULL, fresh));
-            }
-            if (lane == 0) cnt[t] = heads;
+            if (lane == 0) cnt[t] = n;
             __syncwarp();
             continue;
         }
-        int cntv = 0;
-        for (int s0 = 0; s0 < HS; s0 += 32) {
-            int s = s0 + lane;
-            int32_t j = keys[s];
-            int32_t J = j >= 0 ? pcol[j] : -1;
-            bool ok = J >= 0;
-            unsigned bal = __ballot_sync(FULL, ok);
-            if (ok) {
-                int p = cntv + __popc(bal & lanemask_lt());
-                skey[p] = ((unsigned long long)(unsigned)J << 32) | (unsigned)j;
-                if (FILL) sval[p] = vals[s];
-            }
-            cntv += __popc(bal);
+        // coarse columns: table, chains of places, list of slots
+        int32_t *jkey = keys, *head = keys + HH, *slot = (int32_t *)place;
+        const int jb = hs_bits - 1;
+        for (int s = lane; s < HH; s += 32) {
+            jkey[s] = -1;
+            head[s] = -1;
         }
-        int P = 1;
-        while (P < cntv) P <<= 1;
-        for (int s = cntv + lane; s < P; s += 32) skey[s] = ~0ull;
         __syncwarp();
-        for (int size = 2; size <= P; size <<= 1) {
-            for (int stride = size >> 1; stride > 0; stride >>= 1) {
-                for (int idx = lane; idx < (P >> 1); idx += 32) {
-                    int a = 2 * stride * (idx / stride) + (idx % stride);
-                    int b = a + stride;
-                    bool up = (a & size) == 0;
-                    unsigned long long ka = skey[a], kb = skey[b];
-                    if ((ka > kb) == up) {
-                        skey[a] = kb; skey[b] = ka;
-                        if (FILL) { double t1 = sval[a]; sval[a] = sval[b]; sval[b] = t1; }
-                    }
+        int nj = 0;
+        for (int p0 = 0; p0 < n; p0 += 32) {
+            const int p = p0 + lane;
+            const int32_t J = p < n ? pcol[dj[p]] : -1;
+            bool fresh = false;
+            int at = -1;
+            if (J >= 0) {
+                at = rap_insert(jkey, jb, J, fresh);
+                if (at >= 0) chain[p] = atomicExch(&head[at], p);
+                else atomicOr(err, AIR_DEVERR_CAP);
+            }
+            const unsigned bal = __ballot_sync(FULL, fresh);
+            if (fresh) slot[nj + __popc(bal & lanemask_lt())] = at;
+            nj += __popc(bal);
+        }
+        __syncwarp();
+        const int64_t out = acrp[t];
+        for (int x = lane; x < nj; x += 32) {
+            const int at = slot[x];
+            const int32_t J = jkey[at];
+            int rank = 0;
+            for (int y = 0; y < nj; ++y) rank += jkey[slot[y]] < J ? 1 : 0;
+            double acc = 0.0;
+            int32_t last = -1;
+            for (;;) {                                  // the chain's next larger j
+                int32_t next = INT32_MAX;
+                int at_p = -1;
+                for (int p = head[at]; p >= 0; p = chain[p]) {
+                    const int32_t j = dj[p];
+                    if (j > last && j < next) { next = j; at_p = p; }
                 }
-                __syncwarp();
+                if (at_p < 0) break;
+                acc = __dadd_rn(acc, dval[at_p]);
+                last = next;
             }
+            acci[out + rank] = J;
+            acv[out + rank] = acc;
         }
-        int heads = 0;
-        int64_t out = FILL ? acrp[t] : 0;
-        for (int s0 = 0; s0 < cntv; s0 += 32) {
-            int s = s0 + lane;
-            bool head = s < cntv && (s == 0 || (skey[s] >> 32) != (skey[s - 1] >> 32));
-            unsigned bal = __ballot_sync(FULL, head);
-            if (FILL && head) {
-                unsigned long long J = skey[s] >> 32;
-                double acc = 0.0;
-                for (int u = s; u < cntv && (skey[u] >> 32) == J; ++u) acc = __dadd_rn(acc, sval[u]);
-                int64_t p = out + heads + __popc(bal & lanemask_lt());
-                acci[p] = (int32_t)J;
-                acv[p] = acc;
-            }
-            heads += __popc(bal);
-        }
-        if (!FILL && lane == 0) cnt[t] = heads;
         __syncwarp();
     }
 }
@@ -1551,11 +1581,21 @@ int air_rap_terms(const AirLevel &L, int32_t *terms, cudaStream_t s) {
 // class also any longer row).  lists: ncls x nc.
 __global__ void rap_class_kernel(int64_t nc, const int32_t *terms, int min_bits, int ncls, int32_t *lists,
                                  unsigned long long *counts) {
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nc; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t want = 2 * (int64_t)(terms[t] > 1 ? terms[t] : 1);
-        int c = 0;
-        while (c < ncls - 1 && ((int64_t)1 << (min_bits + c)) < want) ++c;
-        lists[(int64_t)c * nc + atomicAdd(&counts[c], 1ull)] = (int32_t)t;
+    // a warp takes its places in a list with one atomic
+    for (int64_t t0 = global_warp() * 32; t0 < nc; t0 += warp_count() * 32) {
+        const int64_t t = t0 + (threadIdx.x & 31);
+        int c = ncls;
+        if (t < nc) {
+            const int64_t want = 2 * (int64_t)(terms[t] > 1 ? terms[t] : 1);
+            c = 0;
+            while (c < ncls - 1 && ((int64_t)1 << (min_bits + c)) < want) ++c;
+        }
+        const unsigned same = __match_any_sync(FULL, c);
+        const int leader = __ffs(same) - 1;
+        unsigned long long at = 0;
+        if (c < ncls && (int)(threadIdx.x & 31) == leader) at = atomicAdd(&counts[c], (unsigned long long)__popc(same));
+        at = __shfl_sync(FULL, at, leader);
+        if (c < ncls) lists[(int64_t)c * nc + (int64_t)at + __popc(same & lanemask_lt())] = (int32_t)t;
     }
 }
 
@@ -1563,7 +1603,7 @@ template <bool FILL>
 int rap_launch(const AirLevel &L, int64_t nrows, const int32_t *rows, int bits, bool gmem, int32_t *cnt,
                const int64_t *acrp, int32_t *acci, double *acv, int *err, cudaStream_t s) {
     if (nrows <= 0) return AIR_OK;
-    const size_t per_warp = (size_t)(1 << bits) * 20;
+    const size_t per_warp = (size_t)(1 << bits) * rap_slot_bytes(FILL, gmem);
     if (!gmem) {
         int warps = (int)((160 * 1024) / per_warp);
         if (warps > 8) warps = 8;
