@@ -3,18 +3,30 @@
 // The V-cycle (Section 3: restriction of b, coarsest solve, one-point
 // interpolation, FCF-Jacobi sweeps) is bandwidth-bound: one right-hand side
 // reads every stored entry of every level for a few flops.  With k right-hand
-// sides stored row-major (row i holds x_i of all k systems, k <= 32) one warp
-// handles one matrix row: lane j carries system j, the row's entries are read
-// once (coalesced, then broadcast by shuffles) and serve all k systems, and
-// the gathered x rows are k contiguous values.  The matrix traffic of one
-// V-cycle is shared by k systems.
+// sides stored row-major (row i holds x_i of all k systems, k <= 32) a group of
+// lanes handles one matrix row: every lane carries up to 16 bytes of systems,
+// the row's entries are read once (coalesced, then broadcast by shuffles) and
+// serve all k systems, and the gathered x rows are k contiguous values.  The
+// matrix traffic of one V-cycle is shared by k systems.
+//
+// Bound: the latency of the gathered rows of x (L1 and L2) in FP32, FP64 issue in
+// FP64.  A whole warp per row with one system per lane issued two shuffles and a
+// load for every entry of every row; with 16 bytes per lane they serve four rows
+// at once (k = 32, FP32).  Four gathered rows in flight and 64 registers (32
+// warps per SM) were the best of 2, 4, 8 rows and 3 to 6 blocks per SM.  571,200
+// unknowns, 36 entries per row, k = 32, FP32: V-cycle 1968 -> 1090 us, the sweeps
+// and their copies 1575 -> 950 us.
 //
 // Every kernel sums a row in the CSR entry order with fused multiply-adds,
 // like the single-right-hand-side SELL kernels, so column j of the result is
 // the FP64 V-cycle of column j.
 #include <string.h>
 
+#include <initializer_list>
+#include <type_traits>
+
 #include "air_internal.cuh"
+#include "dependent.cuh"
 
 namespace {
 
@@ -29,84 +41,170 @@ unsigned grid_for(int64_t items, int threads, int64_t cap = 152 * 32) {
     return (unsigned)b;
 }
 
-// One warp per listed row (rows == NULL: row p itself).
+// V consecutive values as one access
+template <typename T, int V>
+struct alignas(V * sizeof(T)) Pack {
+    T v[V];
+};
+
+template <typename T>
+struct MultiArgs {
+    int64_t m;              // rows of the launch; rows == NULL: row p itself
+    const int32_t *rows;
+    const int64_t *rp;
+    const int32_t *ci;
+    const T *v;
+    int k;
+    const T *X;
+    T *Y;
+    const T *B, *dinv;
+    T omega;
+    int64_t mc;             // MR_JACOBI: rows copied unchanged from X to Y by the blocks past sweep_blocks
+    const int32_t *crows;
+    int64_t sweep_blocks;
+};
+
+// G lanes per row, V systems per lane (G V >= k, k a multiple of V), 32 / G rows per warp.
 //  MR_SPMV:   Y[row] = A_row X
 //  MR_RESID:  Y[row] = B[row] - A_row X
-//  MR_JACOBI: Y[p]   = X[row] + omega (B[row] - A_row X) / a_row,row   (compact; scattered afterwards)
-template <int MODE, typename T>
-__global__ void __launch_bounds__(256) csr_multi_kernel(int64_t m, const int32_t *__restrict__ rows,
-                                                        const int64_t *__restrict__ rp,
-                                                        const int32_t *__restrict__ ci,
-                                                        const T *__restrict__ v, int k,
-                                                        const T *__restrict__ X, T *__restrict__ Y,
-                                                        const T *__restrict__ B,
-                                                        const T *__restrict__ dinv, T omega) {
+//  MR_JACOBI: Y[row] = X[row] + omega (B[row] - A_row X) / a_row,row, the other rows copied: the sweeps alternate
+//             between two vectors
+template <int MODE, typename T, int V, int G>
+__global__ void __launch_bounds__(256, 4) csr_multi_kernel(MultiArgs<T> a) {
+    using P = Pack<T, V>;
+    constexpr int EL = G < 16 ? 16 / G : 1, BATCH = EL * G;    // entries per lane and per batch
+    constexpr int FLY = 4;                                     // rows of X in flight
+    const int lane = threadIdx.x & 31, gl = lane % G;
+    const unsigned gmask = G == 32 ? FULL : ((1u << (G & 31)) - 1u) << (lane / G * G);
+    const bool on = gl * V < a.k;
+    dep_launch();
+    if (MODE == MR_JACOBI && (int64_t)blockIdx.x >= a.sweep_blocks) {
+        const int64_t p = (((int64_t)blockIdx.x - a.sweep_blocks) * blockDim.x + threadIdx.x) / G;
+        const int32_t r = p < a.mc ? a.crows[p] : -1;
+        dep_wait();
+        if (r >= 0 && on) {
+            const int64_t at = (int64_t)r * a.k + gl * V;
+            *(P *)(a.Y + at) = *(const P *)(a.X + at);
+        }
+        return;
+    }
+    const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
+    if (p >= a.m) {                                              // a whole group
+        dep_wait();
+        return;
+    }
+    const int64_t row = a.rows ? (int64_t)a.rows[p] : p;
+    const int64_t e0 = a.rp[row], e1 = a.rp[row + 1];
+    P acc;
+#pragma unroll
+    for (int u = 0; u < V; ++u) acc.v[u] = 0;
+    const int64_t at = row * a.k + gl * V;
+    P b{}, xr{};
+    T d = 0;
+    // entries of the next batch are on their way while the rows of X of this one are
+    int32_t ce[EL];
+    T ve[EL];
+    auto entries = [&](int64_t base, int32_t *c, T *v) {
+#pragma unroll
+        for (int q = 0; q < EL; ++q) {
+            const int64_t e = base + q * G + gl;
+            c[q] = e < e1 ? a.ci[e] : 0;
+            v[q] = e < e1 ? a.v[e] : (T)0;
+        }
+    };
+    entries(e0, ce, ve);
+    if (MODE == MR_JACOBI) d = a.dinv[row];
+    dep_wait();
+    if (MODE != MR_SPMV && on) b = *(const P *)(a.B + at);
+    if (MODE == MR_JACOBI && on) xr = *(const P *)(a.X + at);
+    for (int64_t base = e0; base < e1; base += BATCH) {
+        int32_t cn[EL];
+        T vn[EL];
+        entries(base + BATCH, cn, vn);
+        const int cnt = (int)(e1 - base < BATCH ? e1 - base : BATCH);
+#pragma unroll
+        for (int t0 = 0; t0 < BATCH; t0 += FLY) {
+            if (t0 >= cnt) break;
+            P x[FLY];
+#pragma unroll
+            for (int t = 0; t < FLY; ++t) {
+                const int32_t c = __shfl_sync(gmask, ce[(t0 + t) / G], (t0 + t) % G, G);
+                if (!on) x[t] = P{};
+                else if (t0 + t < cnt) x[t] = *(const P *)(a.X + (int64_t)c * a.k + gl * V);
+            }
+#pragma unroll
+            for (int t = 0; t < FLY; ++t) {
+                const T w = __shfl_sync(gmask, ve[(t0 + t) / G], (t0 + t) % G, G);
+                if (t0 + t < cnt) {
+#pragma unroll
+                    for (int u = 0; u < V; ++u) acc.v[u] += w * x[t].v[u];
+                }
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < EL; ++q) {
+            ce[q] = cn[q];
+            ve[q] = vn[q];
+        }
+    }
+    if (!on) return;
+    if (MODE != MR_SPMV) {
+        if (MODE == MR_RESID) {
+#pragma unroll
+            for (int u = 0; u < V; ++u) acc.v[u] = b.v[u] - acc.v[u];
+        } else {
+#pragma unroll
+            for (int u = 0; u < V; ++u) acc.v[u] = xr.v[u] + a.omega * (b.v[u] - acc.v[u]) * d;
+        }
+    }
+    *(P *)(a.Y + at) = acc;
+}
+
+template <typename T, int V, int G>
+__global__ void __launch_bounds__(256) interp_multi_kernel(int64_t n, const int32_t *pcol, int k, const T *XC, T *X) {
+    using P = Pack<T, V>;
+    const int gl = threadIdx.x % G;
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
+    dep_launch();
+    if (i >= n || gl * V >= k) {
+        dep_wait();
+        return;
+    }
+    const int32_t pc = pcol[i];
+    dep_wait();
+    P x;
+#pragma unroll
+    for (int u = 0; u < V; ++u) x.v[u] = 0;
+    if (pc >= 0) x = *(const P *)(XC + (int64_t)pc * k + gl * V);
+    *(P *)(X + i * k + gl * V) = x;
+}
+
+// X = Cinv B on the coarsest level (Cinv row-major m x m), one warp per row, 32 rows of B in flight
+template <typename T>
+__global__ void __launch_bounds__(128) dense_multi_kernel(int64_t m, const T *__restrict__ Ci, int k,
+                                                          const T *B, T *X) {
     const int lane = threadIdx.x & 31;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; p < m; p += nw) {
-        const int64_t row = rows ? (int64_t)rows[p] : p;
-        const int64_t e0 = rp[row], e1 = rp[row + 1];
-        T acc = 0;
-        for (int64_t base = e0; base < e1; base += 32) {
-            const int64_t e = base + lane;
-            const int32_t ce = e < e1 ? ci[e] : 0;
-            const T ve = e < e1 ? v[e] : (T)0;
-            const int cnt = (int)(e1 - base < 32 ? e1 - base : 32);
-            for (int t = 0; t < cnt; ++t) {
-                const int32_t c = __shfl_sync(FULL, ce, t);
-                const T w = __shfl_sync(FULL, ve, t);
-                if (lane < k) acc += w * X[(int64_t)c * k + lane];
-            }
-        }
-        if (lane < k) {
-            if (MODE == MR_SPMV) {
-                Y[row * k + lane] = acc;
-            } else if (MODE == MR_RESID) {
-                Y[row * k + lane] = B[row * k + lane] - acc;
-            } else {
-                Y[p * k + lane] = X[row * k + lane] + omega * (B[row * k + lane] - acc) * dinv[row];
-            }
+    const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    dep_launch();
+    if (r >= m) {
+        dep_wait();
+        return;
+    }
+    T acc = 0, next = lane < m ? Ci[r * m + lane] : (T)0;
+    dep_wait();
+    for (int64_t c0 = 0; c0 < m; c0 += 32) {
+        const T cv = next;
+        next = c0 + 32 + lane < m ? Ci[r * m + c0 + 32 + lane] : (T)0;
+        T b[32];
+#pragma unroll
+        for (int t = 0; t < 32; ++t) b[t] = c0 + t < m && lane < k ? B[(c0 + t) * k + lane] : (T)0;
+#pragma unroll
+        for (int t = 0; t < 32; ++t) {
+            const T w = __shfl_sync(FULL, cv, t);
+            if (c0 + t < m) acc += w * b[t];
         }
     }
-}
-
-template <typename T>
-__global__ void scatter_multi_kernel(int64_t m, const int32_t *rows, int k, const T *Tc, T *X) {
-    const int64_t tot = m * k;
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < tot; q += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t p = q / k;
-        X[(int64_t)rows[p] * k + (q - p * k)] = Tc[q];
-    }
-}
-
-template <typename T>
-__global__ void interp_multi_kernel(int64_t n, const int32_t *pcol, int k, const T *XC, T *X) {
-    const int64_t tot = n * k;
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < tot; q += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = q / k;
-        const int32_t pc = pcol[i];
-        X[q] = pc >= 0 ? XC[(int64_t)pc * k + (q - i * k)] : (T)0;
-    }
-}
-
-// X = Cinv B on the coarsest level (Cinv row-major m x m), one warp per row
-template <typename T>
-__global__ void dense_multi_kernel(int64_t m, const T *__restrict__ Ci, int k, const T *__restrict__ B,
-                                   T *__restrict__ X) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < m; r += nw) {
-        T acc = 0;
-        for (int64_t c0 = 0; c0 < m; c0 += 32) {
-            const T cv = c0 + lane < m ? Ci[r * m + c0 + lane] : (T)0;
-            const int cnt = (int)(m - c0 < 32 ? m - c0 : 32);
-            for (int t = 0; t < cnt; ++t) {
-                const T w = __shfl_sync(FULL, cv, t);
-                if (lane < k) acc += w * B[(c0 + t) * k + lane];
-            }
-        }
-        if (lane < k) X[r * k + lane] = acc;
-    }
+    if (lane < k) X[r * k + lane] = acc;
 }
 
 // partial column dots: part[blk * 2k + d * k + j] = sum over this block's rows of U_ij W_ij
@@ -173,12 +271,48 @@ __global__ void copy_cols_kernel(int64_t n, int k, const int *mask, const double
         if (mask[q % k]) dst[q] = src[q];
 }
 
+// Systems per lane: 16 bytes where k and the vectors' alignment allow it, then 8, then one value.
+template <typename T>
+int pack_of(int k, std::initializer_list<const void *> vectors) {
+    uintptr_t all = (uintptr_t)k * sizeof(T);        // the length of a row, too
+    for (const void *p : vectors) all |= (uintptr_t)p;
+    return all % 16 == 0 ? (int)(16 / sizeof(T)) : (all % 8 == 0 ? (int)(8 / sizeof(T)) : 1);
+}
+
+// f(V, G) with the packing as compile-time constants: G the smallest power of two of at least four lanes that hold k
+template <typename T, int V, int G, typename F>
+void with_group(int k, F f) {
+    if constexpr (G * V < MK) {
+        if (k > G * V) return with_group<T, V, 2 * G>(k, f);
+    }
+    f(std::integral_constant<int, V>(), std::integral_constant<int, G>());
+}
+template <typename T, typename F>
+void with_pack(int k, int pack, F f) {
+    if (pack == (int)(16 / sizeof(T))) with_group<T, 16 / sizeof(T), 4>(k, f);
+    else if (sizeof(T) == 4 && pack == 2) with_group<T, 2, 4>(k, f);
+    else with_group<T, 1, 4>(k, f);
+}
+
 template <int MODE, typename T>
-void csr_multi(int64_t m, const int32_t *rows, const int64_t *rp, const int32_t *ci, const T *v, int k, const T *X,
-               T *Y, const T *B, const T *dinv, T omega, cudaStream_t s) {
-    if (m <= 0) return;
-    csr_multi_kernel<MODE, T><<<air_counted(grid_for(m * 32, 256)), 256, 0, s>>>(m, rows, rp, ci, v, k, X, Y, B,
-                                                                                dinv, omega);
+void csr_multi(const MultiArgs<T> &a0, bool dependent, cudaStream_t s) {
+    if (a0.m <= 0 && a0.mc <= 0) return;
+    with_pack<T>(a0.k, pack_of<T>(a0.k, {a0.X, a0.Y, a0.B}), [&](auto v, auto g) {
+        MultiArgs<T> a = a0;
+        a.sweep_blocks = (a.m * g() + 255) / 256;
+        const int64_t blocks = a.sweep_blocks + (MODE == MR_JACOBI ? (a.mc * g() + 255) / 256 : 0);
+        const auto kernel = csr_multi_kernel<MODE, T, v(), g()>;
+        if (dependent) launch_dependent(kernel, (unsigned)blocks, 256, s, a);
+        else kernel<<<air_counted((unsigned)blocks), 256, 0, s>>>(a);
+    });
+}
+
+template <int MODE, typename T>
+void csr_multi(int64_t m, const int64_t *rp, const int32_t *ci, const T *v, int k, const T *X, T *Y, const T *B,
+               cudaStream_t s, bool dependent = false) {
+    MultiArgs<T> a{};
+    a.m = m; a.rp = rp; a.ci = ci; a.v = v; a.k = k; a.X = X; a.Y = Y; a.B = B;
+    csr_multi<MODE, T>(a, dependent, s);
 }
 
 // the V-cycle buffers only: the Krylov vectors of a solve in progress stay
@@ -198,10 +332,9 @@ int ensure_multi(air_hierarchy *H, int k) {
     for (int l = 0; l < H->nlev; ++l) {
         const AirLevel &L = H->lev[l];
         const int64_t n = L.n > 0 ? L.n : 1;
-        const int64_t mt = (L.nf > L.nc ? L.nf : L.nc) > 0 ? (L.nf > L.nc ? L.nf : L.nc) : 1;
         AIR_CUDA(air_dmalloc((void **)&H->mb[l], (size_t)n * k * sizeof(double)));
         AIR_CUDA(air_dmalloc((void **)&H->mx[l], (size_t)n * k * sizeof(double)));
-        AIR_CUDA(air_dmalloc((void **)&H->mt[l], (size_t)mt * k * sizeof(double)));
+        AIR_CUDA(air_dmalloc((void **)&H->mt[l], (size_t)n * k * sizeof(double)));
     }
     H->mk = k;
     return AIR_OK;
@@ -266,28 +399,42 @@ int vcycle_multi_t(air_hierarchy *H, int k, const T *b0, T *x0, cudaStream_t s) 
     for (int l = 0; l + 1 < L; ++l) {                      // restriction of b
         const AirLevel &A = H->lev[l];
         const T *bl = l == 0 ? b0 : mb(l);
-        csr_multi<MR_SPMV, T>(A.nc, nullptr, A.rrp, A.rci, rvals(l), k, bl, mb(l + 1), nullptr, nullptr, (T)0, s);
+        csr_multi<MR_SPMV, T>(A.nc, A.rrp, A.rci, rvals(l), k, bl, mb(l + 1), nullptr, s, l > 0);
     }
     {                                                      // coarsest
         const AirLevel &C = H->lev[L - 1];
         const T *bl = L == 1 ? b0 : mb(L - 1);
         T *xl = L == 1 ? x0 : mx(L - 1);
         const T *Ci = F ? (const T *)H->mc32 : (const T *)H->cinv;
-        dense_multi_kernel<T><<<air_counted(grid_for(C.n * 32, 256, 152 * 8)), 256, 0, s>>>(C.n, Ci, k, bl, xl);
+        const auto kernel = dense_multi_kernel<T>;
+        const unsigned blocks = (unsigned)((C.n + 3) / 4);
+        if (L > 1) launch_dependent(kernel, blocks, 128, s, C.n, Ci, k, bl, xl);
+        else kernel<<<air_counted(blocks), 128, 0, s>>>(C.n, Ci, k, bl, xl);
     }
     for (int l = L - 2; l >= 0; --l) {                     // interpolation and sweeps
         const AirLevel &A = H->lev[l];
         const T *bl = l == 0 ? b0 : mb(l);
-        T *out = l == 0 ? x0 : mx(l);
-        interp_multi_kernel<T><<<air_counted(grid_for(A.n * k, 256)), 256, 0, s>>>(A.n, A.pcol, k, mx(l + 1), out);
+        T *out = l == 0 ? x0 : mx(l), *alt = (T *)H->mt[l];
+        const T *xc = mx(l + 1);
+        // P x_c starts in whichever vector makes the last sweep end in out
+        T *cur = ns % 2 == 1 ? alt : out, *nxt = ns % 2 == 1 ? out : alt;
+        with_pack<T>(k, pack_of<T>(k, {xc, cur}), [&](auto v, auto g) {
+            launch_dependent(interp_multi_kernel<T, v(), g()>, (unsigned)((A.n * g() + 255) / 256), 256, s, A.n, A.pcol,
+                             k, xc, cur);
+        });
         for (int q = 0; q < ns; ++q) {
             const bool c = relax[q] == 'C';
-            const int64_t m = c ? A.nc : A.nf;
-            const int32_t *rows = c ? A.crows : A.frows;
-            if (m <= 0) continue;
-            T *tl = (T *)H->mt[l];
-            csr_multi<MR_JACOBI, T>(m, rows, A.rp, A.ci, vals(l), k, out, tl, bl, dinv(l), omega, s);
-            scatter_multi_kernel<T><<<air_counted(grid_for(m * k, 256)), 256, 0, s>>>(m, rows, k, tl, out);
+            MultiArgs<T> a{};
+            a.m = c ? A.nc : A.nf;
+            a.rows = c ? A.crows : A.frows;
+            a.mc = c ? A.nf : A.nc;
+            a.crows = c ? A.frows : A.crows;
+            a.rp = A.rp; a.ci = A.ci; a.v = vals(l); a.k = k; a.X = cur; a.Y = nxt; a.B = bl; a.dinv = dinv(l);
+            a.omega = omega;
+            csr_multi<MR_JACOBI, T>(a, true, s);
+            T *t = cur;
+            cur = nxt;
+            nxt = t;
         }
     }
     AIR_LAUNCH();
@@ -399,7 +546,7 @@ int air_bicgstab_multi_impl(const air_hierarchy *Hc, int k, const double *b, dou
         AIR_TRY(coef(hc2, c2));
         AIR_TRY(lincomb(p, r, ones, p, c1, v, c2));                       // p = r + beta (p - omega v)
         AIR_TRY(precond(p, ph));
-        csr_multi<MR_SPMV, double>(n, nullptr, A0.rp, A0.ci, A0.v, k, ph, v, nullptr, nullptr, 0.0, s);
+        csr_multi<MR_SPMV, double>(n, A0.rp, A0.ci, A0.v, k, ph, v, nullptr, s);
         AIR_TRY(dots(rh, nullptr, v));
         for (int j = 0; j < k; ++j) {
             if (!done[j] && hd[j] == 0.0) { done[j] = true; --active; }
@@ -409,7 +556,7 @@ int air_bicgstab_multi_impl(const air_hierarchy *Hc, int k, const double *b, dou
         AIR_TRY(coef(hc1, c1));
         AIR_TRY(lincomb(sv, r, ones, v, c1, nullptr, nullptr));           // s = r - alpha v
         AIR_TRY(precond(sv, sh));
-        csr_multi<MR_SPMV, double>(n, nullptr, A0.rp, A0.ci, A0.v, k, sh, t, nullptr, nullptr, 0.0, s);
+        csr_multi<MR_SPMV, double>(n, A0.rp, A0.ci, A0.v, k, sh, t, nullptr, s);
         AIR_TRY(dots(sv, t, t));                                           // (s, t), (t, t)
         for (int j = 0; j < k; ++j) {
             const double ts = hd[j], tt = hd[k + j];
@@ -439,7 +586,7 @@ int air_bicgstab_multi_impl(const air_hierarchy *Hc, int k, const double *b, dou
         if (check) {
             // the true residual decides the columns whose recursive residual met rtol;
             // those above rtol restart from it
-            csr_multi<MR_RESID, double>(n, nullptr, A0.rp, A0.ci, A0.v, k, x, t, b, nullptr, 0.0, s);
+            csr_multi<MR_RESID, double>(n, A0.rp, A0.ci, A0.v, k, x, t, b, s);
             AIR_TRY(dots(t, nullptr, t));
             bool restart = false;
             for (int j = 0; j < k; ++j) {
@@ -476,7 +623,7 @@ int air_bicgstab_multi_impl(const air_hierarchy *Hc, int k, const double *b, dou
             if (!done[j] && omega[j] == 0.0) { done[j] = true; --active; }   // stagnation
     }
     // true residual of the columns that did not converge
-    csr_multi<MR_RESID, double>(n, nullptr, A0.rp, A0.ci, A0.v, k, x, t, b, nullptr, 0.0, s);
+    csr_multi<MR_RESID, double>(n, A0.rp, A0.ci, A0.v, k, x, t, b, s);
     AIR_TRY(dots(t, nullptr, t));
     for (int j = 0; j < k; ++j)
         if (info[j].status != AIR_OK) info[j].relres = bn[j] > 0.0 ? sqrt(hd[j]) / bn[j] : 0.0;

@@ -16,6 +16,7 @@
 #include <cuda_bf16.h>
 
 #include "air_internal.cuh"
+#include "dependent.cuh"
 
 namespace {
 
@@ -57,29 +58,6 @@ __device__ __forceinline__ A seg_sum(A s) {
 // and the launch's extra blocks copy the rows the sweep leaves unchanged
 // (crows), so that the sweeps alternate between two vectors.
 enum { ROW_SPMV = 0, ROW_JACOBI = 1 };
-
-// The V-cycle's kernels are launched with programmatic dependence: a grid may
-// start while the one before it still runs, reads what no V-cycle writes (the
-// matrix, row lists, 1 / a_ii) and only then waits for it.  Between kernels of
-// a few microseconds that hides the launch and the first load latencies.  A
-// kernel reads vectors and writes only after dep_wait, which at least one thread
-// of every grid reaches, so the end of a grid also is the end of all before it.
-__device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
-template <typename Args>
-void launch_dependent(void (*kernel)(Args), unsigned grid, const Args &a, cudaStream_t s) {
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = air_counted(grid);
-    cfg.blockDim = dim3(256);
-    cfg.stream = s;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, a);
-}
 
 // Block blk of the copy part of a ROW_JACOBI launch: COPY_R rows per thread.
 constexpr int COPY_R = 4;
@@ -534,7 +512,7 @@ void bsell_launch_b(const BSellArgs<TV, TX> &a0, bool pairs, cudaStream_t s) {
     BSellArgs<TV, TX> a = a0;
     a.sweep_blocks = (a.m + 255) / 256;
     const unsigned g = (unsigned)(a.sweep_blocks + (MODE == ROW_JACOBI ? copy_blocks(a.mc) : 0));
-    launch_dependent(pairs ? bsell_kernel<B, true, TV, TX, MODE> : bsell_kernel<B, false, TV, TX, MODE>, g, a, s);
+    launch_dependent(pairs ? bsell_kernel<B, true, TV, TX, MODE> : bsell_kernel<B, false, TV, TX, MODE>, g, 256, s, a);
 }
 
 // pairs are safe when x starts on a pair boundary (the values always do)
@@ -556,7 +534,7 @@ void sell_lanes_launch(const SellArgs<TV, TX> &a0, cudaStream_t s) {
     SellArgs<TV, TX> a = a0;
     a.sweep_blocks = (a.m * VL + 255) / 256;
     const int64_t g = a.sweep_blocks + (MODE == ROW_JACOBI ? copy_blocks(a.mc) : 0);
-    launch_dependent(sell_kernel<VL, (VL <= 2 && sizeof(TX) == 4 ? 12 : 8), TV, TX, MODE>, (unsigned)g, a, s);
+    launch_dependent(sell_kernel<VL, (VL <= 2 && sizeof(TX) == 4 ? 12 : 8), TV, TX, MODE>, (unsigned)g, 256, s, a);
 }
 
 template <typename TV, typename TX, int MODE>
@@ -885,7 +863,7 @@ int vcycle_t(const air_hierarchy *H, const T *b0, T *x0, cudaStream_t s) {
         const T *bl = L == 1 ? b0 : (const T *)C.b;
         T *xl = L == 1 ? x0 : (T *)C.x;
         const T *Ci = std::is_same<T, double>::value ? (const T *)H->cinv : (const T *)H->cinv32;
-        launch_dependent(dense_gemv_kernel<T>, (unsigned)((C.n + 7) / 8), GemvArgs<T>{C.n, Ci, bl, xl}, s);
+        launch_dependent(dense_gemv_kernel<T>, (unsigned)((C.n + 7) / 8), 256, s, GemvArgs<T>{C.n, Ci, bl, xl});
     }
     // interpolation and relaxation back up
     for (int l = L - 2; l >= 0; --l) {
@@ -899,8 +877,8 @@ int vcycle_t(const air_hierarchy *H, const T *b0, T *x0, cudaStream_t s) {
         // x = P x_c, then the sweeps alternate between out and alt, starting in
         // whichever of the two makes the last one end in out
         T *cur = ns % 2 == 1 ? alt : out, *nxt = ns % 2 == 1 ? out : alt;
-        launch_dependent(interp_kernel<T>, (unsigned)((A.n + 256 * INTERP_R - 1) / (256 * INTERP_R)),
-                         InterpArgs<T>{A.n, A.pcol, xc, cur}, s);
+        launch_dependent(interp_kernel<T>, (unsigned)((A.n + 256 * INTERP_R - 1) / (256 * INTERP_R)), 256, s,
+                         InterpArgs<T>{A.n, A.pcol, xc, cur});
         for (int q = 0; q < ns; ++q) {
             const char c = relax[q];
             if (c == 'A') {
