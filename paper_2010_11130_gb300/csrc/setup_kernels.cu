@@ -7,6 +7,7 @@
 #include <float.h>
 #include <math.h>
 
+#include <type_traits>
 #include <vector>
 
 #include "air_internal.cuh"
@@ -1134,18 +1135,21 @@ __global__ void rap_terms_kernel(int64_t nc, const int64_t *rrp, const int32_t *
 //
 // FILL: (RA)_ij, k ascending, is accumulated per fine column j: a hash table of
 // HS slots finds the column's place in a dense list (within one k the columns
-// are distinct, so no two lanes touch one place).  Then the places are chained
-// by coarse column J = P(j) through a second table of HS / 2 slots in the same
-// memory, every coarse column finds its position in the row by counting the
-// smaller ones, and one lane per coarse column sums its chain in ascending j.
+// are distinct, so no two lanes touch one place).  Then a second table of HS / 2
+// slots in the same memory counts the places of every coarse column J = P(j);
+// the places are listed by coarse column, ordered by j within one (every place
+// counts the smaller ones of its column), every coarse column finds its position
+// in the row by counting the smaller ones, and one lane per coarse column sums its
+// places in ascending j.
 // COUNT: the distinct coarse columns of the terms, from one table.
 // What bounds it: shared-memory latency and instructions, 16 to 24 warps per SM.
-// Sorting all (J, j) pairs by a bitonic network took twice as long: all
-// levels at 2.3 M unknowns, count 1.7 ms and fill 9.3 ms (8.5 and 17.5 ms).
+// All levels at 2.3 M unknowns: count 1.7 ms, fill 5.6 ms.  A bitonic sort of all
+// (J, j) pairs took 17.5 ms, and linked lists by J from which one lane took the
+// smallest j again and again 9.3 ms (a level of 1,745 rows 2.27 ms, now 0.21).
 // Tables live in shared memory, or (GMEM, for rows with more terms than fit
 // there) in a global scratch area per warp of the grid.  rows (if not NULL)
 // lists the nrows coarse rows to process.
-__host__ __device__ constexpr size_t rap_slot_bytes(bool fill, bool gmem) { return fill ? (gmem ? 16 : 14) : 4; }
+__host__ __device__ constexpr size_t rap_slot_bytes(bool fill, bool gmem) { return fill ? (gmem ? 20 : 14) : 4; }
 
 __device__ __forceinline__ unsigned rap_hash(int32_t j, int bits) { return ((unsigned)j * 2654435761u) >> (32 - bits); }
 
@@ -1172,14 +1176,19 @@ __global__ void rap_kernel(int64_t nrows, const int32_t *rows, const int64_t *rr
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const size_t per_warp = (size_t)HS * rap_slot_bytes(FILL, GMEM);
     unsigned char *base = GMEM ? gscratch + (size_t)global_warp() * per_warp : rsm + (size_t)wib * per_warp;
-    // FILL: values and columns of the places (HH each), the table (HS keys, HS places) and the chains (HH); then in the
-    // keys' memory the coarse keys and chain heads (HH each), in the places' the coarse columns' slots (HH)
+    // FILL, HH entries each unless noted: values of the places; the table's keys (HS), later the coarse keys and their
+    // (first place, number of places); (coarse slot, arrival) of the places; their columns; the table's places (HS), later
+    // the coarse columns' slots and the list of places
     using Place = typename std::conditional<GMEM, int32_t, uint16_t>::type;
+    using Pair = typename std::conditional<GMEM, unsigned long long, unsigned>::type;
+    constexpr int SH = GMEM ? 32 : 13;                  // shared tables: both numbers are at most 4096
+    constexpr Pair LOW = ((Pair)1 << SH) - 1, NONE = ~(Pair)0;
     double *dval = (double *)base;
     int32_t *keys = FILL ? (int32_t *)(dval + HH) : (int32_t *)base;
-    int32_t *dj = keys + HS;
+    Pair *seg = (Pair *)(keys + HH);
+    Pair *pair = GMEM ? seg + HH : (Pair *)(keys + HS);
+    int32_t *dj = (int32_t *)(pair + HH);
     Place *place = (Place *)(dj + HH);
-    int32_t *chain = (int32_t *)(place + HS);
     for (int64_t u = global_warp(); u < nrows; u += warp_count()) {
         const int64_t t = rows ? (int64_t)rows[u] : u;
         for (int s = lane; s < HS; s += 32) keys[s] = -1;
@@ -1235,12 +1244,13 @@ __global__ void rap_kernel(int64_t nrows, const int32_t *rows, const int64_t *rr
             __syncwarp();
             continue;
         }
-        // coarse columns: table, chains of places, list of slots
-        int32_t *jkey = keys, *head = keys + HH, *slot = (int32_t *)place;
+        // coarse columns: table, number of places, list of slots
+        int32_t *jkey = keys;
+        Place *slot = place, *list = place + HH;
         const int jb = hs_bits - 1;
         for (int s = lane; s < HH; s += 32) {
             jkey[s] = -1;
-            head[s] = -1;
+            seg[s] = 0;
         }
         __syncwarp();
         int nj = 0;
@@ -1251,13 +1261,46 @@ __global__ void rap_kernel(int64_t nrows, const int32_t *rows, const int64_t *rr
             int at = -1;
             if (J >= 0) {
                 at = rap_insert(jkey, jb, J, fresh);
-                if (at >= 0) chain[p] = atomicExch(&head[at], p);
-                else atomicOr(err, AIR_DEVERR_CAP);
+                if (at < 0) atomicOr(err, AIR_DEVERR_CAP);
             }
+            if (p < n) pair[p] = at >= 0 ? (Pair)at << SH | atomicAdd(&seg[at], (Pair)1) : NONE;
             const unsigned bal = __ballot_sync(FULL, fresh);
-            if (fresh) slot[nj + __popc(bal & lanemask_lt())] = at;
+            if (fresh) slot[nj + __popc(bal & lanemask_lt())] = (Place)at;
             nj += __popc(bal);
         }
+        __syncwarp();
+        int total = 0;
+        for (int x0 = 0; x0 < nj; x0 += 32) {           // first places of the columns
+            const int at = x0 + lane < nj ? (int)slot[x0 + lane] : -1;
+            const int c = at >= 0 ? (int)seg[at] : 0;
+            int sum = c;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int o = __shfl_up_sync(FULL, sum, d);
+                if (lane >= d) sum += o;
+            }
+            if (at >= 0) seg[at] = (Pair)(total + sum - c) << SH | (Pair)c;
+            total += __shfl_sync(FULL, sum, 31);
+        }
+        __syncwarp();
+        for (int p = lane; p < n; p += 32) {            // by column, in order of arrival
+            const Pair a = pair[p];
+            if (a != NONE) list[(int)(seg[(int)(a >> SH)] >> SH) + (int)(a & LOW)] = (Place)p;
+        }
+        __syncwarp();
+        for (int p = lane; p < n; p += 32) {            // the place's position when ordered by j
+            const Pair a = pair[p];
+            if (a == NONE) continue;
+            const Pair sg = seg[(int)(a >> SH)];
+            const int q0 = (int)(sg >> SH), q1 = q0 + (int)(sg & LOW);
+            const int32_t j = dj[p];
+            int at = q0;
+            for (int q = q0; q < q1; ++q) at += dj[list[q]] < j ? 1 : 0;
+            pair[p] = (Pair)at;
+        }
+        __syncwarp();
+        for (int p = lane; p < n; p += 32)
+            if (pair[p] != NONE) list[(int)pair[p]] = (Place)p;
         __syncwarp();
         const int64_t out = acrp[t];
         for (int x = lane; x < nj; x += 32) {
@@ -1265,19 +1308,9 @@ __global__ void rap_kernel(int64_t nrows, const int32_t *rows, const int64_t *rr
             const int32_t J = jkey[at];
             int rank = 0;
             for (int y = 0; y < nj; ++y) rank += jkey[slot[y]] < J ? 1 : 0;
+            const int q0 = (int)(seg[at] >> SH), q1 = q0 + (int)(seg[at] & LOW);
             double acc = 0.0;
-            int32_t last = -1;
-            for (;;) {                                  // the chain's next larger j
-                int32_t next = INT32_MAX;
-                int at_p = -1;
-                for (int p = head[at]; p >= 0; p = chain[p]) {
-                    const int32_t j = dj[p];
-                    if (j > last && j < next) { next = j; at_p = p; }
-                }
-                if (at_p < 0) break;
-                acc = __dadd_rn(acc, dval[at_p]);
-                last = next;
-            }
+            for (int q = q0; q < q1; ++q) acc = __dadd_rn(acc, dval[list[q]]);
             acci[out + rank] = J;
             acv[out + rank] = acc;
         }
