@@ -14,15 +14,16 @@
 // C, its undecided strong dependants in the block become F, every undecided
 // point of the block in S_j of a new F point j gains one, every undecided
 // point of the block in S_i loses one; stop when the largest measure is 0 (the
-// rest become F).  The maximum is found through two levels of upper bounds
-// (per 32 points and per 1024 points) that increments raise and searches
-// repair when they meet a stale one.  What bounds it is the chain of picks of
-// one block (a block of 8192 points has 2,000 to 3,600; blocks run side by
-// side): a pick is about a dozen dependent accesses, in shared memory 30 cycles
-// each, in the L2 300 to 600.  The block's graph, 16-bit local indices both ways,
-// is therefore gathered into shared memory first, and the strong connections of
-// four new F points are raised together.  All levels at 2.3 M unknowns: 17.5 ms
-// (40.8 ms with the graph in global memory and one F point after the other).
+// rest become F).  The maximum is found through upper bounds per 32 points that
+// increments raise and searches repair when they meet a stale one; the largest
+// bound and its first group come out of one maximum over (bound, group) keys.
+// What bounds it is the chain of picks of one block (a block of 8192 points has
+// 2,000 to 3,600; blocks run side by side): a pick is a dozen dependent accesses,
+// in shared memory 30 cycles each, in the L2 300 to 600.  The block's graph, 16-bit
+// local indices both ways, is therefore gathered into shared memory first, and the
+// strong connections of up to sixteen new F points are raised together.  All levels
+// at 2.3 M unknowns: 13.5 ms (40.8 ms with the graph in global memory and one F point
+// after the other, 17.4 ms with two levels of bounds and four F points at a time).
 //
 // Interface rounds: U = F points with S_i non-empty, no C point in S_i and a
 // strong connection (either way) to another block.  Weight
@@ -30,12 +31,14 @@
 // Flood, 2014).  A point of U whose weight beats every point of U in S_i and
 // S^T_i (ties -> smaller index) becomes C; points of U with a C point in S_i
 // leave U; repeat until U is empty.
+#include <type_traits>
+
 #include "air_internal.cuh"
 
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
-constexpr int LT = 256;              // threads per block of points: all gather its graph, one warp picks
+constexpr int LT = 1024;             // threads per block of points: all gather its graph, one warp picks
 constexpr int NEWF_CAP = 1024;       // new F points of one pick
 constexpr int LAM_F = -1, LAM_C = -2;
 constexpr int8_t CF_F = 0, CF_C = 1;
@@ -53,7 +56,7 @@ unsigned grid_for(int64_t items, int threads) {
     return (unsigned)b;
 }
 
-// Shared memory of one block of points: lam[block], g1[block / 32], g2[block / 1024], newF[NEWF_CAP] (int32), then 16
+// Shared memory of one block of points: lam[block], g1[block / 32], newF[NEWF_CAP] (int32), then 16
 // bits each: row starts of S and of S^T (block + 1, padded to even), their entries (cap each).
 struct LocalGraph {
     int64_t lo;                       // first point and number of points
@@ -67,7 +70,8 @@ struct LocalGraph {
 // neighbour or -1 outside the block.
 template <bool SMEM, bool T>
 struct Row {
-    int64_t first, last;
+    using Entry = typename std::conditional<SMEM, int, int64_t>::type;
+    Entry first, last;
     __device__ __forceinline__ Row(const LocalGraph &g, int j) {
         if (SMEM) {
             const uint16_t *p = T ? g.tp : g.sp;
@@ -79,17 +83,65 @@ struct Row {
             last = p[g.lo + j + 1];
         }
     }
-    __device__ __forceinline__ int at(const LocalGraph &g, int64_t e) const {
+    __device__ __forceinline__ int at(const LocalGraph &g, Entry e) const {
         if (SMEM) return (T ? g.te : g.se)[e];
-        const int64_t k = (T ? g.stci : g.sci)[e] - g.lo;
+        return local(g, (T ? g.stci : g.sci)[e]);
+    }
+    static __device__ __forceinline__ int local(const LocalGraph &g, int32_t i) {
+        const int64_t k = i - g.lo;
         return k >= 0 && k < g.m ? (int)k : -1;
     }
 };
 
+// One more for the undecided points in the rows of S listed in newF: eight lanes per row, 4 R rows in flight.
+template <bool SMEM, int R>
+__device__ __forceinline__ void raise_rows(const LocalGraph &g, int nf, const int32_t *newF, int32_t *lam, int32_t *g1) {
+    const int lane = threadIdx.x & 31;
+    for (int q0 = lane >> 3; q0 < nf; q0 += 4 * R) {
+        typename Row<SMEM, false>::Entry first[R], last[R];
+        bool more = false;
+#pragma unroll
+        for (int u = 0; u < R; ++u) {
+            first[u] = last[u] = 0;
+            if (q0 + 4 * u < nf) {
+                const int32_t f = newF[q0 + 4 * u];
+                if (SMEM) {
+                    first[u] = (unsigned)f & 0xffffu;
+                    last[u] = (unsigned)f >> 16;
+                } else {
+                    const Row<false, false> r(g, f);
+                    first[u] = r.first;
+                    last[u] = r.last;
+                }
+            }
+            first[u] += lane & 7;
+            more |= first[u] < last[u];
+        }
+        while (more) {
+            int k[R];
+            bool up[R];
+            more = false;
+#pragma unroll
+            for (int u = 0; u < R; ++u) {
+                k[u] = first[u] < last[u] ? (SMEM ? (int)g.se[first[u]] : Row<false, false>::local(g, g.sci[first[u]])) : -1;
+                first[u] += 8;
+                more |= first[u] < last[u];
+            }
+#pragma unroll
+            for (int u = 0; u < R; ++u) up[u] = k[u] >= 0 && lam[k[u]] >= 0;
+#pragma unroll
+            for (int u = 0; u < R; ++u)
+                if (up[u]) {
+                    const int nv = atomicAdd(&lam[k[u]], 1) + 1;
+                    atomicMax(&g1[k[u] >> 5], nv);
+                }
+        }
+    }
+}
+
 // The picks of one block, by one warp.
 template <bool SMEM>
-__device__ void local_picks(const LocalGraph &g, int ng1, int ng2, int32_t *lam, int32_t *g1, int32_t *g2,
-                            int32_t *newF, int *err) {
+__device__ void local_picks(const LocalGraph &g, int ng1, int32_t *lam, int32_t *g1, int32_t *newF, int *err) {
     const int lane = threadIdx.x & 31;
     const int64_t cap = 64 * (int64_t)g.m + 1024;  // picks plus repairs of stale bounds (a safety net)
     for (int64_t step = 0;; ++step) {
@@ -97,22 +149,17 @@ __device__ void local_picks(const LocalGraph &g, int ng1, int ng2, int32_t *lam,
             if (lane == 0) atomicOr(err, AIR_DEVERR_RS_CAP);
             break;
         }
-        // level 2 (at most 8 ranges): the largest bound and its first 1024-point range
-        const int v2 = lane < ng2 ? g2[lane] : LAM_C;
-        const int top = __reduce_max_sync(FULL, v2);
+        // the largest bound of a 32-point group and the first group that has it, in one maximum: at most 256 groups
+        int key = INT32_MIN;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (32 * u < ng1) {
+                const int q = lane + 32 * u;
+                key = max(key, g1[q] * 256 + (255 - q));
+            }
+        key = __reduce_max_sync(FULL, key);
+        const int top = key >> 8, q1 = 255 - (key & 255);
         if (top < 1) break;
-        const int h = __ffs(__ballot_sync(FULL, v2 == top)) - 1;
-        // level 1: the first 32-point group of that range with the bound
-        const int gi = h * 32 + lane;
-        const int b1 = gi < ng1 ? g1[gi] : LAM_C;
-        const unsigned bal1 = __ballot_sync(FULL, b1 == top);
-        if (!bal1) {                                   // stale range bound: repair it
-            const int mx = __reduce_max_sync(FULL, b1);
-            if (lane == 0) g2[h] = mx;
-            __syncwarp();
-            continue;
-        }
-        const int q1 = h * 32 + __ffs(bal1) - 1;
         const int lv = lam[q1 * 32 + lane];
         const unsigned bal0 = __ballot_sync(FULL, lv == top);
         if (!bal0) {                                   // stale group bound: repair it
@@ -121,28 +168,23 @@ __device__ void local_picks(const LocalGraph &g, int ng1, int ng2, int32_t *lam,
             __syncwarp();
             continue;
         }
-        const int i = q1 * 32 + __ffs(bal0) - 1;
+        const int picked = __ffs(bal0) - 1, i = q1 * 32 + picked;
         const Row<SMEM, true> dep(g, i);
         const Row<SMEM, false> own(g, i);
-        // i leaves its group and range: their exact bounds now cost less than meeting stale ones later
-        const int picked = __ffs(bal0) - 1;
+        // i leaves its group: the exact bound now costs less than meeting a stale one later
         const int m1 = __reduce_max_sync(FULL, lane == picked ? LAM_C : lv);
-        const int m2 = __reduce_max_sync(FULL, lane == (q1 & 31) ? m1 : b1);
-        if (lane == 0) {
-            lam[i] = LAM_C;
-            g1[q1] = m1;
-            g2[h] = m2;
-        }
-        __syncwarp();
-        // undecided strong dependants of i in the block become F
+        // undecided strong dependants of i in the block become F; in shared memory newF keeps their row of S (first
+        // entry and, from bit 16, the one past the last: below 2^16), loaded beside the measure
+        const int k_own = own.first + lane < own.last ? own.at(g, own.first + lane) : -1;
         int nf = 0;
-        for (int64_t a0 = dep.first; a0 < dep.last; a0 += 32) {
+        for (auto a0 = dep.first; a0 < dep.last; a0 += 32) {
             const int j = a0 + lane < dep.last ? dep.at(g, a0 + lane) : -1;
+            const int row = SMEM && j >= 0 ? (int)((unsigned)g.sp[j] | (unsigned)g.sp[j + 1] << 16) : j;
             const bool f = j >= 0 && lam[j] >= 0;
             const unsigned bal = __ballot_sync(FULL, f);
             if (f) {
                 const int p = nf + __popc(bal & lanemask_lt());
-                if (p < NEWF_CAP) newF[p] = j;
+                if (p < NEWF_CAP) newF[p] = row;
                 lam[j] = LAM_F;
             }
             nf += __popc(bal);
@@ -151,24 +193,21 @@ __device__ void local_picks(const LocalGraph &g, int ng1, int ng2, int32_t *lam,
             if (lane == 0) atomicOr(err, AIR_DEVERR_CAP);
             break;
         }
-        __syncwarp();
-        // every undecided point of the block in S_j of a new F point j gains one: eight lanes per j
-        for (int q = lane >> 3; q < nf; q += 4) {
-            const Row<SMEM, false> r(g, newF[q]);
-            for (int64_t a = r.first + (lane & 7); a < r.last; a += 8) {
-                const int k = r.at(g, a);
-                if (k >= 0 && lam[k] >= 0) {
-                    const int nv = atomicAdd(&lam[k], 1) + 1;
-                    atomicMax(&g1[k >> 5], nv);
-                    atomicMax(&g2[k >> 10], nv);
-                }
-            }
+        if (lane == 0) {
+            lam[i] = LAM_C;
+            g1[q1] = m1;
         }
+        __syncwarp();
         // every undecided point of the block in S_i loses one (bounds stay upper bounds, also beside the gains)
-        for (int64_t a = own.first + lane; a < own.last; a += 32) {
+        if (k_own >= 0 && lam[k_own] >= 0) atomicSub(&lam[k_own], 1);
+        for (auto a = own.first + 32 + lane; a < own.last; a += 32) {
             const int k = own.at(g, a);
             if (k >= 0 && lam[k] >= 0) atomicSub(&lam[k], 1);
         }
+        // every undecided point of the block in S_j of a new F point j gains one: eight lanes per j
+        if (!SMEM || nf <= 4) raise_rows<SMEM, 1>(g, nf, newF, lam, g1);
+        else if (nf <= 8) raise_rows<SMEM, 2>(g, nf, newF, lam, g1);
+        else raise_rows<SMEM, 4>(g, nf, newF, lam, g1);
         __syncwarp();
     }
     __syncwarp();
@@ -178,11 +217,11 @@ __global__ void __launch_bounds__(LT) local_pass_kernel(int64_t n, int64_t block
                                                         const int32_t *sci, const int64_t *strp, const int32_t *stci,
                                                         int8_t *cf, int *err) {
     extern __shared__ int32_t fsm[];
-    __shared__ int sum[2][LT];
+    __shared__ int sum[2][LT / 32];
     const int tid = threadIdx.x, lane = tid & 31;
     const int64_t lo = blockIdx.x * block, hi = lo + block < n ? lo + block : n;
-    const int m = (int)(hi - lo), ng1 = (int)(block / 32), ng2 = (int)(block / 1024), nb = (int)block;
-    int32_t *lam = fsm, *g1 = lam + block, *g2 = g1 + ng1, *newF = g2 + ng2;
+    const int m = (int)(hi - lo), ng1 = (int)(block / 32), nb = (int)block;
+    int32_t *lam = fsm, *g1 = lam + block, *newF = g1 + ng1;
     uint16_t *sp = (uint16_t *)(newF + NEWF_CAP), *tp = sp + block + 2, *se = tp + block + 2, *te = se + cap;
     // a thread's consecutive points: entries inside the block, counted, then gathered
     const int per = nb / LT, t0 = tid * per;
@@ -198,12 +237,24 @@ __global__ void __launch_bounds__(LT) local_pass_kernel(int64_t n, int64_t block
         s_sum += ns;
         t_sum += cnt;
     }
-    sum[0][tid] = s_sum;
-    sum[1][tid] = t_sum;
+    // first entries of the thread's points: an inclusive scan in the warp, then over the warps
+    int s_in = s_sum, t_in = t_sum;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int so = __shfl_up_sync(FULL, s_in, d), to = __shfl_up_sync(FULL, t_in, d);
+        if (lane >= d) {
+            s_in += so;
+            t_in += to;
+        }
+    }
+    if (lane == 31) {
+        sum[0][tid >> 5] = s_in;
+        sum[1][tid >> 5] = t_in;
+    }
     __syncthreads();
-    int s_at = 0, t_at = 0, total = 0;
-    for (int u = 0; u < LT; ++u) {                     // the same order for every thread: broadcasts
-        if (u < tid) {
+    int s_at = s_in - s_sum, t_at = t_in - t_sum, total = 0;
+    for (int u = 0; u < LT / 32; ++u) {
+        if (u < (tid >> 5)) {
             s_at += sum[0][u];
             t_at += sum[1][u];
         }
@@ -232,15 +283,10 @@ __global__ void __launch_bounds__(LT) local_pass_kernel(int64_t n, int64_t block
         if (lane == 0) g1[q] = mx;
     }
     __syncthreads();
-    for (int q = tid >> 5; q < ng2; q += LT / 32) {
-        const int mx = __reduce_max_sync(FULL, g1[q * 32 + lane]);
-        if (lane == 0) g2[q] = mx;
-    }
-    __syncthreads();
     if (tid < 32) {
         const LocalGraph g{lo, m, srp, strp, sci, stci, sp, tp, se, te};
-        if (fits) local_picks<true>(g, ng1, ng2, lam, g1, g2, newF, err);
-        else local_picks<false>(g, ng1, ng2, lam, g1, g2, newF, err);
+        if (fits) local_picks<true>(g, ng1, lam, g1, newF, err);
+        else local_picks<false>(g, ng1, lam, g1, newF, err);
     }
     __syncthreads();
     for (int t = tid; t < m; t += LT) cf[lo + t] = lam[t] == LAM_C ? CF_C : CF_F;
@@ -331,7 +377,7 @@ int air_falgout_split(int64_t n, int64_t block, const int64_t *srp, const int32_
     const int64_t nblk = (n + block - 1) / block;
     // entries of a block's graph in shared memory: six per point (HDG levels hold two to five inside a block), up to
     // what the shared memory and 16-bit row starts allow; other blocks read the graph from global memory
-    const size_t fixed = (size_t)(block + block / 32 + block / 1024 + NEWF_CAP) * sizeof(int32_t) +
+    const size_t fixed = (size_t)(block + block / 32 + NEWF_CAP) * sizeof(int32_t) +
                          2 * (size_t)(block + 2) * sizeof(uint16_t);
     if (block > 8192) return AIR_ERR_UNSUPPORTED;
     int64_t cap = (int64_t)((AIR_SMEM_OPTIN - 2048 - fixed) / (2 * sizeof(uint16_t)));   // 2048: the static arrays
