@@ -97,6 +97,7 @@ void free_level(AirLevel &L) {
     dfree(L.cf); dfree(L.cid); dfree(L.crows); dfree(L.frows);
     dfree(L.rrp); dfree(L.rci); dfree(L.rv);
     dfree(L.pcol);
+    dfree(L.fold_ci); dfree(L.fold_rows); dfree(L.fold_crows);
     air_free_sell(L.sset[0]);
     air_free_sell(L.sset[1]);
     air_free_sell(L.sr);
@@ -453,10 +454,12 @@ int air_setup_end(air_hierarchy *H, cudaStream_t s) {
                 AIR_TRY(air_build_sell(L.nc, L.crows, L.rp, L.ci, L.v, opt->precision, bf16, &L.sset[1], s));
             }
             AIR_TRY(air_build_sell(L.nc, nullptr, L.rrp, L.rci, L.rv, opt->precision, 0, &L.sr, s));
+            AIR_TRY(air_build_fold(L, opt->relax[0], s));
         }
         size_t es = f32 ? sizeof(float) : sizeof(double);
         AIR_CUDA(air_dmalloc(&L.b, (size_t)(L.n > 0 ? L.n : 1) * es));
-        AIR_CUDA(air_dmalloc(&L.x, (size_t)(L.n > 0 ? L.n : 1) * es));
+        AIR_CUDA(air_dmalloc(&L.x, (size_t)(L.n + 1) * es));
+        AIR_CUDA(cudaMemsetAsync((char *)L.x + (size_t)L.n * es, 0, es, s));       // P's value without a coarse point
         AIR_CUDA(air_dmalloc(&L.x2, (size_t)(L.n > 0 ? L.n : 1) * es));
     }
     {

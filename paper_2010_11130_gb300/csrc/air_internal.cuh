@@ -135,6 +135,10 @@ struct AirLevel {
     // SELL-32 copies for the V-cycle: the rows of A_l split by point set
     // (0 = F, 1 = C) for the relaxation sweeps, and R_l for the restriction
     Sell sset[2];
+    // the first sweep of the V-cycle (set fold_set) straight from the coarse vector x_c: columns of sset[fold_set], its
+    // rows and the other set's rows mapped through P (no coarse point: n_c, where x_c holds 0); NULL: x = P x_c first
+    int fold_set = 0;
+    int32_t *fold_ci = nullptr, *fold_rows = nullptr, *fold_crows = nullptr;
     Sell sr;
     // lanes per row of the entry-form kernels: F sweep, C sweep, restriction
     // (1: one thread per row; more: the row's entries split over that many lanes)
@@ -184,8 +188,8 @@ struct air_hierarchy {
     double *scal = nullptr;           // [0] norm, [1] estimate, ...
     double *h_est = nullptr;          // pinned host mirror of scalars
     double *xd = nullptr, *bd = nullptr;  // device b and x when the caller passes host vectors
-    // many right-hand sides (allocated on first use): per level, b, x and a
-    // compact sweep buffer of n_l x mk row-major FP64; the Krylov vectors of
+    // many right-hand sides (allocated on first use): per level, b, x and the
+    // sweeps' second vector of n_l x mk row-major FP64; the Krylov vectors of
     // the lockstep solve
     int mk = 0;
     double *mb[AIR_MAX_LEVELS] = {}, *mx[AIR_MAX_LEVELS] = {}, *mt[AIR_MAX_LEVELS] = {};
@@ -340,6 +344,7 @@ int air_build_sell(int64_t m, const int32_t *rows, const int64_t *rp, const int3
 // The block form of the same rows with block size b (2, 3, 4, 6 or 10).
 // AIR_ERR_UNSUPPORTED (out left empty, nothing else changed) when a row is not
 // whole aligned blocks plus at most its diagonal.
+int air_build_fold(AirLevel &L, char first, cudaStream_t s);
 int air_build_sell_blocks(int64_t m, const int32_t *rows, const int64_t *rp, const int32_t *ci, const double *v,
                           int precision, int b, Sell *out, cudaStream_t s);
 void air_free_sell(Sell &S);
