@@ -927,7 +927,7 @@ __global__ void fold_kernel(int64_t count, const int32_t *idx, const int32_t *pc
 // The V-cycle's first sweep (entry form, `first` = 'F' or 'C') reads x = P x_c
 // through P: its columns mapped to coarse points once, here.  That takes a launch
 // and a pass over x out of every level, and the sweep gathers from the shorter
-// vector; the sums are the same.  V-cycles: 1,536 unknowns FP64 37.3 -> 33.4 us,
+// vector; the sums are the same.  V-cycles: 6,144 unknowns FP64 37.3 -> 33.4 us,
 // 291,840 unknowns FP32 98.9 -> 92.8, 7.9 M 1316 -> 1296 us (level 0 in block form
 // still interpolates first: a block's runs of x have no coarse counterpart).
 int air_build_fold(AirLevel &L, char first, cudaStream_t s) {
