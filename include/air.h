@@ -392,7 +392,7 @@ int air_hdg_size(const air_hdg_mesh *M, const air_hdg_ref *R, int scale, int64_t
  * diagonal block of every free facet row-major (the D_b of A = D_b^{-1} S),
  * lam_dir (optional, n_facets x b) the Dirichlet trace values.  One warp per
  * element builds the local matrices by quadrature, condenses them in shared
- * memory and writes its off-diagonal blocks; one warp per facet sums the two
+ * memory and writes its off-diagonal blocks; a pass over the facets sums the two
  * diagonal contributions, inverts and scales its row.  Synchronises the
  * stream.  Errors: INVALID_ARG, CUDA, SINGULAR_COARSE (a singular element
  * matrix A_K or diagonal block). */
