@@ -7,7 +7,8 @@
 //    one row per thread in registers.  A step needs one cluster barrier: every
 //    block pushes its best pivot candidate, that row divided by its pivot and,
 //    from its owner, row k to all blocks, and every thread picks the winner for
-//    itself.  The rows' multipliers are kept by the row they belong to.
+//    itself.  One more barrier, behind the loads of the rows, comes before the
+//    first push.  The rows' multipliers are kept by the row they belong to.
 //  - pivot_rows_kernel: the panel's rows of every other column, step by step.
 //  - update_kernel, all SMs: the panel's steps on every other entry, in order,
 //    reading the old matrix through the panel's row swaps and writing the other
@@ -86,6 +87,9 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(PT) panel_kernel(Pa
     cg::cluster_group cluster = cg::this_cluster();
     const int tid = threadIdx.x, lane = tid & 31, nw = blockDim.x >> 5, rank = (int)cluster.block_rank();
     if (*(volatile int *)g.err & AIR_DEVERR_SINGULAR) return;         // an earlier panel; the same for all blocks
+    // A block's shared memory may be written by the others once it runs: all arrive here and wait below, before the
+    // first remote write.
+    cluster.barrier_arrive();
     const int64_t lo = rank * g.chunk, hi = lo + g.chunk < g.n ? lo + g.chunk : g.n;
     const double tol = 1e-14 * __longlong_as_double((long long)*g.amax);
     double a[PB];
@@ -99,6 +103,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(PT) panel_kernel(Pa
         }
     }
     int32_t id = (int32_t)(lo + tid);                  // REG: the row of the old matrix the thread holds
+    cluster.barrier_wait();
     for (int c = 0; c < g.nb; ++c) {
         const int64_t k = g.k0 + c;
         const int par = c & 1;
