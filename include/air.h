@@ -38,7 +38,7 @@ extern "C" {
 #define AIR_ERR_OOM              -3   /* device allocation failed */
 #define AIR_ERR_CUDA             -4   /* a CUDA runtime call failed */
 #define AIR_ERR_SINGULAR_COARSE  -5   /* coarsest operator singular to working precision */
-#define AIR_ERR_DEVICE_TIMEOUT   -6   /* a bounded device loop hit its iteration cap */
+#define AIR_ERR_DEVICE_TIMEOUT   -6   /* a bounded device loop or wait hit its iteration cap */
 #define AIR_ERR_COARSE_TOO_LARGE -7   /* coarsening stalled above max_dense rows */
 #define AIR_ERR_UNSUPPORTED      -8   /* option value not implemented on the GPU path */
 #define AIR_ERR_NOALLOC_LIMIT    -9   /* problem too large for the fixed workspace of
@@ -64,7 +64,7 @@ typedef struct {
                             'A' a Jacobi sweep over the F, C or all points ("FCF" by default); 'f',
                             'c', 'a' a forward Gauss-Seidel sweep (ascending point order, the
                             values already updated; Section 4 post-relaxes with "fa") over the
-                            same sets, level-scheduled (FP64 and FP32 hierarchies; the many
+                            same sets, one launch each (FP64 and FP32 hierarchies; the many
                             right-hand-side calls take 'F' and 'C' only) */
     double omega;        /* Jacobi weight */
     int max_coarse;      /* stop coarsening at or below this many rows */
@@ -148,8 +148,23 @@ int air_setup(const air_csr *A, double theta, int distance, const air_options *o
  * recursively from a zero guess, followed by the relax sweeps).  b and x are
  * device float64 vectors of length n; an F32 or BF16 hierarchy converts
  * at the finest level.  The first call captures the V-cycle into a CUDA
- * graph (replayed by later calls).  Asynchronous on stream. */
+ * graph (replayed by later calls).  Asynchronous on stream: a Gauss-Seidel
+ * wait that runs out (below) leaves NaN in x and is reported later. */
 int air_vcycle(const air_hierarchy *H, const double *b, double *x, void *stream);
+
+/* Rows of a forward Gauss-Seidel sweep wait on the device for the rows they
+ * need.  Every such wait is bounded; where one runs out the V-cycle finishes
+ * with NaN and the hierarchy keeps a mark.  air_hierarchy_status waits for the
+ * stream and returns AIR_ERR_DEVICE_TIMEOUT if the mark is set, else AIR_OK;
+ * the Krylov solves read it with their scalars, once per iteration, and return
+ * the same error.  Reading the mark clears it; a mark that air_vcycle left
+ * is reported by whichever of these calls comes next.
+ *
+ * air_set_wait_limit sets how often one value is polled before its wait counts
+ * as run out (default 2^20, about half a second; at least 1).  No call on H may
+ * be under way. */
+int air_hierarchy_status(const air_hierarchy *H, void *stream);
+int air_set_wait_limit(air_hierarchy *H, int polls);
 
 /* y = A x for device CSR A and device vectors.  Asynchronous. */
 int air_spmv(const air_csr *A, const double *x, double *y, void *stream);

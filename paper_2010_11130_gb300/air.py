@@ -28,7 +28,7 @@ EXPORTED = ["air_default_options", "air_setup", "air_vcycle", "air_spmv", "air_g
             "air_bicgstab_solve", "air_vcycle_multi", "air_bicgstab_solve_multi",
             "air_vcycle_multi_f32", "air_hdg_points", "air_hdg_size", "air_hdg_assemble",
             "air_hdg_velocity_gradient", "air_csr_transpose_scaled", "air_block_diag_apply",
-            "air_hierarchy_spmv"]
+            "air_hierarchy_spmv", "air_hierarchy_status", "air_set_wait_limit"]
 
 
 class air_csr(C.Structure):
@@ -104,6 +104,10 @@ def lib() -> C.CDLL:
     L.air_spmv.restype = C.c_int
     L.air_hierarchy_spmv.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]
     L.air_hierarchy_spmv.restype = C.c_int
+    L.air_hierarchy_status.argtypes = [C.c_void_p, C.c_void_p]
+    L.air_hierarchy_status.restype = C.c_int
+    L.air_set_wait_limit.argtypes = [C.c_void_p, C.c_int]
+    L.air_set_wait_limit.restype = C.c_int
     L.air_gmres_solve.argtypes = [C.POINTER(air_csr), C.c_void_p, C.c_void_p, C.c_void_p, C.c_double,
                                   C.c_void_p, C.POINTER(air_solve_info)]
     L.air_gmres_solve.restype = C.c_int
@@ -288,6 +292,14 @@ class Hierarchy:
         _check(lib().air_vcycle(self._h, C.c_void_p(b.data_ptr()), C.c_void_p(x.data_ptr()),
                                 C.c_void_p(_stream(stream))), "air_vcycle")
         return x
+
+    def check(self, stream=None):
+        """air_hierarchy_status: waits for the stream; raises if a V-cycle's bounded wait has run out."""
+        _check(lib().air_hierarchy_status(self._h, C.c_void_p(_stream(stream))), "air_hierarchy_status")
+
+    def set_wait_limit(self, polls: int):
+        """air_set_wait_limit: polls of one value before a Gauss-Seidel wait counts as run out."""
+        _check(lib().air_set_wait_limit(self._h, int(polls)), "air_set_wait_limit")
 
     def free(self):
         if self._h is not None and self._h.value:

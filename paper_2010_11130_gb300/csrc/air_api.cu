@@ -625,6 +625,7 @@ int air_gmres_step(AirGmres &g) {
     AIR_TRY(air_arnoldi_givens(j, m, h1, h2, sc + 4, H->Hm, H->cs, H->sn, H->gvec, sc, g.bnorm, g.s));
     AIR_TRY(air_scale_vec(n, w, w, sc + 2, 0, g.s));
     AIR_CUDA(cudaMemcpyAsync(H->h_est + 1, sc + 1, 2 * sizeof(double), cudaMemcpyDeviceToHost, g.s));
+    AIR_TRY(air_gs_fetch(H, (int *)(H->h_est + 7), g.s));
     return AIR_OK;
 }
 
@@ -632,6 +633,7 @@ int air_gmres_step(AirGmres &g) {
 // estimate meets the tolerance, on breakdown, after m steps or at max_iter.
 int air_gmres_after_step(AirGmres &g) {
     air_hierarchy *H = g.H;
+    AIR_TRY(air_gs_take(H, (const int *)(H->h_est + 7), g.s));
     ++g.it;
     g.k = g.j + 1;
     const double est = H->h_est[1], hn = H->h_est[2];
@@ -698,6 +700,11 @@ int bicgstab_impl(const AirLevel &A0, const air_hierarchy *Hc, const double *b, 
         AIR_TRY(air_reduce_partials(k, H->partials, nblk, sc, s));
         return fetch(k);
     };
+    auto dots_checked = [&]() -> int {                                  // (r, r), and the waits of the V-cycles so far
+        AIR_TRY(air_gs_fetch(H, (int *)(H->h_est + 7), s));
+        AIR_TRY(dots(r, 1, r));
+        return air_gs_take(H, (const int *)(H->h_est + 7), s);
+    };
     info->iters = 0;
     info->restarts = 0;
     info->vcycles = 0;
@@ -741,7 +748,7 @@ int bicgstab_impl(const AirLevel &A0, const air_hierarchy *Hc, const double *b, 
         info->vcycles += 2;
         rho_prev = rho;
         ++it;
-        AIR_TRY(dots(r, 1, r));
+        AIR_TRY(dots_checked());
         if (sqrt(H->h_est[0]) / bn <= rtol) {
             AIR_TRY(air_sell_spmv_f64(H->a0, x, r, b, s));                       // true residual b - A x
             AIR_TRY(dots(r, 1, r));
@@ -758,7 +765,7 @@ int bicgstab_impl(const AirLevel &A0, const air_hierarchy *Hc, const double *b, 
     }
     if (!conv) {
         AIR_TRY(air_sell_spmv_f64(H->a0, x, r, b, s));
-        AIR_TRY(dots(r, 1, r));
+        AIR_TRY(dots_checked());
         info->relres = sqrt(H->h_est[0]) / bn;
     }
     info->iters = it;
@@ -1004,6 +1011,27 @@ int air_gmres_solve(const air_csr *A, const air_hierarchy *H, const double *b, d
     AIR_CUDA(cudaMemcpyAsync(x, Hm->xd, (size_t)n * sizeof(double), cudaMemcpyDeviceToHost, s));
     AIR_CUDA(cudaStreamSynchronize(s));
     return st;
+}
+
+int air_hierarchy_status(const air_hierarchy *H, void *stream) {
+    if (!H) return AIR_ERR_INVALID_ARG;
+    cudaStream_t s = (cudaStream_t)stream;
+    int flags = 0;
+    AIR_CUDA(cudaStreamSynchronize(s));
+    AIR_TRY(air_gs_fetch(H, &flags, s));
+    AIR_CUDA(cudaStreamSynchronize(s));
+    return air_gs_take(H, &flags, s);
+}
+
+int air_set_wait_limit(air_hierarchy *H, int polls) {
+    if (!H || polls < 1) return AIR_ERR_INVALID_ARG;
+    if (polls == H->gs_polls) return AIR_OK;
+    H->gs_polls = polls;
+    if (H->gs && H->vgraph) {                  // the captured sweeps hold the old limit
+        AIR_CUDA(cudaGraphExecDestroy(H->vgraph));
+        H->vgraph = nullptr;
+    }
+    return AIR_OK;
 }
 
 int air_hierarchy_levels(const air_hierarchy *H) { return H ? H->nlev : 0; }

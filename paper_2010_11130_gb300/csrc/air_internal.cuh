@@ -168,6 +168,8 @@ struct air_hierarchy {
     float *cinv32 = nullptr;
     // device scalars and scratch
     int *d_err = nullptr;
+    bool gs = false;                  // the relaxation has Gauss-Seidel sweeps
+    int gs_polls = 1 << 20;           // polls of one value before a sweep gives up: about half a second
     unsigned long long *d_stats = nullptr;   // 8 first-pass counters: picks, refills, lines searched, long lists, cursor moves
     // SELL-32 FP64 copy of the finest operator for the GMRES matrix products
     Sell a0;
@@ -320,12 +322,19 @@ void air_free_multi(air_hierarchy *H);
 
 // gauss_seidel.cu: schedules of the forward Gauss-Seidel sweeps the relaxation
 // string asks for ('f', 'c', 'a'), built at the end of setup, and one sweep
-// xn <- GS(x) over set which (0 F, 1 C, 2 all), the other points copied; err
-// gets AIR_DEVERR_RS_CAP if a bounded wait ran out (its value is then NaN)
+// xn <- GS(x) over set which (0 F, 1 C, 2 all), the other points copied; a row
+// polls a value it waits for at most `polls` times, then takes it as NaN and
+// sets AIR_DEVERR_RS_CAP in err
 int air_gs_build(air_hierarchy *H, cudaStream_t s);
 void air_gs_free(AirLevel &L);
 template <typename T>
-int air_gs_sweep(const AirLevel &L, int which, T omega, const T *b, const T *x, T *xn, int *err, cudaStream_t s);
+int air_gs_sweep(const AirLevel &L, int which, T omega, const T *b, const T *x, T *xn, int polls, int *err,
+                 cudaStream_t s);
+// A wait that ran out in a V-cycle: fetch copies the hierarchy's error flags to the host (asynchronous), take, after
+// the stream has been synchronised, returns AIR_ERR_DEVICE_TIMEOUT if the flag was set, and clears it.  Nothing on
+// hierarchies without Gauss-Seidel sweeps.
+int air_gs_fetch(const air_hierarchy *H, int *flags, cudaStream_t s);
+int air_gs_take(const air_hierarchy *H, const int *flags, cudaStream_t s);
 
 // solve_kernels.cu
 // y = A x, or y = b - A x if b != NULL; nnz < 0 / maxrow <= 0 when unknown

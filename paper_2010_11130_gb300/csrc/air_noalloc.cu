@@ -151,7 +151,10 @@ extern "C" int air_gmres_solve_noalloc(const air_csr *A, const air_hierarchy *H,
             AIR_TRY(air_reduce_partials(1, w.partials, nblk, w.sc + 4, s));
             AIR_TRY(air_arnoldi_givens(j, m, w.h1, w.h2, w.sc + 4, w.Hm, w.cs, w.sn, w.g, w.sc, bnorm, s));
             AIR_TRY(air_scale_vec(n, wj, wj, w.sc + 2, 0, s));
+            int flags = 0;
+            AIR_TRY(air_gs_fetch(H, &flags, s));
             AIR_TRY(read_scalars(w.sc + 1, hs + 1, 2, s));
+            AIR_TRY(air_gs_take(H, &flags, s));
             ++it;
             k = j + 1;
             double est = hs[1], hn = hs[2];

@@ -18,7 +18,8 @@
 // write, so a row polls x_j itself and needs no flags and no fences.  Only
 // earlier rows are waited for, and those were taken by warps that already
 // run, so the sweep ends whatever part of its grid is resident and whatever
-// else runs beside it; polls are bounded all the same.  What bounds it is the
+// else runs beside it; polls are bounded all the same, and a wait that runs out
+// is reported by the next solve or air_hierarchy_status.  What bounds it is the
 // chain of depth groups: one hop, a store and a poll through the L2 (0.44 us
 // between two lanes) and one row's sum, takes 0.9 to 1 us, against 6 us for a
 // launch per group.  One lane per entry: with two, four or eight entries per
@@ -136,8 +137,6 @@ __global__ void gs_begin_kernel(int64_t n, const int8_t *cf, int which, const T 
         xn[i] = Slot<T>::value(in_set(cf, which, i) ? Slot<T>::PENDING : settled(x[i]));
 }
 
-constexpr int GS_POLLS = 1 << 20;         // about half a second; then the value is taken as NaN
-
 // One warp per row, one lane per entry: rows order[c K] .. order[c K + K - 1] of ticket c.  The entries' products are
 // summed in FP32 as `vl` lanes with every vl-th entry each would sum them (the order of the sets' storage), in FP64 by
 // a tree over the warp (a dependent DFMA takes 64 cycles here, an FP32 one 7).
@@ -146,7 +145,7 @@ __global__ void __launch_bounds__(128) gs_sweep_kernel(int64_t m, int K, int vl,
                                                        const int64_t *__restrict__ rp, const int32_t *__restrict__ ci,
                                                        const T *__restrict__ v, const T *__restrict__ xo, T *xn,
                                                        const T *__restrict__ b, const T *__restrict__ dinv, T omega,
-                                                       unsigned *ticket, int *err) {
+                                                       unsigned *ticket, int polls_cap, int *err) {
     using S = Slot<T>;
     const int lane = threadIdx.x & 31;
     unsigned c = 0;
@@ -168,7 +167,7 @@ __global__ void __launch_bounds__(128) gs_sweep_kernel(int64_t m, int K, int vl,
                 if (j < i) {
                     typename S::bits w = S::load(xn + j);
                     int polls = 0;
-                    while (w == S::PENDING && ++polls < GS_POLLS) w = S::load(xn + j);
+                    while (w == S::PENDING && ++polls < polls_cap) w = S::load(xn + j);
                     if (w == S::PENDING) {
                         atomicOr(err, AIR_DEVERR_RS_CAP);
                         w = S::QNAN;
@@ -277,6 +276,7 @@ int air_gs_build(air_hierarchy *H, cudaStream_t s) {
         if (*c == 'a') need[2] = true;
     }
     if (!need[0] && !need[1] && !need[2]) return AIR_OK;
+    H->gs = true;
     for (int q = 0; q + 1 < H->nlev; ++q) {
         AirLevel &L = H->lev[q];
         for (int w = 0; w < 3; ++w)
@@ -300,8 +300,22 @@ void air_gs_free(AirLevel &L) {
     L.v32 = nullptr;
 }
 
+int air_gs_fetch(const air_hierarchy *H, int *flags, cudaStream_t s) {
+    if (!H->gs) return AIR_OK;
+    AIR_CUDA(cudaMemcpyAsync(flags, H->d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    return AIR_OK;
+}
+
+int air_gs_take(const air_hierarchy *H, const int *flags, cudaStream_t s) {
+    if (!H->gs || !(*flags & AIR_DEVERR_RS_CAP)) return AIR_OK;
+    AIR_CUDA(cudaMemsetAsync(H->d_err, 0, sizeof(int), s));
+    AIR_CUDA(cudaStreamSynchronize(s));
+    return AIR_ERR_DEVICE_TIMEOUT;
+}
+
 template <typename T>
-int air_gs_sweep(const AirLevel &L, int which, T omega, const T *b, const T *x, T *xn, int *err, cudaStream_t s) {
+int air_gs_sweep(const AirLevel &L, int which, T omega, const T *b, const T *x, T *xn, int polls, int *err,
+                 cudaStream_t s) {
     const AirLevel::GsSchedule &G = L.gs[which];
     const bool f64 = std::is_same<T, double>::value;
     const T *dinv = f64 ? (const T *)L.dinv : (const T *)L.dinv32;
@@ -316,13 +330,13 @@ int air_gs_sweep(const AirLevel &L, int which, T omega, const T *b, const T *x, 
         if (warps > (double)G.m) warps = (double)G.m;
         const int K = width > most ? (width > 8.0 * most ? 8 : (int)(width / most)) : 1;
         gs_sweep_kernel<T><<<air_counted((unsigned)((warps + 3.0) / 4.0)), 128, 0, s>>>(
-            G.m, K, lanes_for(L), G.dev_rows, L.rp, L.ci, v, x, xn, b, dinv, omega, G.ticket, err);
+            G.m, K, lanes_for(L), G.dev_rows, L.rp, L.ci, v, x, xn, b, dinv, omega, G.ticket, polls, err);
     }
     AIR_LAUNCH();
     return AIR_OK;
 }
 
-template int air_gs_sweep<double>(const AirLevel &, int, double, const double *, const double *, double *, int *,
-                                  cudaStream_t);
-template int air_gs_sweep<float>(const AirLevel &, int, float, const float *, const float *, float *, int *,
+template int air_gs_sweep<double>(const AirLevel &, int, double, const double *, const double *, double *, int,
+                                  int *, cudaStream_t);
+template int air_gs_sweep<float>(const AirLevel &, int, float, const float *, const float *, float *, int, int *,
                                  cudaStream_t);

@@ -903,7 +903,7 @@ int vcycle_t(const air_hierarchy *H, const T *b0, T *x0, cudaStream_t s) {
             } else if (c == 'F' || c == 'C') {
                 jacobi_dispatch<TV, T>(A, diag, dinv, c == 'C' ? 1 : 0, omega, bl, cur, nxt, true, s);
             } else {                                   // 'f', 'c', 'a': forward Gauss-Seidel
-                AIR_TRY(air_gs_sweep<T>(A, c == 'f' ? 0 : (c == 'c' ? 1 : 2), omega, bl, cur, nxt, H->d_err, s));
+                AIR_TRY(air_gs_sweep<T>(A, c == 'f' ? 0 : (c == 'c' ? 1 : 2), omega, bl, cur, nxt, H->gs_polls, H->d_err, s));
             }
             T *t = cur;
             cur = nxt;
