@@ -79,9 +79,9 @@ struct Dims {
     static constexpr int PV = QV * NB * (1 + D * D), PF = 4 * QC * NB, PS = NB * B + B * NX;
     static constexpr int PR = PV > PF ? (PV > PS ? PV : PS) : (PF > PS ? PF : PS);
     static constexpr int WARP_DOUBLES = NB * NB + XR + PR + 4 * NF * NQF + B * B + NB + GEO;
-    // gradient: A, volume points, chunk products, facet point weights, two facet fields, Lam, mu, U, y, pivots, geometry
+    // gradient: A, volume points, chunk products, facet point weights, two facet fields, Lam, mu, U, y, F, geometry
     static constexpr int GRAD_DOUBLES =
-        NB * NB + NQ * (D + 1) + QC * NB + 4 * NF * NQF + 2 * NT + 4 * NB + GEO;
+        NB * NB + NQ * (D + 1) + QC * NB + 4 * NF * NQF + 2 * NT + 3 * NB + GEO;
     // reference integrals (doubles): volume stiffness per metric entry k <= l, then per facet and frame the
     // symmetrised trace-gradient matrix
     static constexpr int NM = D * (D + 1) / 2;
@@ -481,10 +481,10 @@ __device__ __forceinline__ void symmetric_part(const ElemArgs &a, const double *
 }
 
 // LU factors of the warp's A (N x N, row-major) with partial pivoting (ties -> smallest row), the row operations
-// applied to the NC columns of X (row stride LDX) on the way; the multipliers stay below the diagonal, rinv gets the
-// reciprocal pivots and perm (registers, lane c < N) the row swapped with row c.  Returns false if a pivot is zero.
+// applied to the NC columns of X (row stride LDX) on the way; the multipliers stay below the diagonal, perm (registers,
+// lane c < N) gets the row swapped with row c.  Returns false if a pivot is zero.
 template <int N, int NC, int LDX>
-__device__ bool warp_factor(double *A, double *X, double *rinv, int &perm) {
+__device__ bool warp_factor(double *A, double *X, int &perm) {
     const int lane = threadIdx.x & 31;
     perm = lane;
     for (int c = 0; c < N; ++c) {
@@ -512,12 +512,7 @@ __device__ bool warp_factor(double *A, double *X, double *rinv, int &perm) {
             }
             __syncwarp();
         }
-        const double piv = A[c * N + c], ri = 1.0 / piv;
-        double l = 0.0;
-        if (rr0 > c && rr0 < N) l = quotient(A[rr0 * N + c], piv, ri);
-        __syncwarp();
-        if (rr0 > c && rr0 < N) A[rr0 * N + c] = l;
-        if (lane == 0) rinv[c] = ri;
+        if (rr0 > c && rr0 < N) A[rr0 * N + c] = A[rr0 * N + c] / A[c * N + c];
         __syncwarp();
         const int wa = N - c - 1, w = wa + NC;
         if (w > 0) {
@@ -537,10 +532,10 @@ __device__ bool warp_factor(double *A, double *X, double *rinv, int &perm) {
 
 // X <- U^{-1} X for the factors of warp_factor, row by row from the last
 template <int N, int NC, int LDX>
-__device__ void warp_back_substitute(const double *A, double *X, const double *rinv) {
+__device__ void warp_back_substitute(const double *A, double *X) {
     const int lane = threadIdx.x & 31;
     for (int r = N - 1; r >= 0; --r) {
-        for (int t = lane; t < NC; t += 32) X[r * LDX + t] = quotient(X[r * LDX + t], A[r * N + r], rinv[r]);
+        for (int t = lane; t < NC; t += 32) X[r * LDX + t] = X[r * LDX + t] / A[r * N + r];
         __syncwarp();
         for (int t = lane; t < r * NC; t += 32) {
             const int rr = t / NC, cc = t % NC;
@@ -1226,7 +1221,7 @@ __global__ void __launch_bounds__(WPB * 32) velocity_gradient_kernel(ElemArgs a)
     double *sA = smem + (size_t)w * Dm::GRAD_DOUBLES;
     double *sV = sA + NB * NB, *sP = sV + NQ * (D + 1), *sW = sP + Dm::QC * NB, *sL = sW + 2 * NF * NQF,
            *sM = sL + NF * NQF, *sLam = sM + NF * NQF, *sMu = sLam + NT, *sU = sMu + NT, *sY = sU + NB, *sF = sY + NB,
-           *sR = sF + NB, *sGeo = sR + NB;
+           *sGeo = sF + NB;
     const int32_t *fr = a.frame + e * NF, *ef = a.elem_facets + e * NF;
     for (int t = lane; t < Dm::GEO; t += 32) sGeo[t] = a.geo[e * Dm::GEO + t];
     for (int t = lane; t < NT; t += 32) {
@@ -1283,15 +1278,15 @@ __global__ void __launch_bounds__(WPB * 32) velocity_gradient_kernel(ElemArgs a)
     }
     __syncwarp();
     int perm;
-    if (!warp_factor<NB, 1, 1>(sA, sU, sR, perm)) {
+    if (!warp_factor<NB, 1, 1>(sA, sU, perm)) {
         if (lane == 0) atomicOr(a.err, AIR_DEVERR_SINGULAR);
         return;
     }
-    warp_back_substitute<NB, 1, 1>(sA, sU, sR);
+    warp_back_substitute<NB, 1, 1>(sA, sU);
     // A^T y = c: U^T z = c, L^T v = z, then the row swaps undone in reverse
     double y = lane < NB ? sY[lane] : 0.0;
     for (int c = 0; c < NB; ++c) {
-        const double z = quotient(__shfl_sync(FULL, y, c), sA[c * NB + c], sR[c]);
+        const double z = __shfl_sync(FULL, y, c) / sA[c * NB + c];
         if (lane == c) y = z;
         if (lane > c && lane < NB) y -= sA[c * NB + lane] * z;
     }

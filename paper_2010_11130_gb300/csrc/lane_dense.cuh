@@ -18,12 +18,6 @@ __device__ __forceinline__ unsigned long long magnitude_key(double x) {
     return b > 0x7ff0000000000000ull ? 0ull : b + 1ull;
 }
 
-// x / p from r = 1 / p: the product corrected once, within an ulp of the division at a third of its FP64 work
-__device__ __forceinline__ double quotient(double x, double p, double r) {
-    const double q = x * r;
-    return fma(fma(-q, p, x), r, q);
-}
-
 // Copies the blocks first .. first + count - 1 (count <= 32) of src (b x b row-major each, transposed when tr) into
 // the warp's layout; the lanes past count get the identity.
 __device__ __forceinline__ void lane_load_blocks(const double *src, int64_t first, int count, int b, bool tr, double *m) {
