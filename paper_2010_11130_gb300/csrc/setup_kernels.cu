@@ -1140,7 +1140,8 @@ __global__ void rap_terms_kernel(int64_t nc, const int64_t *rrp, const int32_t *
 // the places are listed by coarse column, ordered by j within one (every place
 // counts the smaller ones of its column), every coarse column finds its position
 // in the row by counting the smaller ones, and one lane per coarse column sums its
-// places in ascending j.
+// places in ascending j.  Where a row or a column is long, its entries are sorted
+// instead of counted against one another.
 // COUNT: the distinct coarse columns of the terms, from one table.
 // What bounds it: shared-memory latency and instructions, 16 to 24 warps per SM.
 // All levels at 2.3 M unknowns: count 1.7 ms, fill 5.6 ms.  A bitonic sort of all
@@ -1164,6 +1165,52 @@ __device__ __forceinline__ int rap_insert(int32_t *keys, int bits, int32_t key, 
         h = (h + 1) & mask;
     }
     return -1;
+}
+
+// More coarse columns in a row, or places in a column, than this are sorted.  Counting the smaller ones takes n^2 / 32
+// steps of a warp, sorting about n log^2 n / 128 of six times the length: the two meet between 100 and 200.
+constexpr int RAP_RANK = 256;
+
+// Orders idx[0 .. n) by key[idx], distinct keys, one warp: Batcher's merge exchange, which takes any n (Knuth, The Art
+// of Computer Programming, vol. 3, Algorithm 5.2.2M).  The comparisons of a pass touch disjoint pairs, SORT_U of them
+// in flight.
+template <typename I>
+__device__ void warp_sort(I *idx, int n, const int32_t *key) {
+    constexpr int SORT_U = 4;
+    const int lane = threadIdx.x & 31;
+    if (n < 2) return;
+    const int top = 1 << (31 - __clz(n - 1));
+    for (int p = top; p > 0; p >>= 1) {
+        int d = p, r = 0;
+        for (int q = top;; q >>= 1) {
+            // pairs (i, i + d) with i & p == r, i + d < n; the k-th of them
+            for (int k0 = lane; ((k0 & -p) << 1 | (k0 & (p - 1)) | r) < n - d; k0 += 32 * SORT_U) {
+                I a[SORT_U], b[SORT_U];
+                bool swap[SORT_U];
+#pragma unroll
+                for (int u = 0; u < SORT_U; ++u) {
+                    const int k = k0 + 32 * u, i = (k & -p) << 1 | (k & (p - 1)) | r;
+                    swap[u] = i < n - d;
+                    a[u] = swap[u] ? idx[i] : (I)0;
+                    b[u] = swap[u] ? idx[i + d] : (I)0;
+                }
+#pragma unroll
+                for (int u = 0; u < SORT_U; ++u) swap[u] = swap[u] && key[a[u]] > key[b[u]];
+#pragma unroll
+                for (int u = 0; u < SORT_U; ++u) {
+                    const int k = k0 + 32 * u, i = (k & -p) << 1 | (k & (p - 1)) | r;
+                    if (swap[u]) {
+                        idx[i] = b[u];
+                        idx[i + d] = a[u];
+                    }
+                }
+            }
+            __syncwarp();
+            if (q == p) break;
+            d = q - p;
+            r = p;
+        }
+    }
 }
 
 template <bool FILL, bool GMEM>
@@ -1270,6 +1317,7 @@ __global__ void rap_kernel(int64_t nrows, const int32_t *rows, const int64_t *rr
         }
         __syncwarp();
         int total = 0;
+        bool large = false;                             // a column of more than RAP_RANK places
         for (int x0 = 0; x0 < nj; x0 += 32) {           // first places of the columns
             const int at = x0 + lane < nj ? (int)slot[x0 + lane] : -1;
             const int c = at >= 0 ? (int)seg[at] : 0;
@@ -1281,8 +1329,11 @@ __global__ void rap_kernel(int64_t nrows, const int32_t *rows, const int64_t *rr
             }
             if (at >= 0) seg[at] = (Pair)(total + sum - c) << SH | (Pair)c;
             total += __shfl_sync(FULL, sum, 31);
+            large |= c > RAP_RANK;
         }
+        large = __any_sync(FULL, large);
         __syncwarp();
+        if (nj > RAP_RANK) warp_sort(slot, nj, jkey);
         for (int p = lane; p < n; p += 32) {            // by column, in order of arrival
             const Pair a = pair[p];
             if (a != NONE) list[(int)(seg[(int)(a >> SH)] >> SH) + (int)(a & LOW)] = (Place)p;
@@ -1293,6 +1344,10 @@ __global__ void rap_kernel(int64_t nrows, const int32_t *rows, const int64_t *rr
             if (a == NONE) continue;
             const Pair sg = seg[(int)(a >> SH)];
             const int q0 = (int)(sg >> SH), q1 = q0 + (int)(sg & LOW);
+            if (q1 - q0 > RAP_RANK) {                   // sorted below
+                pair[p] = NONE;
+                continue;
+            }
             const int32_t j = dj[p];
             int at = q0;
             for (int q = q0; q < q1; ++q) at += dj[list[q]] < j ? 1 : 0;
@@ -1302,12 +1357,22 @@ __global__ void rap_kernel(int64_t nrows, const int32_t *rows, const int64_t *rr
         for (int p = lane; p < n; p += 32)
             if (pair[p] != NONE) list[(int)pair[p]] = (Place)p;
         __syncwarp();
+        for (int x0 = 0; large && x0 < nj; x0 += 32) {
+            const Pair sg = x0 + lane < nj ? seg[slot[x0 + lane]] : 0;
+            for (unsigned bal = __ballot_sync(FULL, (int)(sg & LOW) > RAP_RANK); bal; bal &= bal - 1) {
+                const Pair g = __shfl_sync(FULL, sg, __ffs(bal) - 1);
+                warp_sort(list + (int)(g >> SH), (int)(g & LOW), dj);
+            }
+        }
         const int64_t out = acrp[t];
         for (int x = lane; x < nj; x += 32) {
             const int at = slot[x];
             const int32_t J = jkey[at];
-            int rank = 0;
-            for (int y = 0; y < nj; ++y) rank += jkey[slot[y]] < J ? 1 : 0;
+            int rank = x;
+            if (nj <= RAP_RANK) {
+                rank = 0;
+                for (int y = 0; y < nj; ++y) rank += jkey[slot[y]] < J ? 1 : 0;
+            }
             const int q0 = (int)(seg[at] >> SH), q1 = q0 + (int)(seg[at] & LOW);
             double acc = 0.0;
             for (int q = q0; q < q1; ++q) acc = __dadd_rn(acc, dval[list[q]]);
@@ -1667,8 +1732,8 @@ int air_rap(const AirLevel &L, int64_t *acrp, int32_t *acci, double *acv, int32_
             int32_t max_terms, const int32_t *terms, int *d_err, cudaStream_t s) {
     int bits = 5;
     while ((1 << bits) < 2 * (max_terms > 1 ? max_terms : 1)) ++bits;
-    constexpr int kSmemBits = 13;                 // 8192 slots, 160 KB: the largest shared table
-    constexpr int kMinBits = 9;                   // 512 slots, 10 KB: 16 warps per SM
+    constexpr int kSmemBits = 13;                 // 8192 slots, 112 KB for the fill: the largest shared table
+    constexpr int kMinBits = 9;                   // 512 slots, 7 KB for the fill: 24 warps per SM
     auto launch = [&](int64_t nrows, const int32_t *rows, int b) {
         const bool gmem = b > kSmemBits;
         return fill ? rap_launch<true>(L, nrows, rows, b, gmem, nullptr, acrp, acci, acv, d_err, s)
