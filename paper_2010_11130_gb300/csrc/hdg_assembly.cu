@@ -545,12 +545,18 @@ __device__ void warp_back_substitute(const double *A, double *X) {
     }
 }
 
-// The assembled system keeps its bits whatever the arrangement of this kernel:
-// FP32 hierarchies built on it would turn the last bit of an entry into a
-// difference of an FP32 rounding.  So every entry is evaluated with the
-// operations, written as intrinsics, that its plain expression (in the comments
-// below) has always compiled to for each D and P, which products are fused
-// included, and summed over the points in their order; what entries share
+// The assembled system keeps the bits it had when every entry was evaluated on
+// its own.  That is a choice: solutions and V-cycles of an FP32 hierarchy stay
+// comparable bit by bit between versions.  Accuracy does not ask for it: with the
+// sums rearranged freely the entries' error against 64 bits was the same, one
+// FP32 V-cycle moved by 1.6e-9 (its own error is 2e-7), and the assembly took 8.9
+// and 14.6 ms instead of 27.0 (82,944 elements, p = 2) and 51.1 ms (29,478
+// elements, p = 3).  So every entry is
+// evaluated with the operations of its plain expression (in the comments below),
+// written as intrinsics, and summed over the points in their order.  Which of an
+// entry's products are fused differs with D and P (the conditions on them
+// below); it was found by comparing outputs with the plain form and means nothing
+// in the mathematics.  What entries share
 // (products of one point's weight with one basis function, the gradient in the
 // flow's direction) is computed once and kept in shared memory, and terms
 // that vanish for every point (a monomial's gradient has few components) are
@@ -1208,7 +1214,7 @@ __global__ void spread_dirichlet_kernel(int64_t F, int B, const int8_t *kind, co
 // at the points the derivative is
 //   sum_facet W n_m [ (1 + s)/2 (y u + u mu - neu lam mu) + (1 - s)/2 (y lam + lam mu) ]
 //   - sum_volume W (Jinv e_m).grad_hat(y) u,    s = sign(a_hat_n), 0 on the kink.
-// 48,000 elements, D = 3, p = 2: 3.2 ms (61.9 ms when A, B, C, D and their
+// 48,000 elements, D = 3, p = 2: 3.7 ms (61.9 ms when A, B, C, D and their
 // derivatives were formed and two factorisations made).
 template <int D, int P>
 __global__ void __launch_bounds__(WPB * 32) velocity_gradient_kernel(ElemArgs a) {
