@@ -164,12 +164,17 @@ def vcycle_bytes(H, wbytes, diag_bytes=0):
     Per non-coarsest level (n rows, nnz z = z_F + z_C, R with nnz_R entries,
     n_C coarse points, w = value bytes, x = vector element bytes):
       restriction     nnz_R (w+4) + 8 n_C + x n + x n_C
-      interpolation   4 n (P's columns) + x n_C + x n
+      interpolation   4 n (P's columns) + x n_C + x n, on a level in the block
+                      form only
       sweep over a point set S of m_S rows (F, C, F), from one full vector
       into the other: the set's matrix, 4 B of row index for every row (the
       set's rows and the copied rows of the other set), b and 1/a_ii of the
       set, the old vector read and the new one written in full:
                       mat(z_S, m_S) + 4 n + 2 x m_S + 2 x n
+      first sweep of a level in the entry form, which reads the coarse vector
+      through P (columns and rows mapped to coarse points at setup): 4 n more
+      of row index, and the coarse vector in place of the old one:
+                      mat(z_F, m_F) + 8 n + 2 x m_F + x n_C + x n
     mat(z, m) = z (w+4) in the entry form; a level stored in the block form
     (facet blocks of b) reads (z - m) w + 4 (z - m) / b + x m instead (the
     standalone diagonal one per row, in the vector type).  coarsest: x n_L^2 +
@@ -207,7 +212,7 @@ def vcycle_bytes(H, wbytes, diag_bytes=0):
         def sweep(z, m):
             return mat(z, m) + 4 * n + 2 * x * m + 2 * x * n + diag_bytes * m
         total += inf.nnz_r * (w + 4) + 8 * nc + x * n + x * nc
-        total += 4 * n + x * nc + x * n
+        total += 4 * n + x * nc + (x * n if bsz else -x * n)     # P x_c and its first reading, or the reading alone
         total += sweep(zf, nf) + sweep(zc, nc) + sweep(zf, nf)
     return total
 
