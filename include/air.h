@@ -139,6 +139,11 @@ void air_default_options(air_options *opt);
  * A's pointers as its finest level: the caller must keep A alive and
  * unchanged until air_free.  A host A is copied to the device.
  * Synchronises the stream (level sizes are read back).
+ * When relax begins with 'F' or 'C', every level in the entry form also keeps
+ * that set's column indices and the row numbers mapped through P (4 bytes per
+ * stored entry of the set and 4 per row; 0.8 GB for 8 million rows of 37
+ * entries), so that its first sweep reads the coarse vector; where
+ * they do not fit, the V-cycle interpolates first.
  * Errors: INVALID_ARG, CSR_MALFORMED (validate = 1), OOM, CUDA,
  * DEVICE_TIMEOUT, COARSE_TOO_LARGE, SINGULAR_COARSE, UNSUPPORTED. */
 int air_setup(const air_csr *A, double theta, int distance, const air_options *opt,
@@ -191,8 +196,9 @@ int air_bicgstab_solve(const air_csr *A, const air_hierarchy *H, const double *b
 
 /* Many right-hand sides through one hierarchy.  b and x are device arrays
  * of n x k doubles, row-major (the k values of row i are contiguous), k in
- * 1 .. 32.  The matrix traffic of a V-cycle is shared by the k systems: one
- * warp per matrix row, one lane per system.
+ * 1 .. 32.  The matrix traffic of a V-cycle is shared by the k systems: a
+ * group of lanes per matrix row, up to 16 bytes of systems per lane.  The first
+ * call with a k allocates three arrays of n_l x k doubles per level.
  *
  * air_vcycle_multi: x = M^{-1} b column by column, the FP64 V-cycle of H
  * (whatever H's storage precision), summed in the same order as air_vcycle's

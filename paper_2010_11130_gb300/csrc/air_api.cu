@@ -454,7 +454,6 @@ int air_setup_end(air_hierarchy *H, cudaStream_t s) {
                 AIR_TRY(air_build_sell(L.nc, L.crows, L.rp, L.ci, L.v, opt->precision, bf16, &L.sset[1], s));
             }
             AIR_TRY(air_build_sell(L.nc, nullptr, L.rrp, L.rci, L.rv, opt->precision, 0, &L.sr, s));
-            AIR_TRY(air_build_fold(L, opt->relax[0], s));
         }
         size_t es = f32 ? sizeof(float) : sizeof(double);
         AIR_CUDA(air_dmalloc(&L.b, (size_t)(L.n > 0 ? L.n : 1) * es));
@@ -479,6 +478,8 @@ int air_setup_end(air_hierarchy *H, cudaStream_t s) {
     }
     AIR_TRY(air_tune_lanes(H, opt->autotune, s));
     AIR_TRY(air_gs_build(H, s));
+    // last: the V-cycle does without it where there is no room, so nothing that setup needs may come after it
+    for (int q = 0; q + 1 < H->nlev; ++q) AIR_TRY(air_build_fold(H->lev[q], opt->relax[0], s));
     AIR_CUDA(cudaStreamSynchronize(s));
     return AIR_OK;
 }

@@ -1215,9 +1215,10 @@ int lanes_rule(const Sell &S) {
     return L;
 }
 
-// Times the candidate lanes per row on the launch the V-cycle makes: a sweep
-// (into the full vector y, with the other point set's rows copied, `other`)
-// or a restriction.
+// Times the candidate lanes per row on a launch like the V-cycle's: a sweep from
+// one full vector into the other (y, with the other point set's rows copied,
+// `other`) or a restriction.  The first sweep of a level, which gathers from the
+// shorter coarse vector, takes the lanes found for the set's other sweeps.
 template <typename TV, typename T>
 int tune_set(const AirLevel &Lv, const Sell &S, const Sell *other, bool jacobi, const T *x, const T *b, T *y,
              const T *dinv, const T *diag, int *out, cudaStream_t s) {
