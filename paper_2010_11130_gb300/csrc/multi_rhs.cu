@@ -15,7 +15,8 @@
 // at once (k = 32, FP32).  Four gathered rows in flight and 64 registers (32
 // warps per SM) were the best of 2, 4, 8 rows and 3 to 6 blocks per SM.  571,200
 // unknowns, 36 entries per row, k = 32, FP32: V-cycle 1968 -> 1090 us, the sweeps
-// and their copies 1575 -> 950 us.
+// and their copies 1575 -> 950 us.  More than 16 systems in FP64, or of a k that is
+// no multiple of four, keep a warp per row (csr_wide_kernel).
 //
 // Every kernel sums a row in the CSR entry order with fused multiply-adds,
 // like the single-right-hand-side SELL kernels, so column j of the result is
@@ -160,23 +161,89 @@ __global__ void __launch_bounds__(256, 4) csr_multi_kernel(MultiArgs<T> a) {
     *(P *)(a.Y + at) = acc;
 }
 
+// The same with one warp per row and one system per lane, for more than 16 systems in FP64 or without 16-byte packs.
+// Groups of lanes gain nothing there: in FP64 the kernel above pads the shorter of the rows that share a warp with whole
+// instructions, and with one or two values per lane it has little of wider loads but only half the warps.  Bound: FP64
+// issue in FP64, the latency of the gathered rows of X in FP32, so 32 registers and every warp slot in use.  The rows
+// that a sweep copies go CR to a warp.  3.3 M unknowns, V-cycle: FP64 k = 17 and 32 26.3 and 25.7 -> 22.1 and 22.4 ms,
+// FP32 k = 17 and 31 11.9 and 12.1 -> 9.0 and 9.5 ms (with 40 registers 12.5 and 13.6, with one copied row 13.1 and 14.1).
+constexpr int CR = 4;
+
+template <int MODE, typename T>
+__global__ void __launch_bounds__(256, 8) csr_wide_kernel(MultiArgs<T> a) {
+    const int lane = threadIdx.x & 31;
+    const bool on = lane < a.k;
+    dep_launch();
+    if (MODE == MR_JACOBI && (int64_t)blockIdx.x >= a.sweep_blocks) {
+        const int64_t p = (((int64_t)blockIdx.x - a.sweep_blocks) * blockDim.x + threadIdx.x) / 32 * CR;
+        int32_t r[CR];
+#pragma unroll
+        for (int u = 0; u < CR; ++u) r[u] = on && p + u < a.mc ? a.crows[p + u] : -1;
+        dep_wait();
+        T x[CR];
+#pragma unroll
+        for (int u = 0; u < CR; ++u) x[u] = r[u] >= 0 ? a.X[(int64_t)r[u] * a.k + lane] : (T)0;
+#pragma unroll
+        for (int u = 0; u < CR; ++u)
+            if (r[u] >= 0) a.Y[(int64_t)r[u] * a.k + lane] = x[u];
+        return;
+    }
+    const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
+    if (p >= a.m) {                                              // a whole warp
+        dep_wait();
+        return;
+    }
+    const int64_t row = a.rows ? (int64_t)a.rows[p] : p;
+    const int64_t e0 = a.rp[row], e1 = a.rp[row + 1];
+    dep_wait();
+    T acc = 0;
+    for (int64_t base = e0; base < e1; base += 32) {
+        const int64_t e = base + lane;
+        const int32_t ce = e < e1 ? a.ci[e] : 0;
+        const T ve = e < e1 ? a.v[e] : (T)0;
+        const int cnt = (int)(e1 - base < 32 ? e1 - base : 32);
+        for (int t = 0; t < cnt; ++t) {
+            const int32_t c = __shfl_sync(FULL, ce, t);
+            const T w = __shfl_sync(FULL, ve, t);
+            if (on) acc += w * a.X[(int64_t)c * a.k + lane];
+        }
+    }
+    if (!on) return;
+    const int64_t at = row * a.k + lane;
+    if (MODE == MR_SPMV) a.Y[at] = acc;
+    else if (MODE == MR_RESID) a.Y[at] = a.B[at] - acc;
+    else a.Y[at] = a.X[at] + a.omega * (a.B[at] - acc) * a.dinv[row];
+}
+
+// X = P X_c; a group of 32 lanes takes four rows, so that enough of them are in flight
+template <int G>
+constexpr int interp_rows = G == 32 ? 4 : 1;
+
 template <typename T, int V, int G>
 __global__ void __launch_bounds__(256) interp_multi_kernel(int64_t n, const int32_t *pcol, int k, const T *XC, T *X) {
     using P = Pack<T, V>;
+    constexpr int R = interp_rows<G>;
     const int gl = threadIdx.x % G;
-    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G * R;
     dep_launch();
     if (i >= n || gl * V >= k) {
         dep_wait();
         return;
     }
-    const int32_t pc = pcol[i];
-    dep_wait();
-    P x;
+    int32_t pc[R];
 #pragma unroll
-    for (int u = 0; u < V; ++u) x.v[u] = 0;
-    if (pc >= 0) x = *(const P *)(XC + (int64_t)pc * k + gl * V);
-    *(P *)(X + i * k + gl * V) = x;
+    for (int u = 0; u < R; ++u) pc[u] = i + u < n ? pcol[i + u] : -1;
+    dep_wait();
+    P x[R];
+#pragma unroll
+    for (int u = 0; u < R; ++u) {
+#pragma unroll
+        for (int v = 0; v < V; ++v) x[u].v[v] = 0;
+        if (pc[u] >= 0) x[u] = *(const P *)(XC + (int64_t)pc[u] * k + gl * V);
+    }
+#pragma unroll
+    for (int u = 0; u < R; ++u)
+        if (i + u < n) *(P *)(X + (i + u) * k + gl * V) = x[u];
 }
 
 // X = Cinv B on the coarsest level (Cinv row-major m x m), one warp per row, 32 rows of B in flight
@@ -299,9 +366,14 @@ void csr_multi(const MultiArgs<T> &a0, bool dependent, cudaStream_t s) {
     if (a0.m <= 0 && a0.mc <= 0) return;
     with_pack<T>(a0.k, pack_of<T>(a0.k, {a0.X, a0.Y, a0.B}), [&](auto v, auto g) {
         MultiArgs<T> a = a0;
-        a.sweep_blocks = (a.m * g() + 255) / 256;
-        const int64_t blocks = a.sweep_blocks + (MODE == MR_JACOBI ? (a.mc * g() + 255) / 256 : 0);
-        const auto kernel = csr_multi_kernel<MODE, T, v(), g()>;
+        constexpr bool wide = v() * g() == MK && (sizeof(T) == 8 || v() < 4);     // more than 16 systems
+        constexpr int lanes = wide ? 32 : g(), copied = wide ? CR : 1;
+        a.sweep_blocks = (a.m * lanes + 255) / 256;
+        const int64_t blocks =
+            a.sweep_blocks + (MODE == MR_JACOBI ? (a.mc * lanes + 256 * copied - 1) / (256 * copied) : 0);
+        void (*kernel)(MultiArgs<T>);
+        if constexpr (wide) kernel = csr_wide_kernel<MODE, T>;
+        else kernel = csr_multi_kernel<MODE, T, v(), g()>;
         if (dependent) launch_dependent(kernel, (unsigned)blocks, 256, s, a);
         else kernel<<<air_counted((unsigned)blocks), 256, 0, s>>>(a);
     });
@@ -419,8 +491,9 @@ int vcycle_multi_t(air_hierarchy *H, int k, const T *b0, T *x0, cudaStream_t s) 
         // P x_c starts in whichever vector makes the last sweep end in out
         T *cur = ns % 2 == 1 ? alt : out, *nxt = ns % 2 == 1 ? out : alt;
         with_pack<T>(k, pack_of<T>(k, {xc, cur}), [&](auto v, auto g) {
-            launch_dependent(interp_multi_kernel<T, v(), g()>, (unsigned)((A.n * g() + 255) / 256), 256, s, A.n, A.pcol,
-                             k, xc, cur);
+            constexpr int per = 256 / g() * interp_rows<g()>;
+            launch_dependent(interp_multi_kernel<T, v(), g()>, (unsigned)((A.n + per - 1) / per), 256, s, A.n, A.pcol, k,
+                             xc, cur);
         });
         for (int q = 0; q < ns; ++q) {
             const bool c = relax[q] == 'C';
