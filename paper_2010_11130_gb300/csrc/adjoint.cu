@@ -207,28 +207,33 @@ __global__ void __launch_bounds__(128) block_scale_t_kernel(int64_t nblk, int b,
     }
 }
 
-// y_k = op(D_k) x_k over the b-blocks: op 0 D, 1 D^T, 2 D^{-1}, 3 D^{-T}; 32 blocks per warp, the inverses one block
-// per lane.  x is read before y is written, so that they may be the same vector.
-__global__ void __launch_bounds__(32) block_apply_kernel(int64_t nblk, int b, const double *diag, int op,
+// y_k = op(D_k) x_k over the b-blocks: op 0 D, 1 D^T, 2 D^{-1}, 3 D^{-T}.  x is read before y is written, so that they
+// may be the same vector.  A group of b lanes per block, a lane per row, 32 / b blocks per warp.  Bound: the blocks'
+// bytes without an inverse, FP64 issue with one; whole calls with their synchronisation, blocks of 10: 300,000 of them
+// 104 us and 1.05 ms (inverse), 1,000 of them 43 and 62 us.  One block per lane, through shared memory, took 698 us and
+// 1.73 ms, 82 and 185 us; one warp per block 266 us and 7.2 ms, 45 and 82 us.
+template <bool INVERT>
+__global__ void __launch_bounds__(128) block_rows_kernel(int64_t nblk, int b, const double *diag, int op,
                                                          const double *x, double *y, int *err) {
     extern __shared__ double bsm[];
-    const int lane = threadIdx.x;
-    const int64_t first = (int64_t)blockIdx.x * 32;
-    const int count = nblk - first < 32 ? (int)(nblk - first) : 32;
-    double *sx = bsm + b * b * LANE_LD;
-    lane_load_blocks(diag, first, count, b, op == 1 || op == 3, bsm);
-    for (int t = lane; t < count * b; t += 32) sx[(t % b) * LANE_LD + t / b] = x[first * b + t];
-    __syncwarp();
-    if (op >= 2) {
-        if (lane < count && !lane_invert(bsm + lane, b)) atomicOr(err, AIR_DEVERR_SINGULAR);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, per = 32 / b, g = lane / b, i = lane % b, bb = b * b;
+    const int64_t k = ((int64_t)blockIdx.x * 4 + w) * per + g;
+    const bool on = g < per && k < nblk;
+    const double *D = diag + (on ? k * bb : 0);
+    double v = 0.0;
+    if (INVERT) {
+        double *m = bsm + (w * per + (on ? g : 0)) * (bb + b), *f = m + bb;
+        if (on)
+            for (int t = i; t < bb; t += b) m[op == 3 ? t % b * b + t / b : t] = D[t];
         __syncwarp();
+        if (!group_invert(m, f, b, on ? i : b) && on) atomicOr(err, AIR_DEVERR_SINGULAR);
+        if (on)
+            for (int j = 0; j < b; ++j) v += m[i * b + j] * x[k * b + j];
+    } else if (on) {
+        for (int j = 0; j < b; ++j) v += D[op == 1 ? j * b + i : i * b + j] * x[k * b + j];
     }
-    for (int t = lane; t < count * b; t += 32) {
-        const int k = t / b, i = t % b;
-        double v = 0.0;
-        for (int j = 0; j < b; ++j) v += bsm[(i * b + j) * LANE_LD + k] * sx[j * LANE_LD + k];
-        y[first * b + t] = v;
-    }
+    __syncwarp();
+    if (on) y[k * b + i] = v;
 }
 
 }  // namespace
@@ -283,8 +288,13 @@ int air_block_scale_transpose_impl(int64_t n, int b, const double *diag, const i
 int air_block_apply_impl(int64_t nblk, int b, const double *diag, int op, const double *x, double *y, int *d_err,
                          cudaStream_t s) {
     if (nblk <= 0) return AIR_OK;
-    block_apply_kernel<<<air_counted((unsigned)((nblk + 31) / 32)), 32, (b * b + b) * LANE_LD * sizeof(double), s>>>(
-        nblk, b, diag, op, x, y, d_err);
+    const int per = 4 * (32 / b);
+    const unsigned groups = (unsigned)((nblk + per - 1) / per);
+    if (op < 2)
+        block_rows_kernel<false><<<air_counted(groups), 128, 0, s>>>(nblk, b, diag, op, x, y, d_err);
+    else
+        block_rows_kernel<true><<<air_counted(groups), 128, per * (b * b + b) * sizeof(double), s>>>(nblk, b, diag, op, x,
+                                                                                                    y, d_err);
     AIR_LAUNCH();
     return AIR_OK;
 }

@@ -42,7 +42,8 @@ __device__ __forceinline__ int lane_pivot(const double *m, int b, int c) {
 }
 
 // Inverts the lane's matrix in place (m points at the lane's first entry) by Gauss-Jordan with partial pivoting: the
-// operations, in order, of the elimination of [M | I] (row / pivot, then fma(-f, row, other row)).  b <= 11.  Returns false, and leaves garbage, if a pivot is zero.
+// operations, in order, of the elimination of [M | I] (row / pivot, then fma(-f, row, other row)).  b <= 11.  Returns
+// false, and leaves garbage, if a pivot is zero.
 __device__ __forceinline__ bool lane_invert(double *m, int b) {
     unsigned long long perm = 0ull;                  // 4 bits per column
     for (int c = 0; c < b; ++c) {
@@ -76,4 +77,49 @@ __device__ __forceinline__ bool lane_invert(double *m, int b) {
         }
     }
     return true;
+}
+
+// The same inverse by a group of b lanes, lane j (of the group) keeping column j; m is the group's matrix, row-major, and
+// f b doubles of its own, both in shared memory.  Every lane of the warp calls it, those without a matrix with j >= b.
+// The operations on an entry, and their order, are lane_invert's; a step is a chain of b of them instead of b^2, and the
+// divisions of a row are one instruction either way.
+__device__ __forceinline__ bool group_invert(double *m, double *f, int b, int j) {
+    unsigned long long perm = 0ull;
+    bool ok = true;
+    for (int c = 0; c < b; ++c) {
+        unsigned long long best = 1ull;
+        int r = -1;
+        for (int rr = c; rr < b; ++rr) {
+            const unsigned long long k = magnitude_key(m[rr * b + c]);
+            if (k > best) { best = k; r = rr; }
+        }
+        ok = ok && r >= 0;
+        __syncwarp();
+        if (ok && j < b && r != c) {
+            const double x = m[c * b + j];
+            m[c * b + j] = m[r * b + j];
+            m[r * b + j] = x;
+        }
+        if (ok) perm |= (unsigned long long)r << (4 * c);
+        __syncwarp();
+        if (j < b) f[j] = m[j * b + c];
+        __syncwarp();
+        if (ok && j < b) {
+            const double v = __ddiv_rn(j == c ? 1.0 : m[c * b + j], f[c]);
+            m[c * b + j] = v;
+            for (int rr = 0; rr < b; ++rr)
+                if (rr != c) m[rr * b + j] = __fma_rn(-f[rr], v, j == c ? 0.0 : m[rr * b + j]);
+        }
+        __syncwarp();
+    }
+    for (int c = b - 1; c >= 0; --c) {
+        const int r = (int)(perm >> (4 * c)) & 15;
+        if (ok && j < b && r != c) {
+            const double x = m[j * b + c];
+            m[j * b + c] = m[j * b + r];
+            m[j * b + r] = x;
+        }
+    }
+    __syncwarp();
+    return ok;
 }
