@@ -90,6 +90,9 @@ struct RowArgs {
     const TX *x;        // input vector (gathered)
     TX *y;              // output
     const TX *b;        // optional (y = b - A x)
+#ifdef DIAG
+    const TX *diag;
+#endif
 };
 
 template <int VL, int U, typename TV, typename TX>
@@ -116,8 +119,14 @@ __global__ void __launch_bounds__(256) row_kernel(RowArgs<TV, TX> a) {
             }
 #pragma unroll
             for (int u = 0; u < U; ++u) acc += to_acc<A, TV>(vals[u]) * (A)__ldg(a.x + cols[u]);
+#ifdef UNR
+#pragma unroll UNR
+#endif
             for (int64_t e = rs + lane + (int64_t)U * VL; e < re; e += VL)
                 acc += to_acc<A, TV>(a.v[e]) * (A)a.x[a.ci[e]];
+#ifdef DIAG
+            if (a.diag && lane == 0) acc += (A)a.diag[row] * (A)a.x[row];
+#endif
         }
         acc = seg_sum<VL, A>(acc);
         if (lane == 0 && valid) a.y[row] = a.b ? (TX)((A)a.b[row] - acc) : (TX)acc;
@@ -457,11 +466,16 @@ struct BSellArgs {
 // b entries of x as runs of consecutive elements.  FP32 takes one block at a
 // time in 32 registers with every warp slot in use (V-cycle at 7.9 M unknowns
 // 1327 us, two blocks 1349, three 1364); FP64 two, its row product is bound by
-// FP64 issue.
+// FP64 issue.  What such a kernel needs is an even number of blocks on every SM,
+// and blocks that start while the grid before them still runs settle where room
+// happens to be: FP64 neither lets its successor start early nor, in the sweeps,
+// starts early itself (FP64 V-cycle of 70,800 and of 60,160 unknowns with blocks of
+// 6 and of 10: 113 and 120 us, 128 and 140 with early starts, 123 and 129 without
+// dependent launches anywhere; matrix product of the latter 9.9, 27.4, 12.3 us).
 template <int B, bool PAIRS, typename TV, typename TX, int MODE>
 __global__ void __launch_bounds__(256) bsell_kernel(BSellArgs<TV, TX> a) {
     using A = typename Acc<TX>::type;
-    dep_launch();
+    if (sizeof(TX) == 4) dep_launch();
     if (MODE == ROW_JACOBI && (int64_t)blockIdx.x >= a.sweep_blocks) {
         copy_rows(a.mc, a.crows, nullptr, a.x, a.y, (int64_t)blockIdx.x - a.sweep_blocks);
         return;
@@ -520,7 +534,9 @@ void bsell_launch_b(const BSellArgs<TV, TX> &a0, bool pairs, cudaStream_t s) {
     BSellArgs<TV, TX> a = a0;
     a.sweep_blocks = (a.m + 255) / 256;
     const unsigned g = (unsigned)(a.sweep_blocks + (MODE == ROW_JACOBI ? copy_blocks(a.mc) : 0));
-    launch_dependent(pairs ? bsell_kernel<B, true, TV, TX, MODE> : bsell_kernel<B, false, TV, TX, MODE>, g, 256, s, a);
+    const auto kernel = pairs ? bsell_kernel<B, true, TV, TX, MODE> : bsell_kernel<B, false, TV, TX, MODE>;
+    if (sizeof(TX) == 8 && MODE == ROW_JACOBI) kernel<<<air_counted(g), 256, 0, s>>>(a);
+    else launch_dependent(kernel, g, 256, s, a);
 }
 
 // pairs are safe when x starts on a pair boundary (the values always do)
