@@ -207,11 +207,43 @@ struct ElemArgs {
     int *err;
 };
 
-// Geometry record and facet frames of every element, one thread per element.
+// gmask[i]: bit k set when component k of grad phi_i is not zero at every volume point.  order: the entries (i, j) of
+// A by falling number of products d_k phi_i d_l phi_j, so that a warp's lanes have equally many.  One thread block.
 template <int D, int P>
-__global__ void __launch_bounds__(128) geometry_kernel(ElemArgs a, double *geo, int32_t *frame) {
+__device__ void order_entries(const double *gphi, int32_t *order, int32_t *gmask) {
+    using Dm = Dims<D, P>;
+    constexpr int NB = Dm::NB, NV = Dm::NQ * NB * D;
+    __shared__ int mask[NB];
+    __shared__ uint8_t products[NB * NB];
+    for (int i = threadIdx.x; i < NB; i += blockDim.x) mask[i] = 0;
+    __syncthreads();
+#pragma unroll 8
+    for (int t = threadIdx.x; t < NV; t += blockDim.x)
+        if (gphi[t] != 0.0) atomicOr(&mask[t / D % NB], 1 << t % D);
+    __syncthreads();
+    for (int i = threadIdx.x; i < NB; i += blockDim.x) gmask[i] = mask[i];
+    for (int t = threadIdx.x; t < NB * NB; t += blockDim.x)
+        products[t] = (uint8_t)(__popc(mask[t / NB]) * __popc(mask[t % NB]));
+    __syncthreads();
+    for (int t = threadIdx.x; t < NB * NB; t += blockDim.x) {
+        const int mine = products[t];
+        int place = 0;
+#pragma unroll 8
+        for (int u = 0; u < NB * NB; ++u) place += products[u] > mine || (products[u] == mine && u < t) ? 1 : 0;
+        order[place] = t;
+    }
+}
+
+// Geometry record and facet frames of every element, one thread per element; with `order` the last block orders the
+// entries of A instead (a launch less on small meshes, which are bound by launches).
+template <int D, int P>
+__global__ void __launch_bounds__(128) geometry_kernel(ElemArgs a, double *geo, int32_t *frame, int32_t *order) {
     using Dm = Dims<D, P>;
     constexpr int NF = Dm::NF;
+    if (order && blockIdx.x == gridDim.x - 1) {
+        order_entries<D, P>(a.gphi, order, order + Dm::NB * Dm::NB);
+        return;
+    }
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= a.E) return;
     const int32_t *ev = a.elems + e * (D + 1);
@@ -296,32 +328,6 @@ __global__ void table_kernel(const double *wq, const double *gphi, const double 
         }
     }
     table[t] = acc;
-}
-
-// gmask[i]: bit k set when component k of grad phi_i is not zero at every volume point.  order: the entries (i, j) of
-// A by falling number of products d_k phi_i d_l phi_j, so that a warp's lanes have equally many.
-template <int D, int P>
-__global__ void __launch_bounds__(512) order_kernel(const double *gphi, int32_t *order, int32_t *gmask) {
-    using Dm = Dims<D, P>;
-    constexpr int NB = Dm::NB;
-    __shared__ int mask[NB];
-    for (int i = threadIdx.x; i < NB; i += blockDim.x) {
-        int m = 0;
-        for (int q = 0; q < Dm::NQ; ++q)
-            for (int k = 0; k < D; ++k) m |= gphi[(q * NB + i) * D + k] != 0.0 ? 1 << k : 0;
-        mask[i] = m;
-        gmask[i] = m;
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < NB * NB; t += blockDim.x) {
-        const int mine = __popc(mask[t / NB]) * __popc(mask[t % NB]);
-        int place = 0;
-        for (int u = 0; u < NB * NB; ++u) {
-            const int o = __popc(mask[u / NB]) * __popc(mask[u % NB]);
-            place += o > mine || (o == mine && u < t) ? 1 : 0;
-        }
-        order[place] = t;
-    }
 }
 
 // Volume part: sA = - sum_q W phi_j a_hat.grad_hat phi_i, sF = sum_q W f phi_i.  sV (NQ (D + 1)) and sP are scratch;
@@ -1443,15 +1449,17 @@ int launch_element(ElemArgs &a, bool gradient, cudaStream_t s) {
     using Dm = Dims<D, P>;
     const size_t smem = (size_t)WPB * (gradient ? Dm::GRAD_DOUBLES : Dm::WARP_DOUBLES) * sizeof(double);
     if (smem > AIR_SMEM_OPTIN) return AIR_ERR_UNSUPPORTED;
-    double *geo = nullptr, *table = nullptr;
-    int32_t *frame = nullptr, *order = nullptr;
-    int st = dalloc(&geo, a.E * Dm::GEO);
-    if (st == AIR_OK) st = dalloc(&frame, a.E * Dm::NF);
-    if (st == AIR_OK && gradient) st = dalloc(&table, Dm::TABLE);
-    if (st == AIR_OK && !gradient) st = dalloc(&order, Dm::NB * Dm::NB + Dm::NB);
+    // geometry records, then the gradient's reference integrals; facet frames, then the assembly's order of entries
+    double *geo = nullptr;
+    int32_t *frame = nullptr;
+    int st = dalloc(&geo, a.E * Dm::GEO + (gradient ? Dm::TABLE : 0));
+    if (st == AIR_OK) st = dalloc(&frame, a.E * Dm::NF + (gradient ? 0 : Dm::NB * Dm::NB + Dm::NB));
     cudaError_t err = cudaSuccess;
     if (st == AIR_OK) {
-        geometry_kernel<D, P><<<air_counted((unsigned)((a.E + 127) / 128)), 128, 0, s>>>(a, geo, frame);
+        double *table = geo + a.E * Dm::GEO;
+        int32_t *order = gradient ? nullptr : frame + a.E * Dm::NF;
+        geometry_kernel<D, P><<<air_counted((unsigned)((a.E + 127) / 128 + (gradient ? 0 : 1))), 128, 0, s>>>(a, geo, frame,
+                                                                                                          order);
         a.geo = geo;
         a.frame = frame;
         const unsigned grid = (unsigned)((a.E + WPB - 1) / WPB);
@@ -1462,7 +1470,6 @@ int launch_element(ElemArgs &a, bool gradient, cudaStream_t s) {
             err = air_smem_optin(velocity_gradient_kernel<D, P>);
             if (err == cudaSuccess) velocity_gradient_kernel<D, P><<<air_counted(grid), WPB * 32, smem, s>>>(a);
         } else {
-            order_kernel<D, P><<<air_counted(1), 512, 0, s>>>(a.gphi, order, order + Dm::NB * Dm::NB);
             a.order = order;
             a.gmask = order + Dm::NB * Dm::NB;
             err = air_smem_optin(hdg_element_kernel<D, P>);
@@ -1472,9 +1479,7 @@ int launch_element(ElemArgs &a, bool gradient, cudaStream_t s) {
         if (err != cudaSuccess) st = AIR_ERR_CUDA;
     }
     air_dfree(geo);
-    air_dfree(table);
     air_dfree(frame);
-    air_dfree(order);
     return st;
 }
 
