@@ -2,7 +2,8 @@
 // memory, entry (r, c) of lane l's matrix at m[(r b + c) LANE_LD + l], so every
 // step of an elimination is one full FP64 instruction for 32 blocks.  (One
 // warp per block leaves most lanes of each instruction idle and repeats the
-// divisions; GB300 issues one FP64 warp instruction per SM in 16 cycles.)
+// divisions; GB300 issues one FP64 warp instruction per SM in 16 cycles.)  Or one
+// per group of lanes, row-major, with shorter chains (group_invert).
 #pragma once
 
 #include <stdint.h>

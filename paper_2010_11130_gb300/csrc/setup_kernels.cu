@@ -935,7 +935,7 @@ __global__ void lair_solve_kernel(LairJob J, int maxm, int ld, int distance, int
 // whatever number of its lanes work, which bounds the solves of a warp each).
 // Entry (r, c) of system s at M[(r LS_M + c) LS_LD + s].  Bound: the rows of
 // A, a few per system, read through the L2.  1.0 M systems of 1.7 points:
-// 1.6 ms and 0.5 ms for the larger ones (5 ms with a warp each).  LS_M = 6 holds 98% of an HDG level's systems in 13 KB a warp.
+// 1.6 ms and 0.5 ms for the larger ones (5 ms with a warp each).  LS_M = 6 holds 98% of an HDG level's systems in 12 KB a warp.
 constexpr int LS_M = 6, LS_LD = 33, LS_WARPS = 4, LS_U = 5;
 constexpr int LS_DOUBLES = (LS_M * LS_M + LS_M) * LS_LD + 32 + (LS_M * 32 + 32) / 2;
 
@@ -1614,7 +1614,7 @@ int air_lair_solve(const AirLevel &L, int32_t max_m, int distance, int64_t *d_ns
     if (distance == 1) {
         const size_t small = (size_t)LS_WARPS * LS_DOUBLES * sizeof(double);
         AIR_CUDA(air_smem_optin(lair_small_kernel));
-        // 32 systems per warp, fewer where that leaves resident warps (4 blocks of 53 KB per SM) without work
+        // 32 systems per warp, fewer where that leaves resident warps (4 blocks of 49 KB per SM) without work
         const int64_t warps = 152 * 4 * LS_WARPS;
         const int64_t share = ((L.nc + warps - 1) / warps + 3) / 4 * 4;
         const int per = (int)(share < 4 ? 4 : (share > 32 ? 32 : share));
